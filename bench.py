@@ -172,11 +172,11 @@ def kernel_bytes(name, st, src, esz):
     Ra_c = Ra + Rc
     table = {
         "router": E * H * esz + T * H * esz + T * E * 4,
-        "generic_up_anchor": ta * 2 * I * H * esz + Ra * H * esz + Ra * 2 * I * 4,
-        "generic_up_V": rt * 2 * H * esz + Rc * H * esz + rr * 2 * 4,
+        "generic_up_anchor_V": (ta * 2 * I * H * esz + Ra * H * esz + Ra * 2 * I * 4 +
+                                rt * 2 * H * esz + Rc * H * esz + rr * 2 * 4),
         "generic_up_U": rt * 2 * I * esz + rr * 2 * 4 + Rc * 2 * I * 4,
-        "generic_dn_anchor": ta * H * I * esz + Ra * I * 4 + Ra * H * 4,
-        "generic_dn_V": rt * I * esz + Rc * I * 4 + rr * 4,
+        "generic_dn_anchor_V": (ta * H * I * esz + Ra * I * 4 + Ra * H * 4 +
+                                rt * I * esz + Rc * I * 4 + rr * 4),
         "generic_dn_U": rt * H * esz + rr * 4 + Rc * H * 4,
         # streaming kernels: weights once, activations in, results out (bf16)
         "stream_up_anchor_V": (ta * 2 * I * H + rt * 2 * H) * esz + Ra_c * H * esz

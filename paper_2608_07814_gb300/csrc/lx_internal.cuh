@@ -152,7 +152,7 @@ struct OpShape {
 };
 
 // Generic tile sizes
-constexpr int G_BM = 32, G_BN = 64, G_BK = 32;
+constexpr int G_BM = 32, G_BN = 64;
 
 struct GemmArgs {
   const int* items;        // node ids [n_items]
