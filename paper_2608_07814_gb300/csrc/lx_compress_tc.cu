@@ -217,12 +217,22 @@ __global__ void k_transpose_bf16(const __nv_bfloat16* __restrict__ W, int rows, 
 // C [M][N] = sum over the K ranges s (ascending) of part[s][M][Npad]
 __global__ void k_sum_parts(const float* __restrict__ part, int splits, int M, int N, int Npad,
                             float* __restrict__ C) {
-  const long total = (long)M * N;
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (long)gridDim.x * blockDim.x) {
-    const long m = i / N, n = i % N;
+  // (rows and columns stay below 65537 and 257: 32-bit indexes; eight ranges'
+  // loads in flight before they are added in order)
+  const uint32_t total = (uint32_t)M * (uint32_t)N;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+    const uint32_t m = i / (uint32_t)N, n = i - m * (uint32_t)N;
+    const float* p = part + (size_t)m * Npad + n;
+    const size_t step = (size_t)M * Npad;
     float acc = 0.f;
-    for (int s = 0; s < splits; ++s) acc += part[((size_t)s * M + m) * Npad + n];
+    for (int s = 0; s < splits; s += 8) {
+      float v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = s + u < splits ? p[(size_t)(s + u) * step] : 0.f;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (s + u < splits) acc += v[u];
+    }
     C[i] = acc;
   }
 }
@@ -239,28 +249,36 @@ size_t res_tc_workspace(long rows, long cols, long l) {
          al((size_t)RES_TC_MAX_SPLITS * Mmax * Npad * 4);
 }
 
+size_t res_tc_part_offset(long rows, long cols, long l) {
+  const long Npad = (l + 15) / 16 * 16, Kp = (std::max(rows, cols) + 63) / 64 * 64;
+  auto al = [](size_t v) { return (v + 255) / 256 * 256; };
+  return al(2 * (size_t)rows * cols * 2) + al((size_t)Npad * 6 * Kp * 2);
+}
+
 bool res_tc_fits(long rows, long cols, long l) {
   return rows % 8 == 0 && cols % 8 == 0 && l >= 1 && (l + 15) / 16 * 16 <= 256;
 }
 
 lx_status res_gemm_tc(bool transposed, const __nv_bfloat16* Wm, const __nv_bfloat16* Wd,
                       long rows, long cols, const float* X, long N, float* C, char* ws,
-                      int num_sms, int dev, cudaStream_t s) {
+                      bool* have_wt, int num_sms, int dev, cudaStream_t s) {
   auto al = [](size_t v) { return (v + 255) / 256 * 256; };
   __nv_bfloat16* Wt = reinterpret_cast<__nv_bfloat16*>(ws);  // [2][cols][rows]
   __nv_bfloat16* Bc = reinterpret_cast<__nv_bfloat16*>(ws + al(2 * (size_t)rows * cols * 2));
   const long M = transposed ? cols : rows, K = transposed ? rows : cols;
   const long Npad = (N + 15) / 16 * 16, Kp = (K + 63) / 64 * 64;
-  float* part = reinterpret_cast<float*>(
-      ws + al(2 * (size_t)rows * cols * 2) +
-      al((size_t)Npad * 6 * ((std::max(rows, cols) + 63) / 64 * 64) * 2));
+  float* part = reinterpret_cast<float*>(ws + res_tc_part_offset(rows, cols, N));
   const __nv_bfloat16* Am = Wm;
   const __nv_bfloat16* Ad = Wd;
   if (transposed) {
-    const dim3 grid((unsigned)((cols + 31) / 32), (unsigned)((rows + 31) / 32));
-    k_transpose_bf16<<<grid, dim3(32, 8), 0, s>>>(Wm, (int)rows, (int)cols, Wt);
-    k_transpose_bf16<<<grid, dim3(32, 8), 0, s>>>(Wd, (int)rows, (int)cols,
-                                                   Wt + (size_t)rows * cols);
+    // W^T is formed by the call's first R^T product and kept for the others
+    if (!*have_wt) {
+      const dim3 grid((unsigned)((cols + 31) / 32), (unsigned)((rows + 31) / 32));
+      k_transpose_bf16<<<grid, dim3(32, 8), 0, s>>>(Wm, (int)rows, (int)cols, Wt);
+      k_transpose_bf16<<<grid, dim3(32, 8), 0, s>>>(Wd, (int)rows, (int)cols,
+                                                     Wt + (size_t)rows * cols);
+      *have_wt = true;
+    }
     Am = Wt;
     Ad = Wt + (size_t)rows * cols;
   }

@@ -502,10 +502,13 @@ bool encode_bf16_2d(CUtensorMap* m, const void* base, long inner, long outer, in
 // R^T X (M = cols, K = rows), R = Wm - Wd [rows][cols], X fp32 [K][N]
 constexpr int RES_TC_MAX_SPLITS = 32;
 size_t res_tc_workspace(long rows, long cols, long l);
+// where the K ranges' partials lie in that workspace (RES_TC_MAX_SPLITS x
+// max(rows, cols) x 16-padded l floats)
+size_t res_tc_part_offset(long rows, long cols, long l);
 bool res_tc_fits(long rows, long cols, long l);
 lx_status res_gemm_tc(bool transposed, const __nv_bfloat16* Wm, const __nv_bfloat16* Wd,
                       long rows, long cols, const float* X, long N, float* C, char* ws,
-                      int num_sms, int dev, cudaStream_t s);
+                      bool* have_wt, int num_sms, int dev, cudaStream_t s);
 // split-K tensor-core product part[s][M][Npad] = A . B^T over K range s (see
 // lx_compress_tc.cu); the number of ranges used is returned in splits_out
 lx_status tc_splitk_gemm_chunks(const CUtensorMap& a, const CUtensorMap& b, int M, int Npad,
