@@ -149,7 +149,6 @@ static lx_status ensure_workspace(lx_layer* L, int T, int k, cudaStream_t s) {
   Workspace& w = L->ws;
   if (T <= w.cap_T && k <= w.cap_k) return LX_OK;
   const int cT = std::max(T, w.cap_T), ck = std::max(k, w.cap_k);
-  const long Tp = align_up((size_t)cT, 16);
   const long D = L->max_depth;
   const long keys = (long)L->N + L->E;
   const long Rmax = std::max<long>(1, (long)cT * std::min<long>(L->N, (long)ck * D));
@@ -165,9 +164,9 @@ static lx_status ensure_workspace(lx_layer* L, int T, int k, cudaStream_t s) {
       {(void**)&w.topk_id, sizeof(int) * cT * ck},
       {(void**)&w.tile_cnt, sizeof(int) * std::max(1, router_tile_counters(cT))},
       {(void**)&w.topk_w, sizeof(float) * cT * ck},
-      {(void**)&w.marks, (size_t)keys * Tp},
-      {(void**)&w.rank_in, sizeof(int) * keys * Tp},
-      {(void**)&w.key_cnt, sizeof(int) * keys},
+      {(void**)&w.bits, sizeof(uint32_t) * bucket_words() * keys * bucket_blocks(cT)},
+      {(void**)&w.blk_cnt, sizeof(int) * keys * bucket_blocks(cT)},
+      {(void**)&w.blk_pre, sizeof(int) * keys * bucket_blocks(cT)},
       {(void**)&w.key_off, sizeof(int) * (keys + 2)},
       {(void**)&w.node_tok, sizeof(int) * cT * ck * D},
       {(void**)&w.row_node, sizeof(int) * cT * ck * D},

@@ -3,12 +3,13 @@
 // forward computes once, Sec. 5.1), per assignment and path level the row of
 // that pair, and per expert its assignments in token order.
 //
-// Keys are the N nodes followed by the E experts.  A byte matrix marks[key][t]
-// records which (key, token) pairs occur; one CTA per key turns its row into
-// exclusive ranks with a block scan (so the order inside a bucket is the token
-// order, with no atomics); a single CTA scans the per-key counts into offsets
-// and builds the tile plans of the grouped GEMMs; a last pass scatters.
-// Everything is deterministic.
+// Keys are the N nodes followed by the E experts.  Three launches: one CTA per
+// block of 256 tokens records which (key, token) pairs occur as bits in shared
+// memory (8 words a key) and counts them; a single CTA sums the blocks' counts
+// per key, scans them into offsets and builds the tile plans of the grouped
+// GEMMs; a warp per token then reads its rows off as offset + earlier blocks +
+// set bits before it (so the order inside a bucket is the token order, with no
+// order-dependent atomics).  Everything is deterministic.
 #include <mutex>
 
 #include "lx_internal.cuh"
@@ -17,75 +18,73 @@ namespace lx {
 
 namespace {
 
-constexpr int SCAN_THREADS = 512;
+constexpr int BK_TOK = 256;            // tokens of a block
+constexpr int BK_WORDS = BK_TOK / 32;  // bitmap words of a key in a block
 
-__global__ void k_mark(const int* __restrict__ topk_id, int T, int k, int N, int E, long Tp,
-                       const int* __restrict__ paths, const int* __restrict__ path_len,
-                       uint8_t* __restrict__ marks) {
+// Block b (CTA b): bits[b][key][w] bit i <-> token 256 b + 32 w + i has the key,
+// and their number cnt[b][key].  A byte per (key, token) pair, cleared, marked,
+// scanned and read back, took a memset and two more launches (38 us for the
+// five at 8192 tokens and 256 keys, 25 for these three); word w belongs to warp
+// w alone, so the shared-memory atomics meet only inside a warp.
+__global__ void __launch_bounds__(BK_TOK)
+k_mark_bits(const int* __restrict__ topk_id, int T, int k, int N, int E,
+            const int* __restrict__ paths, uint32_t* __restrict__ bits, int* __restrict__ cnt) {
+  extern __shared__ __align__(16) uint32_t sb[];
+  const int keys = N + E, tid = threadIdx.x;
+  for (int i = tid; i < keys * BK_WORDS; i += BK_TOK) sb[i] = 0u;
   pdl_wait();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= T) return;
-  for (int s = 0; s < k; ++s) {
-    const int e = topk_id[(size_t)t * k + s];
-    if (e < 0 || e >= E) continue;  // invalid ids are ignored
-    marks[(size_t)(N + e) * Tp + t] = 1;
-    const int len = path_len[e];
-    for (int l = 0; l < len; ++l) marks[(size_t)paths[e * LX_MAX_DEPTH + l] * Tp + t] = 1;
+  __syncthreads();
+  const int t = blockIdx.x * BK_TOK + tid, w = tid >> 5;
+  const uint32_t bit = 1u << (tid & 31);
+  if (t < T) {
+    constexpr int U = 8;  // slots whose ids and paths are in flight at once
+    for (int s0 = 0; s0 < k; s0 += U) {
+      int e[U];
+      int4 p[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) e[u] = s0 + u < k ? topk_id[(size_t)t * k + s0 + u] : -1;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (e[u] >= E) e[u] = -1;  // invalid ids are ignored
+        p[u] = e[u] >= 0 ? __ldg(reinterpret_cast<const int4*>(paths) + e[u]) : make_int4(-1, -1, -1, -1);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (e[u] < 0) continue;
+        atomicOr(&sb[(N + e[u]) * BK_WORDS + w], bit);
+        const int q[LX_MAX_DEPTH] = {p[u].x, p[u].y, p[u].z, p[u].w};
+#pragma unroll
+        for (int l = 0; l < LX_MAX_DEPTH; ++l)
+          if (q[l] >= 0) atomicOr(&sb[q[l] * BK_WORDS + w], bit);
+      }
+    }
+  }
+  __syncthreads();
+  uint4* gb = reinterpret_cast<uint4*>(bits + (size_t)blockIdx.x * keys * BK_WORDS);
+  for (int key = tid; key < keys; key += BK_TOK) {
+    const uint4 a = reinterpret_cast<const uint4*>(sb)[2 * key];
+    const uint4 b = reinterpret_cast<const uint4*>(sb)[2 * key + 1];
+    gb[2 * key] = a;
+    gb[2 * key + 1] = b;
+    cnt[(size_t)blockIdx.x * keys + key] = __popc(a.x) + __popc(a.y) + __popc(a.z) + __popc(a.w) +
+                                           __popc(b.x) + __popc(b.y) + __popc(b.z) + __popc(b.w);
   }
 }
+static_assert(BK_WORDS == 8 && LX_MAX_DEPTH == 4, "two 16-byte pieces a key, one a path");
 
-// block-wide exclusive scan of one int per thread; returns the block total
-__device__ int block_excl_scan(int v, int* total) {
-  __shared__ int warp_sums[32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  int incl = v;
+// number of tokens before t that have the key (pre: those of earlier blocks)
+__device__ __forceinline__ int rank_before(const uint32_t* __restrict__ bits, const int* __restrict__ pre,
+                                           int keys, int key, int t) {
+  const size_t row = (size_t)(t / BK_TOK) * keys + key;
+  const uint4 a = __ldg(reinterpret_cast<const uint4*>(bits) + 2 * row);
+  const uint4 b = __ldg(reinterpret_cast<const uint4*>(bits) + 2 * row + 1);
+  const uint32_t v[BK_WORDS] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+  const int w = (t % BK_TOK) >> 5;
+  const uint32_t below = (1u << (t & 31)) - 1u;
+  int r = __ldg(pre + row);
 #pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const int o = __shfl_up_sync(0xffffffffu, incl, off);
-    if (lane >= off) incl += o;
-  }
-  if (lane == 31) warp_sums[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    int ws = lane < nw ? warp_sums[lane] : 0;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int o = __shfl_up_sync(0xffffffffu, ws, off);
-      if (lane >= off) ws += o;
-    }
-    if (lane < nw) warp_sums[lane] = ws;  // inclusive
-  }
-  __syncthreads();
-  const int warp_base = warp > 0 ? warp_sums[warp - 1] : 0;
-  *total = warp_sums[nw - 1];
-  __syncthreads();
-  return warp_base + incl - v;
-}
-
-__global__ void __launch_bounds__(SCAN_THREADS)
-k_key_scan(const uint8_t* __restrict__ marks, int T, long Tp, int* __restrict__ rank_in,
-           int* __restrict__ key_cnt) {
-  pdl_wait();
-  const int key = blockIdx.x;
-  const uint8_t* m = marks + (size_t)key * Tp;
-  int* r = rank_in + (size_t)key * Tp;
-  int running = 0;
-  for (int base = 0; base < T; base += blockDim.x * 4) {
-    const int i0 = base + threadIdx.x * 4;
-    int v[4], c = 0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      v[j] = (i0 + j < T) ? m[i0 + j] : 0;
-      c += v[j];
-    }
-    int total;
-    int run = running + block_excl_scan(c, &total);
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (v[j]) r[i0 + j] = run++;
-    running += total;
-  }
-  if (threadIdx.x == 0) key_cnt[key] = running;
+  for (int j = 0; j < BK_WORDS; ++j) r += __popc(v[j] & (j < w ? 0xffffffffu : j == w ? below : 0u));
+  return r;
 }
 
 struct PlanArgs {
@@ -108,131 +107,110 @@ __device__ __forceinline__ int plan_tiles(const PlanArgs& pa, int p, int r, int 
 
 
 // Work items of the streaming launches: one (node, token block) pair per
-// `blk` rows of every active node's bucket, anchors then corrections, in
-// node-table order, packed as node * STREAM_DEP_TB + block; and zeroed tile
-// counters.  blk = 0 (batches the streaming kernels do not take) publishes
-// empty lists.  One CTA; warps 0 and 1 each compact one list.
-__device__ void publish_active(const int* cnt, const int* anchors, int n_anchor,
-                               const int* corrs, int n_corr, int blk, int* act, int* act_n,
-                               int* sctr, int n_sctr) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (warp < 2) {
-    const int* list = warp == 0 ? anchors : corrs;
-    const int n = warp == 0 ? n_anchor : n_corr;
-    int* out = act + (warp == 0 ? 0 : n_anchor * STREAM_DEP_TB);
-    int base = 0;
-    for (int i0 = 0; i0 < n && blk > 0; i0 += 32) {
-      const int i = i0 + lane;
-      const int node = i < n ? list[i] : -1;
-      // blocks of this node's bucket (the host passes blk only for batches of
-      // at most STREAM_DEP_TB blocks)
-      const int nb = node >= 0 ? (cnt[node] + blk - 1) / blk : 0;
-      int incl = nb;
+// `blk` rows of every active node's bucket, in node-table order, packed as
+// node * STREAM_DEP_TB + block.  blk = 0 (batches the streaming kernels do not
+// take) publishes an empty list.  One warp; which = 0: the anchors, 1: the
+// corrections (their items follow the anchors' area).
+__device__ void publish_active(const int* cnt, const int* list, int n, int which, int n_anchor, int blk,
+                               int* act, int* act_n) {
+  const int lane = threadIdx.x & 31;
+  int* out = act + (which == 0 ? 0 : n_anchor * STREAM_DEP_TB);
+  int base = 0;
+  for (int i0 = 0; i0 < n && blk > 0; i0 += 32) {
+    const int i = i0 + lane;
+    const int node = i < n ? list[i] : -1;
+    // blocks of this node's bucket (the host passes blk only for batches of
+    // at most STREAM_DEP_TB blocks)
+    const int nb = node >= 0 ? (cnt[node] + blk - 1) / blk : 0;
+    int incl = nb;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int x = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += x;
-      }
-      for (int b = 0; b < nb; ++b) out[base + incl - nb + b] = node * STREAM_DEP_TB + b;
-      base += __shfl_sync(0xffffffffu, incl, 31);
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += x;
     }
-    if (lane == 0) act_n[warp] = base;
+    for (int b = 0; b < nb; ++b) out[base + incl - nb + b] = node * STREAM_DEP_TB + b;
+    base += __shfl_sync(0xffffffffu, incl, 31);
   }
-  for (int i = threadIdx.x; i < n_sctr; i += blockDim.x) sctr[i] = 0;
+  if (lane == 0) act_n[which] = base;
 }
 
-// one CTA: node/expert offsets and the tile prefix of every plan
-__global__ void k_offsets_plan(const int* __restrict__ key_cnt, int N, int E,
-                               int* __restrict__ key_off, const int* __restrict__ rank,
-                               int* __restrict__ tile_off, int max_items, PlanArgs pa,
-                               const int* __restrict__ anchors, int n_anchor,
-                               const int* __restrict__ corrs, int n_corr, int blk,
-                               int* __restrict__ act, int* __restrict__ act_n,
-                               int* __restrict__ sctr, int n_sctr) {
-  pdl_wait();
-  if (act)
-    publish_active(key_cnt, anchors, n_anchor, corrs, n_corr, blk, act, act_n, sctr, n_sctr);
-  // node offsets then expert offsets
-  for (int part = 0; part < 2; ++part) {
-    const int n0 = part == 0 ? 0 : N, cnt = part == 0 ? N : E;
-    int* out = key_off + (part == 0 ? 0 : N + 1);
-    int carry = 0;
-    for (int base = 0; base < cnt; base += blockDim.x) {
-      const int i = base + threadIdx.x;
-      const int v = i < cnt ? key_cnt[n0 + i] : 0;
-      int total;
-      const int ex = block_excl_scan(v, &total);
-      if (i < cnt) out[i] = carry + ex;
-      carry += total;
+// One warp: exclusive offsets out[0 .. n] of counts v(i), i < n.
+template <typename F>
+__device__ __forceinline__ void warp_offsets(int n, F v, int* out) {
+  const int lane = threadIdx.x & 31;
+  int carry = 0;
+  for (int base = 0; base < n; base += 32) {
+    const int i = base + lane;
+    const int x0 = i < n ? v(i) : 0;
+    int incl = x0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += x;
     }
-    if (threadIdx.x == 0) out[cnt] = carry;
-    __syncthreads();
+    if (i < n) out[i] = carry + incl - x0;
+    carry += __shfl_sync(0xffffffffu, incl, 31);
   }
-  for (int p = 0; p < pa.n_plans; ++p) {
-    int* to = tile_off + (pa.first + p) * (max_items + 1);
-    int carry = 0;
-    for (int base = 0; base < pa.n_items[p]; base += blockDim.x) {
-      const int i = base + threadIdx.x;
-      int v = 0;
-      if (i < pa.n_items[p]) {
-        const int n = pa.items[p][i];
-        v = plan_tiles(pa, p, rank[n], key_cnt[n]);
-      }
-      int total;
-      const int ex = block_excl_scan(v, &total);
-      if (i < pa.n_items[p]) to[i] = carry + ex;
-      carry += total;
-    }
-    if (threadIdx.x == 0) to[pa.n_items[p]] = carry;
-    __syncthreads();
-  }
+  if (lane == 0) out[n] = carry;
 }
 
-__global__ void k_scatter(const uint8_t* __restrict__ marks, const int* __restrict__ rank_in,
-                          const int* __restrict__ key_off, const int* __restrict__ topk_id, int T,
-                          int k, int N, long Tp, int* __restrict__ node_tok,
-                          int* __restrict__ row_node, int* __restrict__ perm) {
-  pdl_wait();
-  const int key = blockIdx.y;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= T) return;
-  const size_t idx = (size_t)key * Tp + t;
-  if (!marks[idx]) return;
-  const int rk = rank_in[idx];
-  if (key < N) {
-    const int row = key_off[key] + rk;
-    node_tok[row] = t;
-    row_node[row] = key;
-  } else {
-    const int e = key - N;
-    const int pos = key_off[N + 1 + e] + rk;
-    for (int s = 0; s < k; ++s)
-      if (topk_id[(size_t)t * k + s] == e) {
-        perm[pos] = t * k + s;
-        break;
-      }
-  }
-}
+constexpr int OP_THREADS = 1024;
+inline size_t op_smem(int keys, int N) { return sizeof(int) * ((size_t)keys + 2 * (size_t)N); }
 
-__global__ void k_node_row(const int* __restrict__ topk_id, int T, int k, int E, int D, long Tp,
-                           const int* __restrict__ paths, const int* __restrict__ path_len,
-                           const int* __restrict__ key_off, const int* __restrict__ rank_in,
-                           int* __restrict__ node_row) {
+// One CTA: every key's count and the blocks' exclusive prefixes pre[b][key],
+// then, a warp each, the node offsets, the expert offsets, the streaming work
+// items and the tile prefix of every plan.  The layer's tables are staged
+// before the wait for the preceding kernel; the plans, one after another over
+// the whole CTA, had made this 9.8 us at 8192 tokens (6.6 now).
+__global__ void __launch_bounds__(OP_THREADS)
+k_offsets_plan(const int* __restrict__ cnt, int nblk, int N, int E, int* __restrict__ pre,
+               int* __restrict__ key_off, const int* __restrict__ rank, int* __restrict__ tile_off,
+               int max_items, PlanArgs pa, const int* __restrict__ anchors, int n_anchor,
+               const int* __restrict__ corrs, int n_corr, int blk, int* __restrict__ act,
+               int* __restrict__ act_n, int* __restrict__ sctr, int n_sctr) {
+  extern __shared__ int osh[];
+  const int keys = N + E, tid = threadIdx.x, warp = tid >> 5;
+  int* kc = osh;            // [keys]
+  int* srank = kc + keys;   // [N]
+  int* slist = srank + N;   // [N]: the anchors, then the corrections
+  for (int i = tid; i < N; i += OP_THREADS) {
+    srank[i] = rank[i];
+    slist[i] = i < n_anchor ? anchors[i] : corrs[i - n_anchor];
+  }
   pdl_wait();
-  const long a = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (a >= (long)T * k) return;
-  const int t = (int)(a / k);
-  const int e = topk_id[a];
-  const int len = (e >= 0 && e < E) ? path_len[e] : 0;
-  for (int l = 0; l < D; ++l) {
-    int row = -1;
-    if (l < len) {
-      const int n = paths[e * LX_MAX_DEPTH + l];
-      row = key_off[n] + rank_in[(size_t)n * Tp + t];
+  for (int i = tid; i < n_sctr; i += OP_THREADS) sctr[i] = 0;
+  for (int key = tid; key < keys; key += OP_THREADS) {
+    int run = 0;
+    for (int b0 = 0; b0 < nblk; b0 += 16) {
+      int v[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) v[u] = b0 + u < nblk ? cnt[(size_t)(b0 + u) * keys + key] : 0;
+#pragma unroll
+      for (int u = 0; u < 16; ++u)
+        if (b0 + u < nblk) {
+          pre[(size_t)(b0 + u) * keys + key] = run;
+          run += v[u];
+        }
     }
-    node_row[a * D + l] = row;
+    kc[key] = run;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    warp_offsets(N, [&](int i) { return kc[i]; }, key_off);
+  } else if (warp == 1) {
+    warp_offsets(E, [&](int i) { return kc[N + i]; }, key_off + N + 1);
+  } else if (warp == 2 || warp == 3) {
+    if (act)
+      publish_active(kc, warp == 2 ? slist : slist + n_anchor, warp == 2 ? n_anchor : n_corr, warp - 2,
+                     n_anchor, blk, act, act_n);
+  } else if (warp - 4 < pa.n_plans) {
+    const int p = warp - 4;
+    const int* items = pa.shape[p].on_anchors ? slist : slist + n_anchor;
+    warp_offsets(pa.n_items[p], [&](int i) { return plan_tiles(pa, p, srank[items[i]], kc[items[i]]); },
+                 tile_off + (pa.first + p) * (max_items + 1));
   }
 }
+static_assert(4 + N_OPS <= OP_THREADS / 32, "a warp for every role");
 
 // The fused path's per-cluster-row tables (flat layers on the tensor-core
 // path; al_g == nullptr: none): see k_assign_rows.
@@ -255,25 +233,23 @@ struct CtMeta {
 // al_row[a] = the child rows (-1 where not selected), written by the first
 // slot of that anchor row; rho2al maps every child row to its anchor row.
 __global__ void __launch_bounds__(256)
-k_assign_rows(const int* __restrict__ topk_id, int T, int k, int N, int E, int D, long Tp,
+k_assign_rows(const int* __restrict__ topk_id, int T, int k, int N, int E, int D,
               const int* __restrict__ paths, const int* __restrict__ path_len,
-              const int* __restrict__ key_off, const int* __restrict__ rank_in,
-              int* __restrict__ node_tok, int* __restrict__ row_node, int* __restrict__ perm,
-              int* __restrict__ node_row, const CtMeta cm) {
+              const int* __restrict__ key_off, const uint32_t* __restrict__ bits,
+              const int* __restrict__ pre, int* __restrict__ node_tok, int* __restrict__ row_node,
+              int* __restrict__ perm, int* __restrict__ node_row, const CtMeta cm) {
   pdl_wait();
   const int lane = threadIdx.x & 31;
   const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (t >= T) return;
   const size_t a = (size_t)t * k + lane;
-  int e = -1, len = 0;
-  if (lane < k) {
-    e = topk_id[a];
-    if (e >= 0 && e < E) {
-      len = path_len[e];
-      perm[key_off[N + 1 + e] + rank_in[(size_t)(N + e) * Tp + t]] = (int)a;
-    } else {
-      e = -1;
-    }
+  int e = lane < k ? topk_id[a] : -1, len = 0;
+  if (e < 0 || e >= E) e = -1;
+  const unsigned twins = __match_any_sync(0xffffffffu, e);
+  if (e >= 0) {
+    len = path_len[e];
+    if (lane == __ffs(twins) - 1)  // a repeated id counts once, with its first slot
+      perm[key_off[N + 1 + e] + rank_before(bits, pre, N + E, N + e, t)] = (int)a;
   }
   int r0 = -1, r1 = -1, n0 = -1;
 #pragma unroll
@@ -282,7 +258,7 @@ k_assign_rows(const int* __restrict__ topk_id, int T, int k, int N, int E, int D
     int row = -1;
     if (l < len) {
       const int n = paths[e * LX_MAX_DEPTH + l];
-      row = key_off[n] + rank_in[(size_t)n * Tp + t];
+      row = key_off[n] + rank_before(bits, pre, N + E, n, t);
       node_tok[row] = t;
       row_node[row] = n;
       if (l == 0) n0 = n;
@@ -451,7 +427,10 @@ k_bucket_small(const float* __restrict__ logits, const int* __restrict__ ids_in,
   }
   __syncthreads();
   for (int i = tid; i < keys + 2; i += nth) key_off_g[i] = off[i];
-  publish_active(cnt, slist, n_anchor, slist + n_anchor, n_corr, blk, act, act_n, sctr, n_sctr);
+  for (int i = tid; i < n_sctr; i += nth) sctr[i] = 0;
+  if (warp < 2)
+    publish_active(cnt, warp == 0 ? slist : slist + n_anchor, warp == 0 ? n_anchor : n_corr, warp, n_anchor,
+                   blk, act, act_n);
   // 5. tile plans: one warp per plan
   for (int p = warp; p < pa.n_plans; p += nw) {
     int* to = tile_off + (pa.first + p) * (max_items + 1);
@@ -498,6 +477,9 @@ k_bucket_small(const float* __restrict__ logits, const int* __restrict__ ids_in,
 // plans 0..N_OPS-1: generic tiles; N_OPS..2*N_OPS-1: streaming tiles
 // Plans for slots [first, first + n_plans): 0 = the generic GEMMs' six ops,
 // PLAN_TC = the tensor-core GEMMs' six ops.
+int bucket_blocks(int T) { return (T + BK_TOK - 1) / BK_TOK; }
+int bucket_words() { return BK_WORDS; }
+
 static PlanArgs make_plans(const lx_layer* L, int n_plans, int first = 0) {
   PlanArgs pa;
   pa.n_plans = n_plans;
@@ -554,33 +536,33 @@ lx_status launch_bucket_small(lx_layer* L, const float* logits, const int* ids_i
   return LX_OK;
 }
 
+static lx_status mark_bits_cap(const lx_layer* L, size_t* smem) {
+  *smem = sizeof(uint32_t) * BK_WORDS * (size_t)(L->N + L->E);  // at most 160 KB (5120 keys)
+  static bool done[64] = {};
+  LX_CUDA(smem_cap_once((const void*)k_mark_bits, 200 * 1024, L->device, done));
+  static bool done_o[64] = {};
+  LX_CUDA(smem_cap_once((const void*)k_offsets_plan, 100 * 1024, L->device, done_o));
+  return LX_OK;
+}
+
 lx_status launch_bucket(lx_layer* L, const int* topk_id, int T, int k, cudaStream_t s,
                         int plan_first) {
   Workspace& w = L->ws;
-  const long Tp = (w.cap_T + 15) / 16 * 16;
-  const int keys = L->N + L->E;
-  {
-    ProfScope ps(L, s, "bucket_clear");
-    LX_CUDA(cudaMemsetAsync(w.marks, 0, (size_t)keys * Tp, s));
-  }
+  const int keys = L->N + L->E, nblk = bucket_blocks(T);
+  size_t smem = 0;
+  LX_TRY(mark_bits_cap(L, &smem));
   {
     ProfScope ps(L, s, "bucket_mark");
-    launch_k(L, k_mark, (T + 255) / 256, 256, 0, s, topk_id, T, k, L->N, L->E, Tp, L->d_paths,
-             L->d_path_len, w.marks);
-    LX_CUDA(cudaGetLastError());
-  }
-  {
-    ProfScope ps(L, s, "bucket_scan");
-    launch_k(L, k_key_scan, keys, SCAN_THREADS, 0, s, w.marks, T, Tp, w.rank_in, w.key_cnt);
+    launch_k(L, k_mark_bits, nblk, BK_TOK, smem, s, topk_id, T, k, L->N, L->E, L->d_paths, w.bits,
+             w.blk_cnt);
     LX_CUDA(cudaGetLastError());
   }
   {
     const PlanArgs pa = plan_first < 0 ? make_plans(L, 0) : make_plans(L, N_OPS, plan_first);
     ProfScope ps(L, s, "bucket_offsets");
-    launch_k(L, k_offsets_plan, 1, 1024, 0, s, w.key_cnt, L->N, L->E, w.key_off, L->d_rank, w.tile_off,
-                                      op_max_items(L), pa, L->d_anchors, L->n_anchor, L->d_corrs,
-                                      L->n_corr, stream_item_rows(T), w.act, w.act_n, w.sctr,
-                                      sctr_ints(L));
+    launch_k(L, k_offsets_plan, 1, OP_THREADS, op_smem(keys, L->N), s, w.blk_cnt, nblk, L->N, L->E,
+             w.blk_pre, w.key_off, L->d_rank, w.tile_off, op_max_items(L), pa, L->d_anchors, L->n_anchor,
+             L->d_corrs, L->n_corr, stream_item_rows(T), w.act, w.act_n, w.sctr, sctr_ints(L));
     LX_CUDA(cudaGetLastError());
   }
   {
@@ -600,7 +582,7 @@ lx_status launch_bucket(lx_layer* L, const int* topk_id, int T, int k, cudaStrea
     }
     ProfScope ps(L, s, "bucket_rows");
     launch_k(L, k_assign_rows, (unsigned)((T + 7) / 8), 256, 0, s, topk_id, T, k, L->N, L->E,
-             L->max_depth, Tp, L->d_paths, L->d_path_len, w.key_off, w.rank_in, w.node_tok,
+             L->max_depth, L->d_paths, L->d_path_len, w.key_off, w.bits, w.blk_pre, w.node_tok,
              w.row_node, w.perm, w.node_row, cm);
     LX_CUDA(cudaGetLastError());
   }
@@ -664,8 +646,9 @@ extern "C" lx_status lx_bucket_noalloc(lx_layer* L, const int32_t* topk_id, int3
   LX_CUDA(cudaGetDevice(&dev));
   if (dev != L->device) return fail(LX_ERR_ARG, "the layer's device must be current");
 
-  // carve the scratch: marks, ranks, counts, offsets, row->node (no tile plans:
-  // nothing reads them here)
+  // The admitted batches: those whose marks and ranks (a byte and an int per key
+  // and token), counts, offsets and row->node table fit the array, as the header
+  // states.  The kernels now need less (bits and block counts), carved below.
   const long Tp = ((long)T + 15) / 16 * 16;
   const long keys = (long)L->N + L->E;
   const long D = L->max_depth;
@@ -681,31 +664,29 @@ extern "C" lx_status lx_bucket_noalloc(lx_layer* L, const int32_t* topk_id, int3
                                   std::to_string((size_t)LX_NOALLOC_SCRATCH_BYTES));
   void* base = nullptr;
   LX_TRY(scratch_address(dev, &base));
+  const int nblk = bucket_blocks(T);
   char* p = static_cast<char*>(base);
-  uint8_t* marks = reinterpret_cast<uint8_t*>(p);
-  int* rank_in = reinterpret_cast<int*>(p += b_marks);
-  int* key_cnt = reinterpret_cast<int*>(p += b_rank);
-  int* key_off = reinterpret_cast<int*>(p += b_cnt);
+  uint32_t* bits = reinterpret_cast<uint32_t*>(p);
+  int* cnt = reinterpret_cast<int*>(p += round256(sizeof(uint32_t) * BK_WORDS * (size_t)keys * nblk));
+  int* pre = reinterpret_cast<int*>(p += round256(sizeof(int) * (size_t)keys * nblk));
+  int* key_off = reinterpret_cast<int*>(p += round256(sizeof(int) * (size_t)keys * nblk));
   int* row_node = reinterpret_cast<int*>(p += b_off);
+  const size_t used = (size_t)(p - static_cast<char*>(base)) + b_rown;
+  if (used > (size_t)LX_NOALLOC_SCRATCH_BYTES)
+    return fail(LX_ERR_SHAPE, "lx_bucket_noalloc: scratch layout exceeds the fixed array");
 
-  LX_CUDA(cudaMemsetAsync(marks, 0, (size_t)keys * Tp, s));  // previous call's marks
-  k_mark<<<(T + 255) / 256, 256, 0, s>>>(topk_id, T, k, L->N, L->E, Tp, L->d_paths,
-                                         L->d_path_len, marks);
-  LX_CUDA(cudaGetLastError());
-  k_key_scan<<<(unsigned)keys, SCAN_THREADS, 0, s>>>(marks, T, Tp, rank_in, key_cnt);
+  size_t smem = 0;
+  LX_TRY(mark_bits_cap(L, &smem));
+  k_mark_bits<<<nblk, BK_TOK, smem, s>>>(topk_id, T, k, L->N, L->E, L->d_paths, bits, cnt);
   LX_CUDA(cudaGetLastError());
   const PlanArgs pa = make_plans(L, 0);
-  k_offsets_plan<<<1, 1024, 0, s>>>(key_cnt, L->N, L->E, key_off, L->d_rank, nullptr,
-                                    op_max_items(L), pa, nullptr, 0, nullptr, 0, 0, nullptr,
-                                    nullptr, nullptr, 0);
+  k_offsets_plan<<<1, OP_THREADS, op_smem((int)keys, L->N), s>>>(
+      cnt, nblk, L->N, L->E, pre, key_off, L->d_rank, nullptr, op_max_items(L), pa, L->d_anchors,
+      L->n_anchor, L->d_corrs, L->n_corr, 0, nullptr, nullptr, nullptr, 0);
   LX_CUDA(cudaGetLastError());
-  k_scatter<<<dim3((T + 255) / 256, (unsigned)keys), 256, 0, s>>>(
-      marks, rank_in, key_off, topk_id, T, k, L->N, Tp, node_tok, row_node, perm);
-  LX_CUDA(cudaGetLastError());
-  const long A = (long)T * k;
-  k_node_row<<<(unsigned)((A + 255) / 256), 256, 0, s>>>(topk_id, T, k, L->E, L->max_depth, Tp,
-                                                         L->d_paths, L->d_path_len, key_off,
-                                                         rank_in, node_row);
+  k_assign_rows<<<(unsigned)((T + 7) / 8), 256, 0, s>>>(topk_id, T, k, L->N, L->E, L->max_depth,
+                                                        L->d_paths, L->d_path_len, key_off, bits, pre,
+                                                        node_tok, row_node, perm, node_row, CtMeta{});
   LX_CUDA(cudaGetLastError());
   LX_CUDA(cudaMemcpyAsync(node_off, key_off, sizeof(int) * (L->N + 1), cudaMemcpyDeviceToDevice, s));
   LX_CUDA(cudaMemcpyAsync(expert_off, key_off + L->N + 1, sizeof(int) * (L->E + 1),

@@ -286,9 +286,9 @@ struct Workspace {
   int* tile_cnt = nullptr;   // [router_tile_counters(T)] router slices done per token tile (self-resetting)
   float* topk_w = nullptr;   // [T][k]
   // bucketing
-  uint8_t* marks = nullptr;  // [(N+E)][Tp]
-  int* rank_in = nullptr;    // [(N+E)][Tp]
-  int* key_cnt = nullptr;    // [N+E]
+  uint32_t* bits = nullptr;  // [token blocks][N+E][8] which tokens of a block have a key
+  int* blk_cnt = nullptr;    // [token blocks][N+E] their number
+  int* blk_pre = nullptr;    // [token blocks][N+E] the number in earlier blocks
   int* key_off = nullptr;    // [N+1 + E+1]: node_off then expert_off
   int* node_tok = nullptr;   // [T*k*D]
   int* row_node = nullptr;   // [T*k*D]
@@ -531,6 +531,8 @@ lx_status launch_stream(lx_layer* L, const StreamLaunch& P, cudaStream_t s, cons
 lx_status launch_bucket_small(lx_layer* L, const float* logits, const int* ids_in, int T, int k,
                               int* topk_id, float* topk_w, cudaStream_t s, bool plans = true);
 bool bucket_small_fits(const lx_layer* L, int T, int k);
+int bucket_blocks(int T);  // token blocks of the larger batches' bucketing
+int bucket_words();        // bitmap words of a key in a block
 int stream_tile_rows();
 int stream_tile_tokens();
 int stream_box();
