@@ -172,6 +172,8 @@ static lx_status ensure_workspace(lx_layer* L, int T, int k, cudaStream_t s) {
       {(void**)&w.row_node, sizeof(int) * cT * ck * D},
       {(void**)&w.node_row, sizeof(int) * cT * ck * D},
       {(void**)&w.perm, sizeof(int) * cT * ck},
+      {(void**)&w.trow, L->stream_ok ? sizeof(int) * TOK_ROWS * (size_t)cT : 0},
+      {(void**)&w.tmask, L->stream_ok ? (size_t)TOK_ROWS * cT : 0},
       {(void**)&w.tile_off, sizeof(int) * N_PLANS * (op_max_items(L) + 1)},
       {(void**)&w.h, sizeof(float) * Rmax * 2 * L->I},
       {(void**)&w.P, sizeof(float) * Rmax * 2 * rmax},

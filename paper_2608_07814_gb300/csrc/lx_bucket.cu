@@ -223,6 +223,14 @@ struct CtMeta {
   int nch, gstride, rstride, pslot;
 };
 
+// Per token its distinct rows, ascending, -1 after the last (trow [T][TOK_ROWS]),
+// and the slots whose path holds each (tmask [T][TOK_ROWS]), for the tensor-core
+// path's SwiGLU and combine; flat layers (CtMeta given): the anchor rows alone.
+struct TokRows {
+  int* trow;  // nullptr: none
+  uint8_t* tmask;
+};
+
 // The rows of every assignment, one warp per token (lane s = top-k slot s):
 // its position in its expert's bucket (perm), the rows of the nodes on its
 // path (node_row; the (token, node) pairs shared by several slots write the
@@ -237,7 +245,7 @@ k_assign_rows(const int* __restrict__ topk_id, int T, int k, int N, int E, int D
               const int* __restrict__ paths, const int* __restrict__ path_len,
               const int* __restrict__ key_off, const uint32_t* __restrict__ bits,
               const int* __restrict__ pre, int* __restrict__ node_tok, int* __restrict__ row_node,
-              int* __restrict__ perm, int* __restrict__ node_row, const CtMeta cm) {
+              int* __restrict__ perm, int* __restrict__ node_row, const CtMeta cm, const TokRows tr) {
   pdl_wait();
   const int lane = threadIdx.x & 31;
   const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -251,7 +259,7 @@ k_assign_rows(const int* __restrict__ topk_id, int T, int k, int N, int E, int D
     if (lane == __ffs(twins) - 1)  // a repeated id counts once, with its first slot
       perm[key_off[N + 1 + e] + rank_before(bits, pre, N + E, N + e, t)] = (int)a;
   }
-  int r0 = -1, r1 = -1, n0 = -1;
+  int r0 = -1, r1 = -1, n0 = -1, ev = -1;  // ev: entry `lane` = slot lane / D, level lane % D
 #pragma unroll
   for (int l = 0; l < LX_MAX_DEPTH; ++l) {
     if (l >= D) break;
@@ -266,6 +274,26 @@ k_assign_rows(const int* __restrict__ topk_id, int T, int k, int N, int E, int D
     if (lane < k) node_row[a * D + l] = row;
     if (l == 0) r0 = row;
     if (l == 1) r1 = row;
+    if (tr.tmask) {
+      const int q = __shfl_sync(0xffffffffu, row, min(lane / D, 31));
+      if (lane % D == l && lane < k * D) ev = q;
+    }
+  }
+  if (tr.tmask) {
+    // distinct rows: the first entry of each writes it at its rank
+    const unsigned same = __match_any_sync(0xffffffffu, ev);
+    const bool first = ev >= 0 && lane == __ffs(same) - 1;
+    const unsigned fm = __ballot_sync(0xffffffffu, first);
+    int rank = 0;
+    for (unsigned b = fm; b; b &= b - 1) rank += __shfl_sync(0xffffffffu, ev, __ffs(b) - 1) < ev;
+    unsigned slots = 0;
+    for (int sl = 0; sl < k; ++sl)
+      if ((same >> (sl * D)) & ((1u << D) - 1u)) slots |= 1u << sl;
+    if (first) {
+      tr.trow[(size_t)t * TOK_ROWS + rank] = ev;
+      tr.tmask[(size_t)t * TOK_ROWS + rank] = (uint8_t)slots;
+    }
+    if (lane >= __popc(fm)) tr.trow[(size_t)t * TOK_ROWS + lane] = -1;
   }
   if (!cm.al_g) return;
   // flat layers: a path is [anchor] (the dominant) or [member, anchor]
@@ -294,6 +322,13 @@ k_assign_rows(const int* __restrict__ topk_id, int T, int k, int N, int E, int D
       for (int i = 0; i < CT_MAX_CH; ++i)
         if (i == js) rr[i] = rs;
     }
+  }
+  {
+    const unsigned lm = __ballot_sync(0xffffffffu, leader);
+    int rank = 0;
+    for (unsigned b = lm; b; b &= b - 1) rank += __shfl_sync(0xffffffffu, an, __ffs(b) - 1) < an;
+    if (leader) tr.trow[(size_t)t * TOK_ROWS + rank] = an;
+    if (lane >= __popc(lm)) tr.trow[(size_t)t * TOK_ROWS + lane] = -1;
   }
   if (leader) {
 #pragma unroll
@@ -580,10 +615,15 @@ lx_status launch_bucket(lx_layer* L, const int* topk_id, int T, int k, cudaStrea
       cm.rstride = ct_rstride(L);
       cm.pslot = 2 * std::max(1, L->max_rank);
     }
+    TokRows tr{};
+    if (plan_first == PLAN_TC) {
+      tr.trow = w.trow;
+      if (!L->ct) tr.tmask = w.tmask;
+    }
     ProfScope ps(L, s, "bucket_rows");
     launch_k(L, k_assign_rows, (unsigned)((T + 7) / 8), 256, 0, s, topk_id, T, k, L->N, L->E,
              L->max_depth, L->d_paths, L->d_path_len, w.key_off, w.bits, w.blk_pre, w.node_tok,
-             w.row_node, w.perm, w.node_row, cm);
+             w.row_node, w.perm, w.node_row, cm, tr);
     LX_CUDA(cudaGetLastError());
   }
   return LX_OK;
@@ -686,7 +726,8 @@ extern "C" lx_status lx_bucket_noalloc(lx_layer* L, const int32_t* topk_id, int3
   LX_CUDA(cudaGetLastError());
   k_assign_rows<<<(unsigned)((T + 7) / 8), 256, 0, s>>>(topk_id, T, k, L->N, L->E, L->max_depth,
                                                         L->d_paths, L->d_path_len, key_off, bits, pre,
-                                                        node_tok, row_node, perm, node_row, CtMeta{});
+                                                        node_tok, row_node, perm, node_row, CtMeta{},
+                                                        TokRows{});
   LX_CUDA(cudaGetLastError());
   LX_CUDA(cudaMemcpyAsync(node_off, key_off, sizeof(int) * (L->N + 1), cudaMemcpyDeviceToDevice, s));
   LX_CUDA(cudaMemcpyAsync(expert_off, key_off + L->N + 1, sizeof(int) * (L->E + 1),

@@ -830,7 +830,7 @@ k_swiglu_warp(const float* __restrict__ topk_w, const int* __restrict__ node_row
 
 // y[t] = sum of ypart over t's distinct rows in ascending row order (an
 // anchor row split into K ranges contributes its partials in split order)
-template <typename TP, typename TY, int CPL, bool SPLIT, bool ANCHORS = false>
+template <typename TP, typename TY, int CPL, bool SPLIT>
 __global__ void __launch_bounds__(WT_WARPS * 32, 2)
 k_combine_warp(const int* __restrict__ node_row, int k, int D, const TP* __restrict__ ypart,
                int H, TY* __restrict__ y, int T, int cols_per_item, const SplitParts ys) {
@@ -850,67 +850,8 @@ k_combine_warp(const int* __restrict__ node_row, int k, int D, const TP* __restr
     const int t = (int)(it / per_tok);
     const int c_begin = (int)(it % per_tok) * cols_per_item;
     const int c_end = min(H, c_begin + cols_per_item);
-    int v_cur;
-    if constexpr (ANCHORS) {
-      // the next item's node rows are requested now, ahead of their use
-      v_cur = v_pre;
-      const long itn = it + (long)gridDim.x * WT_WARPS;
-      v_pre = (itn < items && lane < kD) ? node_row[(size_t)(itn / per_tok) * kD + lane] : -1;
-    } else {
-      v_cur = first ? v_pre : (lane < kD ? node_row[(size_t)t * kD + lane] : -1);
-    }
-    warp_token_rows(v_cur, kD, D, wr);
+    warp_token_rows(first ? v_pre : (lane < kD ? node_row[(size_t)t * kD + lane] : -1), kD, D, wr);
     const int nd = wr.nd;
-    if constexpr (ANCHORS && !SPLIT && CPL == 8 && sizeof(TP) == 2) {
-      {
-        // only the anchor rows (their down tiles already hold the members'
-        // corrections), ascending; four column passes' 16-byte loads of a
-        // batch of four rows in flight at once, each column summed in row order
-        for (int c0 = c_begin + CPL * lane; c0 < c_end; c0 += 4 * 32 * CPL) {
-          Cols<CPL> acc[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int i = 0; i < CPL; ++i) acc[u].v[i] = 0.f;
-          for (unsigned am = wr.anchor_rows; am;) {
-            int rq[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              rq[q] = -1;
-              if (am) {
-                rq[q] = wr.drow[__ffs(am) - 1];
-                am &= am - 1u;
-              }
-            }
-            uint4 v[4][4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-              for (int q = 0; q < 4; ++q)
-                if (rq[q] >= 0 && c0 + u * 32 * CPL < c_end)
-                  v[u][q] = __ldg(reinterpret_cast<const uint4*>(ypart + (size_t)rq[q] * H + c0 +
-                                                                 u * 32 * CPL));
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-              for (int q = 0; q < 4; ++q)
-                if (rq[q] >= 0 && c0 + u * 32 * CPL < c_end) {
-                  const uint32_t w4[4] = {v[u][q].x, v[u][q].y, v[u][q].z, v[u][q].w};
-#pragma unroll
-                  for (int i = 0; i < 4; ++i) {
-                    acc[u].v[2 * i] += __uint_as_float(w4[i] << 16);
-                    acc[u].v[2 * i + 1] += __uint_as_float(w4[i] & 0xFFFF0000u);
-                  }
-                }
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (c0 + u * 32 * CPL < c_end) st_cols<TY, CPL>(y + (size_t)t * H + c0 + u * 32 * CPL, acc[u]);
-        }
-        __syncwarp();
-        continue;
-      }
-    }
     for (int c = c_begin + CPL * lane; c < c_end; c += 32 * CPL) {
       Cols<CPL> acc;
 #pragma unroll
@@ -962,6 +903,133 @@ k_combine_warp(const int* __restrict__ node_row, int k, int D, const TP* __restr
       st_cols<TY, CPL>(y + (size_t)t * H + c, acc);
     }
     __syncwarp();
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The same two steps for prefill batches, a CTA per token: the bucketing has
+// written the token's distinct rows (and the slots that share each), every thread
+// owns a few columns and has several rows' loads in flight.  Finding the rows
+// in the same kernel, a warp a token, is a chain of dependent shuffles that few
+// resident warps hid: combine 38 -> 27.5 us (8192 tokens) and 23.5 ->
+// 7.4 (1031 tokens) of the Qwen3-30B-A3B-shaped layer, whose rows take 22
+// and 3 us at the HBM rate; SwiGLU of the depth-2 tree, 2048 tokens, 49 ->
+// 43 us (17 at that rate).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 ra, rb, rd;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+      "add.rn.f32x2 rd, ra, rb;\n\tmov.b64 {%0, %1}, rd;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+__device__ __forceinline__ float2 bf2(uint32_t w) {
+  return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
+}
+__device__ __forceinline__ uint32_t pack2(float2 v) {
+  const __nv_bfloat162 b = __floats2bfloat162_rn(v.x, v.y);
+  return *reinterpret_cast<const uint32_t*>(&b);
+}
+
+// y[t] = sum of ypart over t's listed rows in ascending row order
+__global__ void __launch_bounds__(256, 6)
+k_combine_tok(const int* __restrict__ trow, int max_rows, const __nv_bfloat16* __restrict__ ypart, int H,
+              __nv_bfloat16* __restrict__ y) {
+  const int4* rows = reinterpret_cast<const int4*>(trow + (size_t)blockIdx.x * TOK_ROWS);
+  // (the list comes from the bucketing, several launches before this one)
+  int4 r = __ldg(rows);
+  pdl_wait();
+  for (int c = 8 * threadIdx.x; c < H; c += 8 * blockDim.x) {
+    float2 acc[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i] = make_float2(0.f, 0.f);
+    int4 q = r;
+    for (int d = 0; d < max_rows && q.x >= 0; d += 4) {
+      const int rr[4] = {q.x, q.y, q.z, q.w};
+      uint4 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (rr[u] >= 0) v[u] = *reinterpret_cast<const uint4*>(ypart + (size_t)rr[u] * H + c);
+      if (d + 4 < max_rows) q = __ldg(rows + d / 4 + 1);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (rr[u] >= 0) {
+          const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+          for (int i = 0; i < 4; ++i) acc[i] = add2(acc[i], bf2(w[i]));
+        }
+    }
+    *reinterpret_cast<uint4*>(y + (size_t)blockIdx.x * H + c) =
+        make_uint4(pack2(acc[0]), pack2(acc[1]), pack2(acc[2]), pack2(acc[3]));
+  }
+}
+
+// z(t, n) = sum of g_s silu(sum of h_g over the path) * (sum of h_u) over the
+// slots s whose path holds n.  A thread owns four columns: every distinct row's
+// gate and up values are loaded once (six rows in flight) and added to the slots
+// whose path holds the row, rows ascending; then the acts, then the rows' z.
+__global__ void __launch_bounds__(256, 2)
+k_swiglu_tok(const float* __restrict__ topk_w, const int* __restrict__ trow,
+             const uint8_t* __restrict__ tmask, int k, const __nv_bfloat16* __restrict__ h, int I,
+             __nv_bfloat16* __restrict__ z) {
+  __shared__ int srow[TOK_ROWS], smask[TOK_ROWS];
+  __shared__ float sg[WT_SLOTS];
+  const int t = blockIdx.x, tid = threadIdx.x;
+  if (tid < TOK_ROWS) {
+    srow[tid] = trow[(size_t)t * TOK_ROWS + tid];
+    smask[tid] = tmask[(size_t)t * TOK_ROWS + tid];
+    if (tid < WT_SLOTS) sg[tid] = tid < k ? topk_w[(size_t)t * k + tid] : 0.f;
+  }
+  pdl_wait();
+  const int nd = __syncthreads_count(tid < TOK_ROWS && srow[tid < TOK_ROWS ? tid : 0] >= 0);
+  for (int c = 4 * tid; c < I; c += 4 * blockDim.x) {
+    float2 pg[WT_SLOTS][2], pu[WT_SLOTS][2];
+#pragma unroll
+    for (int s = 0; s < WT_SLOTS; ++s) pg[s][0] = pg[s][1] = pu[s][0] = pu[s][1] = make_float2(0.f, 0.f);
+    constexpr int U = 6;
+    for (int d0 = 0; d0 < nd; d0 += U) {
+      uint2 g[U], u[U];
+#pragma unroll
+      for (int q = 0; q < U; ++q)
+        if (d0 + q < nd) {
+          const __nv_bfloat16* hp = h + (size_t)srow[d0 + q] * 2 * I + c;
+          g[q] = *reinterpret_cast<const uint2*>(hp);
+          u[q] = *reinterpret_cast<const uint2*>(hp + I);
+        }
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        if (d0 + q >= nd) break;
+        const int m = smask[d0 + q];
+        const float2 g0 = bf2(g[q].x), g1 = bf2(g[q].y), u0 = bf2(u[q].x), u1 = bf2(u[q].y);
+#pragma unroll
+        for (int s = 0; s < WT_SLOTS; ++s)
+          if ((m >> s) & 1) {  // CTA-uniform
+            pg[s][0] = add2(pg[s][0], g0);
+            pg[s][1] = add2(pg[s][1], g1);
+            pu[s][0] = add2(pu[s][0], u0);
+            pu[s][1] = add2(pu[s][1], u1);
+          }
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < WT_SLOTS; ++s)  // the slot's act, in place of its gate sums
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        pg[s][i].x = sg[s] * silu_fast(pg[s][i].x) * pu[s][i].x;
+        pg[s][i].y = sg[s] * silu_fast(pg[s][i].y) * pu[s][i].y;
+      }
+    for (int d = 0; d < nd; ++d) {
+      const int m = smask[d];
+      float2 a0 = make_float2(0.f, 0.f), a1 = a0;
+#pragma unroll
+      for (int s = 0; s < WT_SLOTS; ++s)  // slots ascending
+        if ((m >> s) & 1) {
+          a0 = add2(a0, pg[s][0]);
+          a1 = add2(a1, pg[s][1]);
+        }
+      *reinterpret_cast<uint2*>(z + (size_t)srow[d] * I + c) = make_uint2(pack2(a0), pack2(a1));
+    }
   }
 }
 
@@ -1046,7 +1114,7 @@ static void launch_swiglu_warp(lx_layer* L, int T, int k, const TH* h, TZ* z, cu
 // every batch size)
 template <typename TP, typename TY>
 static void launch_combine_warp(lx_layer* L, int T, int k, const TP* ypart, TY* y, cudaStream_t s,
-                                const SplitParts& ys, bool anchors_only = false) {
+                                const SplitParts& ys) {
   Workspace& w = L->ws;
   if (ys.splits > 1) {
     const int cols = warp_item_cols(L, T, L->H, 128);
@@ -1059,13 +1127,28 @@ static void launch_combine_warp(lx_layer* L, int T, int k, const TP* ypart, TY* 
   // and loop instructions of four (measured faster at decode and prefill)
   const int cols = warp_item_cols(L, T, L->H, 256);
   const int grid = warp_grid(L, T, L->H, cols);
-  if (anchors_only && sizeof(TP) == 2) {
-    launch_k(L, k_combine_warp<TP, TY, 8, false, true>, grid, WT_WARPS * 32, 0, s, w.node_row, k,
-             L->max_depth, ypart, L->H, y, T, cols, ys);
-    return;
-  }
   launch_k(L, k_combine_warp<TP, TY, 8, false>, grid, WT_WARPS * 32, 0, s, w.node_row, k,
            L->max_depth, ypart, L->H, y, T, cols, ys);
+}
+
+// threads of a CTA that gives each thread `per` of `width` columns
+static int tok_threads(int width, int per) { return std::min(256, (width / per + 31) / 32 * 32); }
+
+lx_status launch_swiglu_tok(lx_layer* L, int T, int k, cudaStream_t s) {
+  Workspace& w = L->ws;
+  ProfScope ps(L, s, "swiglu");
+  launch_k(L, k_swiglu_tok, T, tok_threads(L->I, 4), 0, s, w.topk_w, w.trow, w.tmask, k, w.hb, L->I, w.zb);
+  LX_CUDA(cudaGetLastError());
+  return LX_OK;
+}
+
+lx_status launch_combine_tok(lx_layer* L, int T, int k, void* y, cudaStream_t s) {
+  Workspace& w = L->ws;
+  ProfScope ps(L, s, "combine");
+  launch_k(L, k_combine_tok, T, tok_threads(L->H, 8), 0, s, w.trow, k * (L->ct ? 1 : L->max_depth), w.yb,
+           L->H, static_cast<__nv_bfloat16*>(y));
+  LX_CUDA(cudaGetLastError());
+  return LX_OK;
 }
 
 lx_status launch_swiglu(lx_layer* L, int T, int k, bool bf16, cudaStream_t s, SplitParts hs) {
@@ -1092,14 +1175,12 @@ lx_status launch_swiglu(lx_layer* L, int T, int k, bool bf16, cudaStream_t s, Sp
 }
 
 lx_status launch_combine(lx_layer* L, int T, int k, void* y, bool bf16, cudaStream_t s,
-                         SplitParts ys, bool anchors_only) {
+                         SplitParts ys) {
   Workspace& w = L->ws;
   ProfScope ps(L, s, "combine");
-  if (anchors_only && !(bf16 && ys.splits <= 1 && warp_kernels_fit(L, k)))
-    return fail(LX_ERR_STATE, "anchor-row combine needs the bf16 warp form");
   if (warp_kernels_fit(L, k)) {
     if (bf16)
-      launch_combine_warp(L, T, k, L->ws.yb, static_cast<__nv_bfloat16*>(y), s, ys, anchors_only);
+      launch_combine_warp(L, T, k, L->ws.yb, static_cast<__nv_bfloat16*>(y), s, ys);
     else if (L->dtype == LX_BF16)
       launch_combine_warp(L, T, k, L->ws.ypart, static_cast<__nv_bfloat16*>(y), s, ys);
     else

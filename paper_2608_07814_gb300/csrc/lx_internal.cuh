@@ -142,6 +142,7 @@ enum OpKind {
 // The streaming kernels decode their tiles from the streaming work items instead.
 constexpr int N_PLANS = 2 * N_OPS;
 constexpr int PLAN_TC = N_OPS;
+constexpr int TOK_ROWS = 32;  // k * depth of the tensor-core path at most
 constexpr int N_TILE_COUNTERS = 16;  // dynamic tile counters, zeroed by the bucketing
 
 // Per-op shape rule: for node n with rank r, each group has
@@ -294,6 +295,8 @@ struct Workspace {
   int* row_node = nullptr;   // [T*k*D]
   int* node_row = nullptr;   // [T*k*D]
   int* perm = nullptr;       // [T*k]
+  int* trow = nullptr;       // [T][TOK_ROWS] a token's distinct rows (tensor-core path)
+  uint8_t* tmask = nullptr;  // [T][TOK_ROWS] the slots whose path holds them
   int* tile_off = nullptr;   // [N_PLANS][max_items+1]
   // generic path intermediates (fp32)
   float* h = nullptr;        // [Rmax][2I]
@@ -483,10 +486,12 @@ bool warp_kernels_fit(const lx_layer* L, int k);
 // all bf16); false: the generic form (fp32 h, z, ypart)
 lx_status launch_swiglu(lx_layer* L, int T, int k, bool bf16, cudaStream_t s,
                         SplitParts hs = SplitParts());
-// anchors_only: sum only the anchor rows of each token (their down tiles
-// already hold the members' corrections)
 lx_status launch_combine(lx_layer* L, int T, int k, void* y, bool bf16, cudaStream_t s,
-                         SplitParts ys = SplitParts(), bool anchors_only = false);
+                         SplitParts ys = SplitParts());
+// the tensor-core path's forms, a CTA per token over the rows the bucketing
+// listed (bf16 h, z, ypart; warp_kernels_fit)
+lx_status launch_swiglu_tok(lx_layer* L, int T, int k, cudaStream_t s);
+lx_status launch_combine_tok(lx_layer* L, int T, int k, void* y, cudaStream_t s);
 lx_status launch_fast_experts(lx_layer* L, const void* x, int T, int k, void* y, cudaStream_t s);
 lx_status launch_tc_experts(lx_layer* L, const void* x, int T, int k, void* y, cudaStream_t s);
 int tc_tile_tokens();  // rows of the TMA boxes of the tensor-core A operands

@@ -868,13 +868,13 @@ lx_status launch_tc_experts(lx_layer* L, const void* x, int T, int k, void* y, c
     dn.kc_slot = (int)rmax;
     dn.omap = w.omaps ? w.omaps + 1 : nullptr;  // yb
     LX_TRY(run(dn, "tc_dn_anchor_U"));
-    return launch_combine(L, T, k, y, true, s, SplitParts(), /*anchors_only=*/true);
+    return launch_combine_tok(L, T, k, y, s);
   } else {
     LX_TRY(run(gathered(tc_op(L, OP_UP_V, w.gmap, 0, w.Pb, 2 * rmax, false, 1)),
                "tc_up_V"));
     LX_TRY(run(tc_op(L, OP_UP_U, w.xmaps + 0, 0, w.hb, 2 * I, false, 2),
                "tc_up_U"));
-    LX_TRY(launch_swiglu(L, T, k, true, s));
+    LX_TRY(launch_swiglu_tok(L, T, k, s));
   }
   LX_TRY(run(tc_op(L, OP_DN_ANCHOR, w.xmaps + 1, 0, w.yb, H, false, 3),
              "tc_dn_anchor"));
@@ -882,7 +882,7 @@ lx_status launch_tc_experts(lx_layer* L, const void* x, int T, int k, void* y, c
              "tc_dn_V"));
   LX_TRY(run(tc_op(L, OP_DN_U, w.xmaps + 2, 0, w.yb, H, false, 5),
              "tc_dn_U"));
-  LX_TRY(launch_combine(L, T, k, y, true, s));
+  LX_TRY(launch_combine_tok(L, T, k, y, s));
   return LX_OK;
 }
 
