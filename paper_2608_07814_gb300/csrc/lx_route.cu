@@ -382,10 +382,23 @@ k_router_tiled(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restr
 constexpr float RS_EPS_REL = 1e-3f;
 constexpr int RS_MAX_CAND = 32;
 constexpr int RS_WARPS = 8;
-constexpr int RS_U = 4;  // 16-byte weight chunks of a lane in flight per candidate (two candidates)
 
-template <int EPL>
-__global__ void __launch_bounds__(RS_WARPS * 32, 3)
+// A warp per token.  Instructions and the latency of warp-wide reductions bound
+// it (a shuffle or redux with its use takes 40 to 55 cycles here), so the two
+// selections are kept short: the k-th largest approximate logit by k rounds over
+// lane-sorted keys (one redux a round; equal keys leave together, which can only
+// lower the threshold), and the top-k of the candidates, at most one a lane, by
+// counting for each the candidates ahead of it (independent shuffles).
+// U: 16-byte chunks of a candidate's router row that a lane has in flight (two
+// candidates at a time): 8, whole rows of up to 2048 elements at once, with three
+// CTAs an SM; 4 and four CTAs for longer rows (measured at H = 2560, E = 256, 4096
+// tokens: 41 us, 53 with 8).  Measured, Qwen3-30B-A3B-shaped router: 8192 tokens
+// 49 -> 46 us; a route call of 2048 tokens 35.0 -> 33.0, of 1031 32.6 -> 29.1 (two
+// ordered top-k a token and U = 4 before).  Tried: the candidates of 8 or 16
+// tokens gathered per expert, so that a router row is loaded once for all of them:
+// 50 and 67 us at 8192 tokens (the loads do not bound it).
+template <int EPL, int U>
+__global__ void __launch_bounds__(RS_WARPS * 32, U == 8 ? 3 : 4)
 k_router_screen(const float* __restrict__ part, int splits, int Epad,
                 const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ W,
                 const float* __restrict__ bias, int T, int E, int H, float wmax, int k,
@@ -393,30 +406,21 @@ k_router_screen(const float* __restrict__ part, int splits, int Epad,
   extern __shared__ __align__(16) unsigned char smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   __nv_bfloat16* xs = reinterpret_cast<__nv_bfloat16*>(smem) + (size_t)warp * H;
-  float* ls = reinterpret_cast<float*>(smem + (size_t)RS_WARPS * H * 2) + (size_t)warp * E;
+  float* ls = reinterpret_cast<float*>(smem + (size_t)RS_WARPS * H * 2) + (size_t)warp * max(E, 2 * LX_MAX_K);
   pdl_wait();
-  const int t = blockIdx.x * RS_WARPS + warp;
+  const int t = blockIdx.x * RS_WARPS + warp, nchunk = H / 8;
   if (t >= T) return;
-  // the token's row into shared memory, and ||x_t||^2
-  const uint4* xr = reinterpret_cast<const uint4*>(x + (size_t)t * H);
-  uint4* xw = reinterpret_cast<uint4*>(xs);
-  float ss = 0.f;
-  for (int i = lane; i < H / 8; i += 32) {
-    const uint4 v = __ldg(xr + i);
-    xw[i] = v;
-    const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float a = __uint_as_float(w4[q] << 16), b = __uint_as_float(w4[q] & 0xFFFF0000u);
-      ss = fmaf(a, a, ss);
-      ss = fmaf(b, b, ss);
-    }
+  // the token's row into shared memory, while the approximate logits (K ranges
+  // in order, then the bias) come
+  {
+    const uint4* xr = reinterpret_cast<const uint4*>(x + (size_t)t * H);
+    const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(xs));
+    for (int i = lane; i < nchunk; i += 32)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * i), "l"(xr + i) : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
   }
-#pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-  // the approximate logits (K ranges in order, then the bias)
   float ap[EPL];
-  bool finite = ss == ss && ss <= 3.0e38f;
+  bool finite = true;
 #pragma unroll
   for (int i = 0; i < EPL; ++i) {
     const int e = lane + 32 * i;
@@ -425,20 +429,56 @@ k_router_screen(const float* __restrict__ part, int splits, int Epad,
       for (int sp = 0; sp < splits; ++sp) v += part[((size_t)sp * T + t) * Epad + e];
       if (bias) v += bias[e];
       finite = finite && (v - v == 0.f);
-      ls[e] = v;
     }
     ap[i] = v;
   }
-  finite = __all_sync(0xffffffffu, finite);
+  // this lane's keys in descending order (0: none)
+  uint32_t key[EPL];
+#pragma unroll
+  for (int i = 0; i < EPL; ++i) key[i] = lane + 32 * i < E ? topk_key(ap[i]) : 0u;
+#pragma unroll
+  for (int n = 0; n < EPL; ++n)
+#pragma unroll
+    for (int i = n & 1; i + 1 < EPL; i += 2) {  // odd-even transposition
+      const uint32_t hi = max(key[i], key[i + 1]), lo = min(key[i], key[i + 1]);
+      key[i] = hi;
+      key[i + 1] = lo;
+    }
+  uint32_t kth = 0u;
+  for (int j = 0; j < k; ++j) {
+    kth = __reduce_max_sync(0xffffffffu, key[0]);
+    if (key[0] == kth) {
+#pragma unroll
+      for (int i = 0; i + 1 < EPL; ++i) key[i] = key[i + 1];
+      key[EPL - 1] = 0u;
+    }
+  }
+  // ||x_t||^2
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncwarp();
+  const uint4* xw = reinterpret_cast<const uint4*>(xs);
+  float s2[2] = {0.f, 0.f};
+  for (int i = lane; i < nchunk; i += 32) {
+    const uint4 v = xw[i];
+    const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float a = __uint_as_float(w4[q] << 16), b = __uint_as_float(w4[q] & 0xFFFF0000u);
+      s2[0] = fmaf(a, a, s2[0]);
+      s2[1] = fmaf(b, b, s2[1]);
+    }
+  }
+  float ss = s2[0] + s2[1];
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  finite = finite && ss == ss && ss <= 3.0e38f;
+  finite = __all_sync(0xffffffffu, finite);
   unsigned cand[EPL];
   int ncand = E;
   if (finite) {
-    // the k-th largest approximate logit
-    int sid;
-    float sw;
-    warp_topk(ls, E, k, sid, sw);
-    const float Lk = ls[__shfl_sync(0xffffffffu, sid, k - 1)];
+    // (k distinct keys at most were left: E >= k, so a missing one is the least
+    // key, which makes every expert a candidate)
+    const float Lk = kth ? topk_key_value(kth) : -INFINITY;
     // both terms of the bound, with a margin for the fp32 norm itself
     const float eps = RS_EPS_REL * sqrtf(ss) * 1.001f * wmax;
     ncand = 0;
@@ -449,26 +489,16 @@ k_router_screen(const float* __restrict__ part, int splits, int Epad,
       ncand += __popc(cand[i]);
     }
   }
-  if (!finite || ncand > RS_MAX_CAND) {
-#pragma unroll
-    for (int i = 0; i < EPL; ++i) cand[i] = (lane + 32 * i) < E ? 0xffffffffu : 0u;
+  const bool all = !finite || ncand > RS_MAX_CAND;
+  if (all) {
 #pragma unroll
     for (int i = 0; i < EPL; ++i) cand[i] = __ballot_sync(0xffffffffu, lane + 32 * i < E);
   }
-  __syncwarp();
-  // non-candidates can never be selected
-#pragma unroll
-  for (int i = 0; i < EPL; ++i) {
-    const int e = lane + 32 * i;
-    if (e < E && !((cand[i] >> lane) & 1u)) ls[e] = -INFINITY;
-  }
-  __syncwarp();
   // canonical fp32 logits of the candidates: lane j accumulates the 8-element
   // chunks q = j, j + 32, ... of the dot product with fused multiply-adds in
   // ascending order; the lane partials are added at offsets 16, 8, 4, 2, 1
   // (lane j, j < off, adds lane j + off's); the bias last
   // Two candidates at a time (two independent chains sharing the x loads).
-  const int nchunk = H / 8;
   auto pop = [&]() {  // the next candidate (warp-uniform), -1 when none is left
     int e = -1;
 #pragma unroll
@@ -479,21 +509,23 @@ k_router_screen(const float* __restrict__ part, int splits, int Epad,
       }
     return e;
   };
+  int my_id = 0x7fffffff, at = 0;  // lane c: the c-th candidate (ascending ids) and its logit
+  float my_l = 0.f;
   for (int e0 = pop(); e0 >= 0; e0 = pop()) {
     const int e1 = pop();
     const uint4* w0 = reinterpret_cast<const uint4*>(W + (size_t)e0 * H);
     const uint4* w1 = reinterpret_cast<const uint4*>(W + (size_t)(e1 >= 0 ? e1 : e0) * H);
     float acc0 = 0.f, acc1 = 0.f;
-    for (int q0 = lane; q0 < nchunk; q0 += 32 * RS_U) {
-      uint4 wv0[RS_U], wv1[RS_U];
+    for (int q0 = lane; q0 < nchunk; q0 += 32 * U) {
+      uint4 wv0[U], wv1[U];
 #pragma unroll
-      for (int u = 0; u < RS_U; ++u) {
+      for (int u = 0; u < U; ++u) {
         const bool in = q0 + 32 * u < nchunk;
         wv0[u] = in ? __ldg(w0 + q0 + 32 * u) : make_uint4(0u, 0u, 0u, 0u);
         wv1[u] = in && e1 >= 0 ? __ldg(w1 + q0 + 32 * u) : make_uint4(0u, 0u, 0u, 0u);
       }
 #pragma unroll
-      for (int u = 0; u < RS_U; ++u) {
+      for (int u = 0; u < U; ++u) {
         if (q0 + 32 * u >= nchunk) break;
         const uint4 xv = xw[q0 + 32 * u];
         acc0 = fma_bf16_pair(acc0, xv.x, wv0[u].x);
@@ -511,15 +543,58 @@ k_router_screen(const float* __restrict__ part, int splits, int Epad,
       acc0 = __fadd_rn(acc0, __shfl_down_sync(0xffffffffu, acc0, off));
       acc1 = __fadd_rn(acc1, __shfl_down_sync(0xffffffffu, acc1, off));
     }
-    if (lane == 0) {
-      ls[e0] = bias ? __fadd_rn(acc0, bias[e0]) : acc0;
-      if (e1 >= 0) ls[e1] = bias ? __fadd_rn(acc1, bias[e1]) : acc1;
+    acc0 = __shfl_sync(0xffffffffu, acc0, 0);
+    acc1 = __shfl_sync(0xffffffffu, acc1, 0);
+    if (bias) {
+      acc0 = __fadd_rn(acc0, bias[e0]);
+      if (e1 >= 0) acc1 = __fadd_rn(acc1, bias[e1]);
     }
+    if (all) {
+      if (lane == 0) {
+        ls[e0] = acc0;
+        if (e1 >= 0) ls[e1] = acc1;
+      }
+    } else {
+      if (lane == at) {
+        my_id = e0;
+        my_l = acc0;
+      }
+      if (lane == at + 1 && e1 >= 0) {
+        my_id = e1;
+        my_l = acc1;
+      }
+    }
+    at += 2;
   }
-  __syncwarp();
   int id;
   float w;
-  warp_topk(ls, E, k, id, w);
+  if (all) {
+    __syncwarp();
+    warp_topk_t<EPL>(ls, E, k, id, w);
+  } else {
+    // the candidates ahead of this lane's: larger logit, or equal and a lower id
+    // (lanes hold them in ascending id); finite logits, so the keys order them
+    const uint32_t mk = lane < ncand ? topk_key(my_l) : 0u;
+    int ahead = 0;
+    for (int c = 0; c < ncand; ++c) {
+      const uint32_t kc = __shfl_sync(0xffffffffu, mk, c);
+      ahead += kc > mk || (kc == mk && c < lane);
+    }
+    // slot `ahead` (ls: scratch of this warp) <- (logit, id)
+    int* lid = reinterpret_cast<int*>(ls) + k;
+    if (lane < ncand && ahead < k) {
+      ls[ahead] = my_l;
+      lid[ahead] = my_id;
+    }
+    __syncwarp();
+    const float v = lane < k ? ls[lane] : 0.f;
+    id = lane < k ? lid[lane] : 0;
+    // softmax over the k, summed in slot order
+    const float ex = expf(v - __shfl_sync(0xffffffffu, v, 0));
+    float denom = 0.f;
+    for (int j = 0; j < k; ++j) denom += __shfl_sync(0xffffffffu, ex, j);
+    w = ex / denom;
+  }
   if (lane < k) {
     topk_id[(size_t)t * k + lane] = id;
     topk_w[(size_t)t * k + lane] = w;
@@ -534,12 +609,42 @@ bool router_is_tiled(const lx_layer* L, int T) {
          2 * (size_t)RTT_TOK * L->H * 2 + (size_t)RTT_TOK * L->E * 4 <= 200 * 1024;
 }
 
+// a token row and E logits (or k logits and ids) a warp
+static size_t screen_smem(const lx_layer* L) {
+  return (size_t)RS_WARPS * ((size_t)L->H * 2 + 4 * (size_t)std::max(L->E, 2 * LX_MAX_K));
+}
+
+// Whether the screened route pays when only ids and gates are asked for.  Its
+// cost hardly depends on the batch below about 1200 tokens (two launches, about
+// 16 us); the full logits' grows with T E H.  Measured route calls (bucketing
+// included), full -> screened: E = 128, H = 2048: T = 257 26.5 -> 28.8 us, 320
+// 29.9 -> 28.2, 512 37.7 -> 29.4, 1031 48.3 -> 29.1; E = 256, H = 2560: T = 200
+// 41.3 -> 41.6, 257 44.3 -> 40.1, 1031 102 -> 45.8.
+static bool screen_pays(const lx_layer* L, int T) {
+  if (!L->router_screen || screen_smem(L) > 200 * 1024) return false;
+  return router_is_tiled(L, T) || (T >= 256 && (double)T * L->E * L->H >= 80e6);
+}
+
+template <int EPL, int U>
+static lx_status launch_screen(lx_layer* L, const void* x, int T, int k, int splits, int Epad, int* topk_id,
+                               float* topk_w, cudaStream_t s) {
+  static bool done[64] = {};
+  LX_CUDA(smem_cap_once((const void*)k_router_screen<EPL, U>, 200 * 1024, L->device, done));
+  ProfScope ps(L, s, "router_select");
+  launch_k(L, k_router_screen<EPL, U>, (unsigned)((T + RS_WARPS - 1) / RS_WARPS), RS_WARPS * 32,
+           screen_smem(L), s, (const float*)L->ws.rs_part, splits, Epad, (const __nv_bfloat16*)x,
+           (const __nv_bfloat16*)L->router_w, (const float*)L->router_bias, T, L->E, L->H, L->router_wmax,
+           k, topk_id, topk_w);
+  LX_CUDA(cudaGetLastError());
+  return LX_OK;
+}
+
 lx_status launch_router(lx_layer* L, const void* x, int T, int k, float* logits, int* topk_id,
                         float* topk_w, cudaStream_t s, bool need_logits) {
   if (reinterpret_cast<uintptr_t>(x) % 16)
     return fail(LX_ERR_ARG, "x must be 16-byte aligned");
   const int tiles = (T + RT_TOK - 1) / RT_TOK;
-  if (!need_logits && L->router_screen && router_is_tiled(L, T)) {
+  if (!need_logits && screen_pays(L, T)) {
     // screened: approximate logits on the tensor cores, then the candidates'
     // canonical logits and the top-k (the logits buffer is not written)
     CUtensorMap xm;
@@ -550,25 +655,11 @@ lx_status launch_router(lx_layer* L, const void* x, int T, int k, float* logits,
     int splits = 1;
     LX_TRY(tc_splitk_gemm(L, xm, L->router_map, T, Epad, L->H, L->ws.rs_part, RS_MAX_SPLITS,
                           &splits, s, "router_screen"));
-    const size_t smem = (size_t)RS_WARPS * ((size_t)L->H * 2 + (size_t)L->E * 4);
-    if (smem > 200 * 1024) return fail(LX_ERR_SHAPE, "router screening rows exceed shared memory");
-    const unsigned grid = (unsigned)((T + RS_WARPS - 1) / RS_WARPS);
-    ProfScope ps(L, s, "router_select");
-    if (L->E <= 128) {
-      static bool done4[64] = {};
-      LX_CUDA(smem_cap_once((const void*)k_router_screen<4>, 200 * 1024, L->device, done4));
-      launch_k(L, k_router_screen<4>, grid, RS_WARPS * 32, smem, s, (const float*)L->ws.rs_part,
-               splits, Epad, (const __nv_bfloat16*)x, (const __nv_bfloat16*)L->router_w,
-               (const float*)L->router_bias, T, L->E, L->H, L->router_wmax, k, topk_id, topk_w);
-    } else {
-      static bool done8[64] = {};
-      LX_CUDA(smem_cap_once((const void*)k_router_screen<8>, 200 * 1024, L->device, done8));
-      launch_k(L, k_router_screen<8>, grid, RS_WARPS * 32, smem, s, (const float*)L->ws.rs_part,
-               splits, Epad, (const __nv_bfloat16*)x, (const __nv_bfloat16*)L->router_w,
-               (const float*)L->router_bias, T, L->E, L->H, L->router_wmax, k, topk_id, topk_w);
-    }
-    LX_CUDA(cudaGetLastError());
-    return LX_OK;
+    if (L->E <= 128)
+      return L->H <= 2048 ? launch_screen<4, 8>(L, x, T, k, splits, Epad, topk_id, topk_w, s)
+                          : launch_screen<4, 4>(L, x, T, k, splits, Epad, topk_id, topk_w, s);
+    return L->H <= 2048 ? launch_screen<8, 8>(L, x, T, k, splits, Epad, topk_id, topk_w, s)
+                        : launch_screen<8, 4>(L, x, T, k, splits, Epad, topk_id, topk_w, s);
   }
   if (router_is_tiled(L, T)) {
     // large batch: persistent register-tiled kernel
