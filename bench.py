@@ -678,7 +678,7 @@ def run_offline(args, rank, world, local_rank):
                      "value": round(whole_job_rate(T, 1, world, ms), 1), "unit": "tokens/s",
                      "ms_per_step": round(ms, 5), "higher_is_better": True, "dtype": "int64",
                      "gpu_launches": args.steps,
-                     "roofline": {"kernel": "k_coact_smem", "bound": "hbm",
+                     "roofline": {"kernel": "k_coact_bits", "bound": "hbm",
                                   "achieved": round(byts / (ms * 1e-3) / 1e9, 1), "peak": hbm,
                                   "unit": "GB/s", "frac": round(byts / (ms * 1e-3) / 1e9 / hbm, 5),
                                   "traffic": None, "note": "latency-bound: 256 KB of ids per launch"},
