@@ -108,3 +108,22 @@ def test_rejected_calls():
     perm = torch.arange(16, dtype=torch.int32, device="cuda")
     assert L.lx_permute_neurons(lx.LX_F32, 16, 16, lx._ptr(perm), p, p, p, p, p, p,
                                 None) == lx.LX_ERR_ARG   # in place
+
+
+@pytest.mark.parametrize("H,I,dtype", [(8, 8, torch.bfloat16), (264, 520, torch.float32), (16, 24584, torch.bfloat16),
+                                       (24, 12296, torch.float32), (520, 2056, torch.bfloat16)])
+def test_permute_row_stages(H, I, dtype):
+    """Down rows around the staging limit (48 KB), a last block of few rows, and
+    entries of perm outside the range."""
+    g = torch.Generator().manual_seed(I)
+    gate, up = torch.randn(I, H, generator=g).to(dtype), torch.randn(I, H, generator=g).to(dtype)
+    down = torch.randn(H, I, generator=g).to(dtype)
+    perm = torch.randperm(I, generator=g).to(torch.int32)
+    perm[1], perm[I // 2] = -1, I
+    out = lx.permute_neurons(perm.cuda(), gate.cuda(), up.cuda(), down.cuda())
+    ok = (perm >= 0) & (perm < I)
+    at = torch.where(ok, perm, 0).long()
+    zero = torch.zeros((), dtype=dtype)
+    assert torch.equal(out[0].cpu(), torch.where(ok[:, None], gate[at], zero))
+    assert torch.equal(out[1].cpu(), torch.where(ok[:, None], up[at], zero))
+    assert torch.equal(out[2].cpu(), torch.where(ok[None], down[:, at], zero))
