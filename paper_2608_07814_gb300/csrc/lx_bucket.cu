@@ -76,12 +76,12 @@ static_assert(BK_WORDS == 8 && LX_MAX_DEPTH == 4, "two 16-byte pieces a key, one
 __device__ __forceinline__ int rank_before(const uint32_t* __restrict__ bits, const int* __restrict__ pre,
                                            int keys, int key, int t) {
   const size_t row = (size_t)(t / BK_TOK) * keys + key;
-  const uint4 a = __ldg(reinterpret_cast<const uint4*>(bits) + 2 * row);
-  const uint4 b = __ldg(reinterpret_cast<const uint4*>(bits) + 2 * row + 1);
+  const uint4 a = __ldcg(reinterpret_cast<const uint4*>(bits) + 2 * row);
+  const uint4 b = __ldcg(reinterpret_cast<const uint4*>(bits) + 2 * row + 1);
   const uint32_t v[BK_WORDS] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
   const int w = (t % BK_TOK) >> 5;
   const uint32_t below = (1u << (t & 31)) - 1u;
-  int r = __ldg(pre + row);
+  int r = __ldcg(pre + row);
 #pragma unroll
   for (int j = 0; j < BK_WORDS; ++j) r += __popc(v[j] & (j < w ? 0xffffffffu : j == w ? below : 0u));
   return r;
