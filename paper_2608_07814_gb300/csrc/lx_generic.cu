@@ -672,23 +672,25 @@ k_swiglu_warp(const float* __restrict__ topk_w, const int* __restrict__ node_row
   const long items = (long)T * per_tok;
   long it = (long)blockIdx.x * WT_WARPS + warp;
   // The routing tables (node rows, gates) come from the routing and bucketing
-  // kernels, at least two launches before this one: the first item's entries
-  // are loaded before the wait for the preceding kernel.
-  int v_pre = -1;
-  float g_pre = 0.f;
+  // kernels, at least two launches before this one: the first item's rows are
+  // found before the wait for the preceding kernel (a small batch has one item a
+  // warp, and the search is a chain of shuffles).
   if (it < items) {
     const int t = (int)(it / per_tok);
-    if (lane < kD) v_pre = node_row[(size_t)t * kD + lane];
-    if (lane < k) g_pre = topk_w[(size_t)t * k + lane];
+    warp_token_rows(lane < kD ? node_row[(size_t)t * kD + lane] : -1, kD, D, wr);
+    if (lane < k) wr.g[lane] = topk_w[(size_t)t * k + lane];
+    __syncwarp();
   }
   pdl_wait();
   for (bool first = true; it < items; it += (long)gridDim.x * WT_WARPS, first = false) {
     const int t = (int)(it / per_tok);
     const int c_begin = (int)(it % per_tok) * cols_per_item;
     const int c_end = min(I, c_begin + cols_per_item);
-    warp_token_rows(first ? v_pre : (lane < kD ? node_row[(size_t)t * kD + lane] : -1), kD, D, wr);
-    if (lane < k) wr.g[lane] = first ? g_pre : topk_w[(size_t)t * k + lane];
-    __syncwarp();
+    if (!first) {
+      warp_token_rows(lane < kD ? node_row[(size_t)t * kD + lane] : -1, kD, D, wr);
+      if (lane < k) wr.g[lane] = topk_w[(size_t)t * k + lane];
+      __syncwarp();
+    }
     const int nd = wr.nd;
     for (int c = c_begin + CPL * lane; c < c_end; c += 32 * CPL) {
       Cols<CPL> act[WT_SLOTS];
@@ -842,15 +844,15 @@ k_combine_warp(const int* __restrict__ node_row, int k, int D, const TP* __restr
   const long items = (long)T * per_tok;
   long it = (long)blockIdx.x * WT_WARPS + warp;
   // node rows come from the bucketing, several launches before this one: the
-  // first item's entries are loaded before the wait for the preceding kernel
-  int v_pre = -1;
-  if (it < items && lane < kD) v_pre = node_row[(size_t)(it / per_tok) * kD + lane];
+  // first item's rows are found before the wait for the preceding kernel
+  if (it < items)
+    warp_token_rows(lane < kD ? node_row[(size_t)(it / per_tok) * kD + lane] : -1, kD, D, wr);
   pdl_wait();
   for (bool first = true; it < items; it += (long)gridDim.x * WT_WARPS, first = false) {
     const int t = (int)(it / per_tok);
     const int c_begin = (int)(it % per_tok) * cols_per_item;
     const int c_end = min(H, c_begin + cols_per_item);
-    warp_token_rows(first ? v_pre : (lane < kD ? node_row[(size_t)t * kD + lane] : -1), kD, D, wr);
+    if (!first) warp_token_rows(lane < kD ? node_row[(size_t)t * kD + lane] : -1, kD, D, wr);
     const int nd = wr.nd;
     for (int c = c_begin + CPL * lane; c < c_end; c += 32 * CPL) {
       Cols<CPL> acc;
