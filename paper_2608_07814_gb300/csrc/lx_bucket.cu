@@ -116,40 +116,66 @@ __device__ void publish_active(const int* cnt, const int* list, int n, int which
   const int lane = threadIdx.x & 31;
   int* out = act + (which == 0 ? 0 : n_anchor * STREAM_DEP_TB);
   int base = 0;
-  for (int i0 = 0; i0 < n && blk > 0; i0 += 32) {
-    const int i = i0 + lane;
-    const int node = i < n ? list[i] : -1;
-    // blocks of this node's bucket (the host passes blk only for batches of
-    // at most STREAM_DEP_TB blocks)
-    const int nb = node >= 0 ? (cnt[node] + blk - 1) / blk : 0;
-    int incl = nb;
+  constexpr int U = 4;  // groups of 32 nodes whose scans overlap
+  for (int i0 = 0; i0 < n && blk > 0; i0 += 32 * U) {
+    int node[U], nb[U], incl[U];
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int x = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += x;
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + 32 * u + lane;
+      node[u] = i < n ? list[i] : -1;
+      // blocks of this node's bucket (the host passes blk only for batches of
+      // at most STREAM_DEP_TB blocks)
+      nb[u] = incl[u] = node[u] >= 0 ? (cnt[node[u]] + blk - 1) / blk : 0;
     }
-    for (int b = 0; b < nb; ++b) out[base + incl - nb + b] = node * STREAM_DEP_TB + b;
-    base += __shfl_sync(0xffffffffu, incl, 31);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int x = __shfl_up_sync(0xffffffffu, incl[u], o);
+        if (lane >= o) incl[u] += x;
+      }
+    int total[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) total[u] = __shfl_sync(0xffffffffu, incl[u], 31);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      for (int b = 0; b < nb[u]; ++b) out[base + incl[u] - nb[u] + b] = node[u] * STREAM_DEP_TB + b;
+      base += total[u];
+    }
   }
   if (lane == 0) act_n[which] = base;
 }
 
-// One warp: exclusive offsets out[0 .. n] of counts v(i), i < n.
+// One warp: exclusive offsets out[0 .. n] of counts v(i), i < n.  Four groups of
+// 32 at a time, so that their scans' shuffles (about 40 cycles each) overlap.
 template <typename F>
 __device__ __forceinline__ void warp_offsets(int n, F v, int* out) {
   const int lane = threadIdx.x & 31;
+  constexpr int U = 4;
   int carry = 0;
-  for (int base = 0; base < n; base += 32) {
-    const int i = base + lane;
-    const int x0 = i < n ? v(i) : 0;
-    int incl = x0;
+  for (int base = 0; base < n; base += 32 * U) {
+    int x[U], incl[U];
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int x = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += x;
+    for (int u = 0; u < U; ++u) {
+      const int i = base + 32 * u + lane;
+      x[u] = incl[u] = i < n ? v(i) : 0;
     }
-    if (i < n) out[i] = carry + incl - x0;
-    carry += __shfl_sync(0xffffffffu, incl, 31);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int y = __shfl_up_sync(0xffffffffu, incl[u], o);
+        if (lane >= o) incl[u] += y;
+      }
+    int total[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) total[u] = __shfl_sync(0xffffffffu, incl[u], 31);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = base + 32 * u + lane;
+      if (i < n) out[i] = carry + incl[u] - x[u];
+      carry += total[u];
+    }
   }
   if (lane == 0) out[n] = carry;
 }
@@ -444,31 +470,20 @@ k_bucket_small(const float* __restrict__ logits, const int* __restrict__ ids_in,
     return r;
   };
   __syncthreads();
-  // 4. node offsets (warp 0) and expert offsets (warp 1): warp scans with a carry
-  if (warp < 2) {
-    const int n0 = warp == 0 ? 0 : N, n = warp == 0 ? N : E;
-    const int o0 = warp == 0 ? 0 : N + 1;
-    int carry = 0;
-    for (int base = 0; base < n; base += 32) {
-      const int i = base + lane;
-      const int v = i < n ? cnt[n0 + i] : 0;
-      int incl = v;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int x = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += x;
-      }
-      if (i < n) off[o0 + i] = carry + incl - v;
-      carry += __shfl_sync(0xffffffffu, incl, 31);
-    }
-    if (lane == 0) off[o0 + n] = carry;
+  // 4. node offsets (warp 0), expert offsets (warp 1) and, from the same counts,
+  // the streaming work items (warps 2 and 3); the others clear the counters
+  if (warp == 0) {
+    warp_offsets(N, [&](int i) { return cnt[i]; }, off);
+  } else if (warp == 1) {
+    warp_offsets(E, [&](int i) { return cnt[N + i]; }, off + N + 1);
+  } else if (warp < 4) {
+    publish_active(cnt, warp == 2 ? slist : slist + n_anchor, warp == 2 ? n_anchor : n_corr, warp - 2, n_anchor,
+                   blk, act, act_n);
+  } else {
+    for (int i = tid - 4 * 32; i < n_sctr; i += nth - 4 * 32) sctr[i] = 0;
   }
   __syncthreads();
   for (int i = tid; i < keys + 2; i += nth) key_off_g[i] = off[i];
-  for (int i = tid; i < n_sctr; i += nth) sctr[i] = 0;
-  if (warp < 2)
-    publish_active(cnt, warp == 0 ? slist : slist + n_anchor, warp == 0 ? n_anchor : n_corr, warp, n_anchor,
-                   blk, act, act_n);
   // 5. tile plans: one warp per plan
   for (int p = warp; p < pa.n_plans; p += nw) {
     int* to = tile_off + (pa.first + p) * (max_items + 1);

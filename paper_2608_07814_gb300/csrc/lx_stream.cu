@@ -353,8 +353,6 @@ __device__ __forceinline__ bool consume_tile(const StreamLaunch& P, const TileIn
 
 __global__ void __launch_bounds__(SW_THREADS, SW_CTAS_PER_SM)
 k_stream_gemm(const __grid_constant__ StreamLaunch P) {
-  if (!P.early_weights) pdl_wait();
-  else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -375,6 +373,9 @@ k_stream_gemm(const __grid_constant__ StreamLaunch P) {
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // (the barriers' set-up overlaps the preceding kernel)
+  if (!P.early_weights) pdl_wait();
+  else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   __syncthreads();
   uint32_t it = 0;
   if (warp == 0) {
