@@ -88,7 +88,6 @@ __device__ __forceinline__ int rank_before(const uint32_t* __restrict__ bits, co
 }
 
 struct PlanArgs {
-  const int* items[N_PLANS];
   int n_items[N_PLANS];
   OpShape shape[N_PLANS];
   int bm[N_PLANS], bn[N_PLANS];  // token rows and output columns per tile
@@ -236,7 +235,7 @@ k_offsets_plan(const int* __restrict__ cnt, int nblk, int N, int E, int* __restr
                  tile_off + (pa.first + p) * (max_items + 1));
   }
 }
-static_assert(4 + N_OPS <= OP_THREADS / 32, "a warp for every role");
+static_assert(4 + N_OPS < OP_THREADS / 32 && 4 + N_OPS < 32, "a warp for every role, here and in k_bucket_small");
 
 // The fused path's per-cluster-row tables (flat layers on the tensor-core
 // path; al_g == nullptr: none): see k_assign_rows.
@@ -471,7 +470,8 @@ k_bucket_small(const float* __restrict__ logits, const int* __restrict__ ids_in,
   };
   __syncthreads();
   // 4. node offsets (warp 0), expert offsets (warp 1) and, from the same counts,
-  // the streaming work items (warps 2 and 3); the others clear the counters
+  // the streaming work items (warps 2 and 3) and the tile plans (a warp each); the
+  // others clear the counters
   if (warp == 0) {
     warp_offsets(N, [&](int i) { return cnt[i]; }, off);
   } else if (warp == 1) {
@@ -479,34 +479,19 @@ k_bucket_small(const float* __restrict__ logits, const int* __restrict__ ids_in,
   } else if (warp < 4) {
     publish_active(cnt, warp == 2 ? slist : slist + n_anchor, warp == 2 ? n_anchor : n_corr, warp - 2, n_anchor,
                    blk, act, act_n);
+  } else if (warp - 4 < pa.n_plans) {
+    const int p = warp - 4;
+    warp_offsets(pa.n_items[p], [&](int i) {
+      const int n = pa.shape[p].on_anchors ? slist[i] : slist[n_anchor + i];
+      return plan_tiles(pa, p, srank[n], cnt[n]);
+    }, tile_off + (pa.first + p) * (max_items + 1));
   } else {
-    for (int i = tid - 4 * 32; i < n_sctr; i += nth - 4 * 32) sctr[i] = 0;
+    const int first = 32 * (4 + pa.n_plans);
+    for (int i = tid - first; i < n_sctr; i += nth - first) sctr[i] = 0;
   }
   __syncthreads();
   for (int i = tid; i < keys + 2; i += nth) key_off_g[i] = off[i];
-  // 5. tile plans: one warp per plan
-  for (int p = warp; p < pa.n_plans; p += nw) {
-    int* to = tile_off + (pa.first + p) * (max_items + 1);
-    int carry = 0;
-    for (int base = 0; base < pa.n_items[p]; base += 32) {
-      const int i = base + lane;
-      int v = 0;
-      if (i < pa.n_items[p]) {
-        const int n = pa.items[p][i];
-        v = plan_tiles(pa, p, srank[n], cnt[n]);
-      }
-      int incl = v;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int x = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += x;
-      }
-      if (i < pa.n_items[p]) to[i] = carry + incl - v;
-      carry += __shfl_sync(0xffffffffu, incl, 31);
-    }
-    if (lane == 0) to[pa.n_items[p]] = carry;
-  }
-  // 6. scatter from the assignments: bucket rows, node rows, permutation
+  // 5. scatter from the assignments: bucket rows, node rows, permutation
   for (int a = tid; a < T * k; a += nth) {
     const int t = a / k, e = ids[a];
     const bool valid = e >= 0 && e < E;
@@ -541,7 +526,6 @@ static PlanArgs make_plans(const lx_layer* L, int n_plans, int first = 0) {
     const int slot = first + p;
     const int op = slot % N_OPS;
     pa.shape[p] = op_shape(L, op);
-    pa.items[p] = pa.shape[p].on_anchors ? L->d_anchors : L->d_corrs;
     pa.n_items[p] = pa.shape[p].on_anchors ? L->n_anchor : L->n_corr;
     pa.bm[p] = slot < PLAN_TC ? G_BM : tc_tile_rows(L, op);
     pa.bn[p] = slot < PLAN_TC ? G_BN : tc_tile_cols();
@@ -549,7 +533,6 @@ static PlanArgs make_plans(const lx_layer* L, int n_plans, int first = 0) {
       // the fused correction + SwiGLU kernel takes this slot: tiles of 128
       // cluster rows x CT_CW d_ff columns over the anchors
       pa.shape[p] = OpShape{L->I, 0, 0, 0, 1, 1};
-      pa.items[p] = L->d_anchors;
       pa.n_items[p] = L->n_anchor;
       pa.bm[p] = 128;
       pa.bn[p] = CT_CW;

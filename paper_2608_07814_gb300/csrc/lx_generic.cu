@@ -40,8 +40,10 @@ namespace {
 // fp32 weights: fused multiply-adds in ascending K (4 x 4 outputs a thread).
 // Measured on the Qwen3-30B-A3B-shaped layer with rank 32 at 96 tokens, whole
 // forward: 1669 us with a
-// scalar-load, single-buffered form, 214 us with this one; the tiny fp32 layer
-// (d_model 64, 256 tokens) 74.6 -> 33.7 us.
+// scalar-load, single-buffered form, 195 us with this one (212 before the first
+// tile of a launch was looked up, and its weights requested, ahead of the wait for
+// the preceding one); the tiny fp32 layer
+// (d_model 64, 256 tokens) 74.6 -> 30.6 us.
 // ---------------------------------------------------------------------------
 constexpr int GG_THREADS = 128;
 constexpr int GG_STAGES = 4;
@@ -51,6 +53,10 @@ constexpr int GG_WBYTES = G_BN * 128;  // weight rows of a chunk, 128 bytes each
 struct GemmLaunch {
   GemmArgs op[2];
   int n_ops;
+  // 1: the tile lists and buckets were complete before the preceding launch
+  // (only the rows of A come from it): the first tile is looked up and its
+  // weights are requested before the wait for that launch
+  int early;
 };
 
 template <typename TA, typename TW>
@@ -166,7 +172,9 @@ k_grouped_gemm(const __grid_constant__ GemmLaunch P) {
   using C = GG<TA, TW>;
   constexpr int BK = C::BK, UA = C::AROW / 16;
   constexpr int EW = 16 / (int)sizeof(TW), EA = 16 / (int)sizeof(TA);  // elements of a unit
-  pdl_wait();
+  if (P.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  else pdl_wait();
+  bool waited = !P.early;
   extern __shared__ __align__(128) unsigned char gsm[];
   __shared__ const TA* arow[G_BM];  // the tile's rows of A (null past the bucket)
   const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(gsm));
@@ -211,17 +219,21 @@ k_grouped_gemm(const __grid_constant__ GemmLaunch P) {
       return o.tiled ? W + ((((size_t)((col0 + c) >> 6) * (K >> 6) + (kx >> 6)) * 64 + ((col0 + c) & 63)) * 64 + (kx & 63))
                      : W + (size_t)(col0 + c) * K + kx;
     };
-    auto fetch = [&](int ch) {
-      if (ch < nch) {
-        const int k0 = ch * BK;
-        const uint32_t ws = base + (ch % GG_STAGES) * C::STAGE, as = ws + G_BN * C::WLD;
-        if (vec) {
+    // what: 1 the weights, 2 the rows of A, 3 both
+    auto fetch = [&](int ch, int what) {
+      if (ch >= nch) return;
+      const int k0 = ch * BK;
+      const uint32_t ws = base + (ch % GG_STAGES) * C::STAGE, as = ws + G_BN * C::WLD;
+      if (vec) {
+        if (what & 1) {
 #pragma unroll
           for (int i = 0; i < G_BN * 8 / GG_THREADS; ++i) {
             const int q = tid + i * GG_THREADS, c = q >> 3, u = q & 7;
             const bool ok = c < cols && k0 + u * EW < K;
             gg_cp16(ws + c * C::WLD + 16 * (C::MMA ? gg_pos<8>(u, c) : u), ok ? w_at(c, k0 + u * EW) : W, ok);
           }
+        }
+        if (what & 2) {
 #pragma unroll
           for (int i = 0; i < G_BM * UA / GG_THREADS; ++i) {
             const int q = tid + i * GG_THREADS, m = q / UA, u = q % UA;
@@ -229,38 +241,50 @@ k_grouped_gemm(const __grid_constant__ GemmLaunch P) {
             gg_cp16(as + m * C::ALD + 16 * (C::MMA ? gg_pos<UA>(u, m) : u),
                     ok ? (const void*)(arow[m] + k0 + u * EA) : o.A, ok);
           }
-        } else {
-          unsigned char* wsp = gsm + (ch % GG_STAGES) * C::STAGE;
-          unsigned char* asp = wsp + G_BN * C::WLD;
+        }
+      } else {
+        unsigned char* wsp = gsm + (ch % GG_STAGES) * C::STAGE;
+        unsigned char* asp = wsp + G_BN * C::WLD;
+        if (what & 1)
           for (int q = tid; q < G_BN * BK; q += GG_THREADS) {
             const int c = q / BK, k = q % BK, u = k / EW;
             TW v = from_f32<TW>(0.f);
             if (c < cols && k0 + k < K) v = *w_at(c, k0 + k);
             *reinterpret_cast<TW*>(wsp + c * C::WLD + 16 * (C::MMA ? gg_pos<8>(u, c) : u) + (k % EW) * sizeof(TW)) = v;
           }
+        if (what & 2)
           for (int q = tid; q < G_BM * BK; q += GG_THREADS) {
             const int m = q / BK, k = q % BK, u = k / EA;
             TA v = from_f32<TA>(0.f);
             if (m < rows && k0 + k < K) v = arow[m][k0 + k];
             *reinterpret_cast<TA*>(asp + m * C::ALD + 16 * (C::MMA ? gg_pos<UA>(u, m) : u) + (k % EA) * sizeof(TA)) = v;
           }
-        }
       }
-      asm volatile("cp.async.commit_group;" ::: "memory");
     };
+    auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
     float sum[G_BM / 8][4];  // mma: [8-row group][fragment]; fp32: [row][column]
 #pragma unroll
     for (int j = 0; j < G_BM / 8; ++j)
 #pragma unroll
       for (int c = 0; c < 4; ++c) sum[j][c] = 0.f;
-#pragma unroll
-    for (int ch = 0; ch < GG_STAGES - 1; ++ch) fetch(ch);
+    int left = 3;  // what is left to fetch of the first chunks
+    if (!waited) {
+      for (int ch = 0; ch < GG_STAGES - 1; ++ch) fetch(ch, 1);
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      waited = true;
+      left = 2;
+    }
+    for (int ch = 0; ch < GG_STAGES - 1; ++ch) {
+      fetch(ch, left);
+      commit();
+    }
     const int nt = (rows + 7) / 8;
     const int tx = tid & 15, ty = tid >> 4;
     for (int ch = 0; ch < nch; ++ch) {
       asm volatile("cp.async.wait_group %0;" ::"n"(GG_STAGES - 2) : "memory");
       __syncthreads();  // chunk ch has landed, and chunk ch - 1's stage is free
-      fetch(ch + GG_STAGES - 1);
+      fetch(ch + GG_STAGES - 1, 3);
+      commit();
       const uint32_t ws = base + (ch % GG_STAGES) * C::STAGE, as = ws + G_BN * C::WLD;
       if constexpr (C::MMA) {
         if (nt == 1) gg_chunk_mma<TA, 1>(ws, as, sum);
@@ -309,6 +333,8 @@ k_grouped_gemm(const __grid_constant__ GemmLaunch P) {
           if (4 * ty + i < rows && tx + 16 * j < cols) out[(size_t)(4 * ty + i) * o.ldo + tx + 16 * j] = sum[i][j];
     }
   }
+  // (a CTA without tiles: this grid may not complete before its predecessor)
+  if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 __device__ __forceinline__ float silu_f(float v) { return v / (1.f + expf(-v)); }
@@ -1227,6 +1253,7 @@ template <typename TA, typename TW, int OPK>
 lx_status run_gemm(lx_layer* L, std::initializer_list<GemmArgs> ops, cudaStream_t s, const char* name) {
   GemmLaunch P;
   P.n_ops = 0;
+  P.early = OPK != OP_UP_ANCHOR;  // the x side follows the bucketing directly
   for (const GemmArgs& g : ops)
     if (g.n_items > 0) P.op[P.n_ops++] = g;
   if (P.n_ops == 0) return LX_OK;
