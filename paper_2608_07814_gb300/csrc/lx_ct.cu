@@ -112,16 +112,16 @@ __device__ __forceinline__ void ct_decode_warp(const CtLaunch& P, int tile, CtTi
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int i = i0 + lane + 32 * j;
-      v[j] = i < P.n_items ? __ldg(to + i) : INT_MAX;
+      v[j] = i < P.n_items ? __ldcg(to + i) : INT_MAX;
     }
 #pragma unroll
     for (int j = 0; j < 8; ++j) cnt += __popc(__ballot_sync(0xffffffffu, v[j] <= tile));
   }
   const int lo = cnt - 1;
   const int n = __ldg(P.items + lo);
-  const int local = tile - __ldg(to + lo);
+  const int local = tile - __ldcg(to + lo);
   const int nchunk = P.I / CT_CW;
-  const int b0 = __ldg(P.node_off + n), b1 = __ldg(P.node_off + n + 1);
+  const int b0 = __ldcg(P.node_off + n), b1 = __ldcg(P.node_off + n + 1);
   t.node = n;
   t.q = local % nchunk;
   t.tok0 = b0 + (local / nchunk) * CT_BM;
@@ -209,7 +209,9 @@ __device__ __forceinline__ uint32_t pack_bf2(float a, float b) {
 
 __global__ void __launch_bounds__(CT_THREADS, 1) k_ct_swiglu(const __grid_constant__ CtLaunch P) {
   constexpr int S = CT_STAGES;
-  pdl_wait();
+  // (set-up and the first tiles' lookups need nothing of the preceding launch; the
+  // producer waits for it before its first load)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -272,6 +274,7 @@ __global__ void __launch_bounds__(CT_THREADS, 1) k_ct_swiglu(const __grid_consta
     // ------------------------------------------------------------ producer
     uint32_t it = 0, qi = 0, ht = 0;
     bool ok = true;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     while (ok) {
       int got = 1;
       if (lane == 0) got = mbar_wait(qfull, qi & 1, abort_flag, P.wait_cycles);
@@ -385,6 +388,8 @@ __global__ void __launch_bounds__(CT_THREADS, 1) k_ct_swiglu(const __grid_consta
       }
       ++qi;
       if (cur >= total) break;
+      // (one tile a CTA before the preceding launch is done, as in the GEMM)
+      if (qi == 1) asm volatile("griddepcontrol.wait;" ::: "memory");
     }
     if (!ok && lane == 0) {
       atomicExch(P.err, LX_ERR_TIMEOUT);

@@ -95,16 +95,16 @@ __device__ __forceinline__ void tc_decode_warp(const TcLaunch& P, int tile, TcTi
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int i = i0 + lane + 32 * j;
-      v[j] = i < P.n_items ? __ldg(to + i) : INT_MAX;
+      v[j] = i < P.n_items ? __ldcg(to + i) : INT_MAX;
     }
 #pragma unroll
     for (int j = 0; j < 8; ++j) cnt += __popc(__ballot_sync(0xffffffffu, v[j] <= tile));
   }
   const int lo = cnt - 1;
   const int n = __ldg(P.items + lo);
-  const int local = tile - __ldg(to + lo);
+  const int local = tile - __ldcg(to + lo);
   const int r = __ldg(P.rank + n);
-  const int b0 = __ldg(P.node_off + n), b1 = __ldg(P.node_off + n + 1);
+  const int b0 = __ldcg(P.node_off + n), b1 = __ldcg(P.node_off + n + 1);
   t.Ng = P.shape.n_const + P.shape.n_rank * r;
   t.K = P.shape.k_const + P.shape.k_rank * r;
   if (P.kc_child) {
@@ -144,7 +144,13 @@ k_tc_gemm(const __grid_constant__ TcLaunch P) {
   using C = TcCfg<BM, EPI>;
   constexpr int TC_STAGES = C::STAGES, TC_STAGE_BYTES = C::STAGE_BYTES, TC_A_BYTES = C::A_BYTES;
   constexpr int NH = C::NH, NBUF = C::NBUF;
-  pdl_wait();
+  // No wait for the preceding launch here: the tile lists, the gathered token rows
+  // and the weights were complete before it.  Only the A rows read by TMA come from
+  // it: the producer waits before it loads the first of them (the first tile's
+  // weight boxes are on their way by then), so a CTA's set-up, its first tile and
+  // those boxes overlap the preceding launch's last tiles on other SMs.  Every
+  // CTA's producer waits before the CTA ends, so the launches complete in order.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -200,7 +206,7 @@ k_tc_gemm(const __grid_constant__ TcLaunch P) {
     // Tiles come decoded from the scheduler warp's queue, so that the TMA
     // issue never waits on the plan lookups.
     uint32_t it = 0, qi = 0;
-    bool ok = true;
+    bool ok = true, waited = false;
     while (ok) {
       const uint32_t q = qi % TC_QN;
       int got = 1;
@@ -228,6 +234,23 @@ k_tc_gemm(const __grid_constant__ TcLaunch P) {
         my_nkb = my_child >= 0 ? __ldg(P.rank + my_child) / TC_BK : 0;
       }
       int cj = 0, ckb = 0;
+      // a 256-row tile whose rows end within its first half loads one half
+      const int nh = GATHER ? 0 : ((NH == 2 && t.M > 128) ? 2 : 1);
+      int npre = 0;  // first K blocks whose stage already has its weights
+      if (!waited && !GATHER) {
+        npre = min(min(nkb, kb_own), TC_STAGES);
+        if (lane == 0)
+          for (int kb = 0; kb < npre; ++kb) {  // fresh stages: nothing to wait for
+            if (kb == 0) slot[0] = t;
+            mbar_expect_tx(full0 + 8 * kb, nbox * 8192 + nh * 128 * TC_BK * 2);
+            for (int b = 0; b < nbox; ++b)
+              tma_load_4d(smem_base + kb * TC_STAGE_BYTES + TC_A_BYTES + b * 8192, P.wmaps + t.node, 0, 0, kb,
+                          rt0 + b, full0 + 8 * kb);
+          }
+        __syncwarp();
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        waited = true;
+      }
       for (int kb = 0; kb < nkb; ++kb, ++it) {
         const uint32_t s = it % TC_STAGES;
         int cnode = -1, cnkb = 0;
@@ -237,16 +260,16 @@ k_tc_gemm(const __grid_constant__ TcLaunch P) {
         }
         int good = 1;
         if (lane == 0) {
-          good = mbar_wait(empty0 + 8 * s, ((it / TC_STAGES) & 1) ^ 1, abort_flag,
-                           P.wait_cycles) ? 1 : 0;
+          const bool pre = kb < npre;
+          if (!pre)
+            good = mbar_wait(empty0 + 8 * s, ((it / TC_STAGES) & 1) ^ 1, abort_flag,
+                             P.wait_cycles) ? 1 : 0;
           if (good) {
-            if (kb == 0) slot[s] = t;
-            // a 256-row tile whose rows end within its first half loads one half
-            const int nh = GATHER ? 0 : ((NH == 2 && t.M > 128) ? 2 : 1);
-            mbar_expect_tx(full0 + 8 * s, nbox * 8192 + nh * 128 * TC_BK * 2);
+            if (kb == 0 && !pre) slot[s] = t;
+            if (!pre) mbar_expect_tx(full0 + 8 * s, nbox * 8192 + nh * 128 * TC_BK * 2);
             const uint32_t a_s = smem_base + s * TC_STAGE_BYTES, b_s = a_s + TC_A_BYTES;
             if (kb < kb_own) {
-              for (int b = 0; b < nbox; ++b)
+              for (int b = 0; b < nbox && !pre; ++b)
                 tma_load_4d(b_s + b * 8192, P.wmaps + t.node, 0, 0, kb, rt0 + b, full0 + 8 * s);
               for (int h = 0; h < nh; ++h)
                 tma_load_2d(a_s + h * 128 * TC_BK * 2, P.xmap,
@@ -297,6 +320,8 @@ k_tc_gemm(const __grid_constant__ TcLaunch P) {
       atomicExch(P.err, LX_ERR_TIMEOUT);
       *abort_flag = 1;
     }
+    __syncwarp();
+    if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
     prod_it = it;
   } else if (GATHER && (warp == 3 || warp >= 4 + EPI)) {
     // ------------------------------------------------------------ gather
@@ -338,7 +363,7 @@ k_tc_gemm(const __grid_constant__ TcLaunch P) {
 #pragma unroll
       for (int i = 0; i < GR; ++i) {
         const int m = 4 * (gw * GR + i) + r8;
-        const int tr = (m < t.M && (long)t.tok0 + m < P.rows_cap) ? __ldg(P.gather + t.tok0 + m) : -1;
+        const int tr = (m < t.M && (long)t.tok0 + m < P.rows_cap) ? __ldcg(P.gather + t.tok0 + m) : -1;
         src[i] = tr >= 0 ? P.xsrc + (size_t)tr * P.ldx + (size_t)(t.grp * t.K) + 8 * u : nullptr;
       }
       const int nkb = (t.K + TC_BK - 1) / TC_BK;
@@ -418,6 +443,10 @@ k_tc_gemm(const __grid_constant__ TcLaunch P) {
       }
       ++qi;
       if (cur >= total) break;
+      // a CTA that starts beside the preceding launch takes one tile and no more
+      // before that launch is done: the first CTAs would otherwise hold the tiles
+      // of a short launch while the others find none
+      if (!GATHER && qi == 1) asm volatile("griddepcontrol.wait;" ::: "memory");
     }
     if (!ok && lane == 0) {
       atomicExch(P.err, LX_ERR_TIMEOUT);
