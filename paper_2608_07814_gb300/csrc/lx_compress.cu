@@ -159,11 +159,28 @@ k_cgemm(const TW* __restrict__ Wm, const TW* __restrict__ Wd, const float* __res
 // L = 136) leave most SMs idle and each runs n serial steps, so the rows are
 // cut into up to GR_SPLITS ranges (blockIdx.z) of 256 or more, whose pairs the
 // Cholesky adds in order: 26.9 -> 19.1 us a launch at L = 136 (n = 768 and 2048).
+// The issue rate bounds it, so the ranges are counted by the rows of the SM with
+// the most CTAs (gram_parts): n = 2048 takes 3 (135 CTAs, one an SM, 683 rows
+// each) before 4 (180 CTAs, two on some SMs): 28.0 -> 24.4 us.
 constexpr int GR_SPLITS = 4;
 constexpr int GR_T = 16;
 constexpr int GR_KC = 64;
 constexpr int GR_CH = 4;
 static_assert(GR_KC * GR_T % (GR_T * GR_T) == 0, "whole staged values per thread");
+
+// row ranges of a Gram of n rows and L columns
+static int gram_parts(int n, int L, int sms) {
+  const int t = (L + GR_T - 1) / GR_T, tiles = t * (t + 1) / 2;
+  int best = 1, cost = 0x7fffffff;
+  for (int p = 1; p <= std::min(GR_SPLITS, std::max(1, n / 256)); ++p) {
+    const int c = (tiles * p + sms - 1) / sms * ((n + p - 1) / p);
+    if (c < cost) {
+      cost = c;
+      best = p;
+    }
+  }
+  return best;
+}
 
 struct DF {
   float hi, lo;
@@ -472,18 +489,18 @@ __device__ __forceinline__ uint32_t os_smem(const void* p) {
 // factor's inverse is never formed and half of the products of a full GEMM are
 // left out.  One CTA takes TS_ROWS rows against the whole factor in shared
 // memory (block rows of 16, each as long as it is, four words of padding so
-// that the eight rows a warp reads fall on distinct banks); thread (row, c)
-// owns columns c and c + 8 of a block.  Latency of the nine block steps bounds
-// it at l = 136: 16 us (the GEMM with the formed inverse took
-// 13, but forming it 80 of the Cholesky's 152).
+// that eight rows read at once fall on distinct banks); thread (row, c) owns
+// column c of a block.  Instruction latency of its few warps bounds it: at
+// l = 136 16.8 us with two columns a thread and copies of 4 bytes, 9.7 so (the
+// GEMM with the formed inverse took 13, but forming it 80 of the Cholesky's 152).
 constexpr int TS_ROWS = 16;
-constexpr int TS_THREADS = 8 * TS_ROWS;
+constexpr int TS_THREADS = CH_B * TS_ROWS;
 __host__ __device__ inline int ts_off(int kb) { return CH_B * (8 * kb * (kb + 1) + 4 * kb); }
 __host__ __device__ inline int ts_ldy(int nb) { return nb * CH_B + 4; }
 
 __global__ void __launch_bounds__(TS_THREADS)
 k_trsm(const float* __restrict__ X, const float* __restrict__ Lf, const float* __restrict__ Dinv,
-       int n, int L, float* __restrict__ Y) {
+       int n, int L, int vec, float* __restrict__ Y) {
   extern __shared__ __align__(16) float ts[];
   const int nb = (L + CH_B - 1) / CH_B, ldy = ts_ldy(nb);
   float* Lb = ts;                       // block row kb at ts_off(kb), rows of 16 (kb + 1) + 4
@@ -491,63 +508,69 @@ k_trsm(const float* __restrict__ X, const float* __restrict__ Lf, const float* _
   float* Ss = Ys + TS_ROWS * ldy;       // [TS_ROWS][CH_B + 4]
   float* Ds = Ss + TS_ROWS * (CH_B + 4);  // [nb][CH_B][CH_B + 4]
   const int tid = threadIdx.x, row0 = blockIdx.x * TS_ROWS;
-  // every copy in flight at once (4 bytes each: l need not be a multiple of 4)
+  // every copy in flight at once: 16 bytes each where the rows allow it
   auto cp4 = [](float* dst, const float* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(os_smem(dst)), "l"(src) : "memory");
   };
-  for (int r = tid >> 5; r < L; r += TS_THREADS / 32) {
-    const int kb = r / CH_B, ld = CH_B * (kb + 1) + 4;
-    float* dst = Lb + ts_off(kb) + (r - kb * CH_B) * ld;
-    for (int c = tid & 31; c < CH_B * kb; c += 32) cp4(dst + c, Lf + (size_t)r * L + c);
-  }
-  for (int r = tid >> 5; r < TS_ROWS; r += TS_THREADS / 32)
-    for (int c = tid & 31; c < nb * CH_B; c += 32) {
-      if (row0 + r < n && c < L) cp4(Ys + r * ldy + c, X + (size_t)(row0 + r) * L + c);
-      else Ys[r * ldy + c] = 0.f;
+  auto cp16 = [](float* dst, const float* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(os_smem(dst)), "l"(src) : "memory");
+  };
+  if (L % 4 == 0 && vec) {
+    for (int r = tid >> 4; r < L; r += TS_THREADS / 16) {
+      const int kb = r / CH_B, ld = CH_B * (kb + 1) + 4;
+      float* dst = Lb + ts_off(kb) + (r - kb * CH_B) * ld;
+      for (int c = 4 * (tid & 15); c < CH_B * kb; c += 64) cp16(dst + c, Lf + (size_t)r * L + c);
     }
-  for (int e = tid; e < nb * CH_B * CH_B; e += TS_THREADS)
-    cp4(Ds + (e / CH_B) * (CH_B + 4) + e % CH_B, Dinv + e);
+    for (int r = tid >> 4; r < TS_ROWS; r += TS_THREADS / 16)
+      for (int c = 4 * (tid & 15); c < nb * CH_B; c += 64) {
+        if (row0 + r < n && c < L) cp16(Ys + r * ldy + c, X + (size_t)(row0 + r) * L + c);
+        else *reinterpret_cast<float4*>(Ys + r * ldy + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+  } else {
+    for (int r = tid >> 5; r < L; r += TS_THREADS / 32) {
+      const int kb = r / CH_B, ld = CH_B * (kb + 1) + 4;
+      float* dst = Lb + ts_off(kb) + (r - kb * CH_B) * ld;
+      for (int c = tid & 31; c < CH_B * kb; c += 32) cp4(dst + c, Lf + (size_t)r * L + c);
+    }
+    for (int r = tid >> 5; r < TS_ROWS; r += TS_THREADS / 32)
+      for (int c = tid & 31; c < nb * CH_B; c += 32) {
+        if (row0 + r < n && c < L) cp4(Ys + r * ldy + c, X + (size_t)(row0 + r) * L + c);
+        else Ys[r * ldy + c] = 0.f;
+      }
+  }
+  for (int e = 4 * tid; e < nb * CH_B * CH_B; e += 4 * TS_THREADS)
+    cp16(Ds + (e / CH_B) * (CH_B + 4) + e % CH_B, Dinv + e);
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
-  const int c = tid & 7, r = tid >> 3;
+  const int c = tid % CH_B, r = tid / CH_B;
   float* yr = Ys + r * ldy;
   float* sr = Ss + r * (CH_B + 4);
   for (int kb = 0; kb < nb; ++kb) {
     const int j0 = kb * CH_B, ld = CH_B * (kb + 1) + 4;
     const float* l0 = Lb + ts_off(kb) + c * ld;
-    const float* l1 = l0 + 8 * ld;
-    float s0[4] = {}, s1[4] = {};
-    const bool in0 = j0 + c < L, in1 = j0 + c + 8 < L;  // factor rows that exist
+    float s0[4] = {};
+    if (j0 + c < L) {  // a factor row that exists
 #pragma unroll 4
-    for (int j = 0; j < j0; j += 4) {
-      const float4 y = *reinterpret_cast<const float4*>(yr + j);
-      const float4 a = in0 ? *reinterpret_cast<const float4*>(l0 + j) : make_float4(0.f, 0.f, 0.f, 0.f);
-      const float4 b = in1 ? *reinterpret_cast<const float4*>(l1 + j) : make_float4(0.f, 0.f, 0.f, 0.f);
-      s0[0] = fmaf(y.x, a.x, s0[0]);
-      s0[1] = fmaf(y.y, a.y, s0[1]);
-      s0[2] = fmaf(y.z, a.z, s0[2]);
-      s0[3] = fmaf(y.w, a.w, s0[3]);
-      s1[0] = fmaf(y.x, b.x, s1[0]);
-      s1[1] = fmaf(y.y, b.y, s1[1]);
-      s1[2] = fmaf(y.z, b.z, s1[2]);
-      s1[3] = fmaf(y.w, b.w, s1[3]);
+      for (int j = 0; j < j0; j += 4) {
+        const float4 y = *reinterpret_cast<const float4*>(yr + j);
+        const float4 a = *reinterpret_cast<const float4*>(l0 + j);
+        s0[0] = fmaf(y.x, a.x, s0[0]);
+        s0[1] = fmaf(y.y, a.y, s0[1]);
+        s0[2] = fmaf(y.z, a.z, s0[2]);
+        s0[3] = fmaf(y.w, a.w, s0[3]);
+      }
     }
     sr[c] = yr[j0 + c] - ((s0[0] + s0[1]) + (s0[2] + s0[3]));
-    sr[c + 8] = yr[j0 + c + 8] - ((s1[0] + s1[1]) + (s1[2] + s1[3]));
-    __syncwarp();  // a row's eight threads are in one warp
+    __syncwarp();  // a row's sixteen threads are in one warp
     const float* d0 = Ds + (j0 + c) * (CH_B + 4);
-    const float* d1 = d0 + 8 * (CH_B + 4);
-    float t0 = 0.f, t1 = 0.f;
+    float t0 = 0.f;
 #pragma unroll
     for (int p = 0; p < CH_B; p += 4) {
       const float4 s = *reinterpret_cast<const float4*>(sr + p);
       const float4 a = *reinterpret_cast<const float4*>(d0 + p);
-      const float4 b = *reinterpret_cast<const float4*>(d1 + p);
       t0 = fmaf(s.w, a.w, fmaf(s.z, a.z, fmaf(s.y, a.y, fmaf(s.x, a.x, t0))));
-      t1 = fmaf(s.w, b.w, fmaf(s.z, b.z, fmaf(s.y, b.y, fmaf(s.x, b.x, t1))));
     }
     yr[j0 + c] = t0;
-    yr[j0 + c + 8] = t1;
     __syncwarp();
   }
   __syncthreads();
@@ -562,19 +585,21 @@ __global__ void k_trmm(const float* __restrict__ L1, const float* __restrict__ L
                        float* __restrict__ Mt) {
   const int i = blockIdx.x, j = threadIdx.x;
   if (j >= L) return;
-  // two compensated sums (as in the Gram), sixteen loads in flight: a float64
-  // fma and the widening of its operands run at 1/64 of the fp32 rate
+  // two compensated sums (as in the Gram): a float64 fma and the widening of its
+  // operands run at 1/64 of the fp32 rate.  Thirty-two loads in flight, and a
+  // warp's lanes walk the same k from its first column on (zeros before a lane's
+  // own), so that a load reads one row piece: 20.1 us at L = 136 with every lane starting at its column, 5.6 so.
   DF acc[2] = {DF{0.f, 0.f}, DF{0.f, 0.f}};
-  for (int k = j; k <= i; k += 16) {
-    float a[16], b[16];
+  for (int k = j & ~31; k <= i; k += 32) {
+    float a[32], b[32];
 #pragma unroll
-    for (int u = 0; u < 16; ++u) {
-      const bool in = k + u <= i;
+    for (int u = 0; u < 32; ++u) {
+      const bool in = k + u >= j && k + u <= i;
       a[u] = in ? L1[(size_t)i * L + k + u] : 0.f;
       b[u] = in ? L2[(size_t)(k + u) * L + j] : 0.f;
     }
 #pragma unroll
-    for (int u = 0; u < 16; ++u) {
+    for (int u = 0; u < 32; ++u) {
       const float p = __fmul_rn(a[u], b[u]);
       df_add(acc[u & 1], p, __fmaf_rn(a[u], b[u], -p));
     }
@@ -1159,13 +1184,14 @@ lx_status run_compress(int rows, int cols, const TW* Wd, const TW* Wm, const flo
   LX_CUDA(smem_cap_once((const void*)k_chol32, (int)CP_SMEM_CAP, dev, g_ch_cap));
   LX_CUDA(smem_cap_once((const void*)k_trsm, (int)CP_SMEM_CAP, dev, g_ts_cap));
   auto cholqr = [&](const float* X, float* out, int n, float shift, float* Lf) {
-    const int want = std::min(GR_SPLITS, std::max(1, n / 256));
+    const int want = gram_parts(n, l, num_sms);
     const int span = ((n + want - 1) / want + GR_KC - 1) / GR_KC * GR_KC;
     const int parts = (n + span - 1) / span;
     const dim3 grid((l + GR_T - 1) / GR_T, (l + GR_T - 1) / GR_T, parts);
     k_gram<<<grid, GR_T * GR_T, 0, s>>>(X, n, l, span, G);
     k_chol32<<<1, CH_THREADS, ch_smem, s>>>(G, parts, l, ldp, shift, Lf, w.Dinv);
-    k_trsm<<<(n + TS_ROWS - 1) / TS_ROWS, TS_THREADS, ts_smem, s>>>(X, Lf, w.Dinv, n, l, out);
+    k_trsm<<<(n + TS_ROWS - 1) / TS_ROWS, TS_THREADS, ts_smem, s>>>(X, Lf, w.Dinv, n, l,
+                                                                        reinterpret_cast<uintptr_t>(X) % 16 == 0, out);
   };
   // CholeskyQR (the first pass shifted by 1e-6 of the largest Gram diagonal,
   // so rank-deficient bases stay factorable).  orth2 runs it twice, X [n][l]
