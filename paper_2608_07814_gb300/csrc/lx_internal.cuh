@@ -264,6 +264,11 @@ struct TcLaunch {
   const int* gather;
   const __nv_bfloat16* xsrc;
   long ldx;
+  // late: this launch lets its successor start only once its own predecessor is
+  // complete, so that a successor with `ready` set finds its A rows (not those of
+  // the concatenated children) written and reads them without a wait
+  int late;
+  int ready;
   // optional TMA map of out (bf16, 32 x 32 boxes, 64-byte swizzle): 256-row
   // tiles store whole 32-row blocks with TMA (row_map null)
   const CUtensorMap* omap;

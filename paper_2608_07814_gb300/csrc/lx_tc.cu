@@ -150,7 +150,9 @@ k_tc_gemm(const __grid_constant__ TcLaunch P) {
   // weight boxes are on their way by then), so a CTA's set-up, its first tile and
   // those boxes overlap the preceding launch's last tiles on other SMs.  Every
   // CTA's producer waits before the CTA ends, so the launches complete in order.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // (`late` and `ready`: see TcLaunch; a ready launch waits only where it needs
+  // its predecessor's own output, the children's rows along K.)
+  if (!P.late) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -237,7 +239,7 @@ k_tc_gemm(const __grid_constant__ TcLaunch P) {
       // a 256-row tile whose rows end within its first half loads one half
       const int nh = GATHER ? 0 : ((NH == 2 && t.M > 128) ? 2 : 1);
       int npre = 0;  // first K blocks whose stage already has its weights
-      if (!waited && !GATHER) {
+      if (!waited && !GATHER && !P.ready) {
         npre = min(min(nkb, kb_own), TC_STAGES);
         if (lane == 0)
           for (int kb = 0; kb < npre; ++kb) {  // fresh stages: nothing to wait for
@@ -249,12 +251,17 @@ k_tc_gemm(const __grid_constant__ TcLaunch P) {
           }
         __syncwarp();
         asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (P.late) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         waited = true;
       }
       for (int kb = 0; kb < nkb; ++kb, ++it) {
         const uint32_t s = it % TC_STAGES;
         int cnode = -1, cnkb = 0;
         if (kb >= kb_own) {  // warp-uniform: every lane takes child cj's entry
+          if (!waited) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            waited = true;
+          }
           cnode = __shfl_sync(0xffffffffu, my_child, cj);
           cnkb = __shfl_sync(0xffffffffu, my_nkb, cj);
         }
@@ -446,7 +453,7 @@ k_tc_gemm(const __grid_constant__ TcLaunch P) {
       // a CTA that starts beside the preceding launch takes one tile and no more
       // before that launch is done: the first CTAs would otherwise hold the tiles
       // of a short launch while the others find none
-      if (!GATHER && qi == 1) asm volatile("griddepcontrol.wait;" ::: "memory");
+      if (!GATHER && qi == 1 && (!P.ready || P.kc_child)) asm volatile("griddepcontrol.wait;" ::: "memory");
     }
     if (!ok && lane == 0) {
       atomicExch(P.err, LX_ERR_TIMEOUT);
@@ -800,6 +807,8 @@ static TcLaunch tc_op(lx_layer* L, int op, const CUtensorMap* xmap, int xcol, vo
   P.gather = nullptr;
   P.xsrc = nullptr;
   P.ldx = 0;
+  P.late = 0;
+  P.ready = 0;
   P.omap = nullptr;
   return P;
 }
@@ -889,12 +898,14 @@ lx_status launch_tc_experts(lx_layer* L, const void* x, int T, int k, void* y, c
     TcLaunch qv = tc_op(L, OP_DN_V, w.xmaps + 1, 0, w.Qal, (long)L->ct_nch * rmax, false, 4);
     qv.row_map = w.rho2al;
     qv.node_col = L->d_child_qcol;
+    qv.late = 1;
     LX_TRY(run(qv, "tc_dn_V"));
     TcLaunch dn = tc_op(L, OP_DN_ANCHOR, w.xmaps + 1, 0, w.yb, H, false, 3);
     dn.kc_child = L->d_child;
     dn.kc_wmaps = L->d_tmaps + (size_t)OP_DN_U * L->N;
     dn.kc_xmap = w.pamap + 2;
     dn.kc_slot = (int)rmax;
+    dn.ready = L->n_corr > 0;  // z was complete before tc_dn_V let this launch start
     dn.omap = w.omaps ? w.omaps + 1 : nullptr;  // yb
     LX_TRY(run(dn, "tc_dn_anchor_U"));
     return launch_combine_tok(L, T, k, y, s);
