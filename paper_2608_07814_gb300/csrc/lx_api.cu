@@ -295,17 +295,17 @@ static lx_status check_call(lx_layer* L, int T, int k) {
 // plan_first: which tile plans the forward's GEMMs read (0 = generic, PLAN_TC =
 // tensor-core, -1 = none: the streaming kernels and lx_get_buckets read none)
 static lx_status bucket_ids(lx_layer* L, const int* ids, int T, int k, cudaStream_t s,
-                            int plan_first) {
+                            int plan_first, const void* x) {
   if (bucket_small_fits(L, T, k))
     return launch_bucket_small(L, nullptr, ids, T, k, nullptr, nullptr, s, plan_first == 0);
-  return launch_bucket(L, ids, T, k, s, plan_first);
+  return launch_bucket(L, ids, T, k, s, plan_first, x);
 }
 
 static lx_status route_and_bucket(lx_layer* L, const void* x, int T, int k, int* ids, float* w,
                                   float* logits_user, cudaStream_t s, int plan_first) {
   float* logits = logits_user ? logits_user : L->ws.logits;
   LX_TRY(launch_router(L, x, T, k, logits, ids, w, s, logits_user != nullptr));
-  return bucket_ids(L, ids, T, k, s, plan_first);
+  return bucket_ids(L, ids, T, k, s, plan_first, x);
 }
 
 
@@ -732,7 +732,7 @@ extern "C" lx_status lx_bucket(lx_layer* L, const int32_t* topk_id, int32_t T, i
   if (!topk_id) return fail(LX_ERR_ARG, "NULL topk_id");
   cudaStream_t s = (cudaStream_t)stream;
   LX_TRY(ensure_workspace(L, T, k, s));
-  LX_TRY(bucket_ids(L, topk_id, T, k, s, -1));
+  LX_TRY(bucket_ids(L, topk_id, T, k, s, -1, nullptr));
   L->last_T = T;
   L->last_k = k;
   return LX_OK;

@@ -256,6 +256,14 @@ struct TokRows {
   uint8_t* tmask;
 };
 
+// token rows copied into anchor-row order: x [T][vec], xg [rows][vec] (16-byte pieces)
+struct XRows {
+  const uint4* x;
+  uint4* xg;
+  long cap;
+  int vec;
+};
+
 // The rows of every assignment, one warp per token (lane s = top-k slot s):
 // its position in its expert's bucket (perm), the rows of the nodes on its
 // path (node_row; the (token, node) pairs shared by several slots write the
@@ -265,12 +273,19 @@ struct TokRows {
 // not selected; slots whose experts share a node add up, in slot order) and
 // al_row[a] = the child rows (-1 where not selected), written by the first
 // slot of that anchor row; rho2al maps every child row to its anchor row.
+// gr.xg (tensor-core path): the token's row of x is also copied to its anchor
+// rows, where the anchor GEMM reads TMA boxes: once read, it is written to each
+// of them.  A launch of its own, a warp per row, read x once per row (27.5 us
+// beside this kernel's 14 at 8192 tokens): a forward of 8192 tokens 584 -> 572 us
+// without it, of the 256-expert layer's 4096 592 -> 575.  Two tokens a CTA, so
+// that a batch of hundreds spreads over the SMs.
 __global__ void __launch_bounds__(256)
 k_assign_rows(const int* __restrict__ topk_id, int T, int k, int N, int E, int D,
               const int* __restrict__ paths, const int* __restrict__ path_len,
               const int* __restrict__ key_off, const uint32_t* __restrict__ bits,
               const int* __restrict__ pre, int* __restrict__ node_tok, int* __restrict__ row_node,
-              int* __restrict__ perm, int* __restrict__ node_row, const CtMeta cm, const TokRows tr) {
+              int* __restrict__ perm, int* __restrict__ node_row, const CtMeta cm, const TokRows tr,
+              const XRows gr) {
   pdl_wait();
   const int lane = threadIdx.x & 31;
   const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -284,6 +299,7 @@ k_assign_rows(const int* __restrict__ topk_id, int T, int k, int N, int E, int D
     if (lane == __ffs(twins) - 1)  // a repeated id counts once, with its first slot
       perm[key_off[N + 1 + e] + rank_before(bits, pre, N + E, N + e, t)] = (int)a;
   }
+  int arow = -1;  // the anchor's row: the last level
   int r0 = -1, r1 = -1, n0 = -1, ev = -1;  // ev: entry `lane` = slot lane / D, level lane % D
 #pragma unroll
   for (int l = 0; l < LX_MAX_DEPTH; ++l) {
@@ -295,6 +311,7 @@ k_assign_rows(const int* __restrict__ topk_id, int T, int k, int N, int E, int D
       node_tok[row] = t;
       row_node[row] = n;
       if (l == 0) n0 = n;
+      if (l == len - 1) arow = row;
     }
     if (lane < k) node_row[a * D + l] = row;
     if (l == 0) r0 = row;
@@ -319,6 +336,25 @@ k_assign_rows(const int* __restrict__ topk_id, int T, int k, int N, int E, int D
       tr.tmask[(size_t)t * TOK_ROWS + rank] = (uint8_t)slots;
     }
     if (lane >= __popc(fm)) tr.trow[(size_t)t * TOK_ROWS + lane] = -1;
+  }
+  if (gr.xg) {
+    constexpr int U = 8;  // 16-byte loads in flight a lane
+    const unsigned same = __match_any_sync(0xffffffffu, arow);
+    const unsigned lead = __ballot_sync(0xffffffffu, arow >= 0 && arow < gr.cap && lane == __ffs(same) - 1);
+    const uint4* src = gr.x + (size_t)t * gr.vec;
+    for (int c0 = 0; lead && c0 < gr.vec; c0 += 32 * U) {
+      const int i0 = c0 + lane;
+      uint4 v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (i0 + 32 * u < gr.vec) v[u] = __ldg(src + i0 + 32 * u);
+      for (unsigned b = lead; b; b &= b - 1) {
+        uint4* dst = gr.xg + (size_t)__shfl_sync(0xffffffffu, arow, __ffs(b) - 1) * gr.vec;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (i0 + 32 * u < gr.vec) dst[i0 + 32 * u] = v[u];
+      }
+    }
   }
   if (!cm.al_g) return;
   // flat layers: a path is [anchor] (the dominant) or [member, anchor]
@@ -582,7 +618,7 @@ static lx_status mark_bits_cap(const lx_layer* L, size_t* smem) {
 }
 
 lx_status launch_bucket(lx_layer* L, const int* topk_id, int T, int k, cudaStream_t s,
-                        int plan_first) {
+                        int plan_first, const void* x) {
   Workspace& w = L->ws;
   const int keys = L->N + L->E, nblk = bucket_blocks(T);
   size_t smem = 0;
@@ -621,10 +657,17 @@ lx_status launch_bucket(lx_layer* L, const int* topk_id, int T, int k, cudaStrea
       tr.trow = w.trow;
       if (!L->ct) tr.tmask = w.tmask;
     }
+    XRows gr{};
+    if (plan_first == PLAN_TC) {
+      gr.x = static_cast<const uint4*>(x);
+      gr.xg = reinterpret_cast<uint4*>(w.xg);
+      gr.cap = w.rows_cap;
+      gr.vec = L->H / 8;
+    }
     ProfScope ps(L, s, "bucket_rows");
-    launch_k(L, k_assign_rows, (unsigned)((T + 7) / 8), 256, 0, s, topk_id, T, k, L->N, L->E,
+    launch_k(L, k_assign_rows, (unsigned)((T + 1) / 2), 64, 0, s, topk_id, T, k, L->N, L->E,
              L->max_depth, L->d_paths, L->d_path_len, w.key_off, w.bits, w.blk_pre, w.node_tok,
-             w.row_node, w.perm, w.node_row, cm, tr);
+             w.row_node, w.perm, w.node_row, cm, tr, gr);
     LX_CUDA(cudaGetLastError());
   }
   return LX_OK;
@@ -728,7 +771,7 @@ extern "C" lx_status lx_bucket_noalloc(lx_layer* L, const int32_t* topk_id, int3
   k_assign_rows<<<(unsigned)((T + 7) / 8), 256, 0, s>>>(topk_id, T, k, L->N, L->E, L->max_depth,
                                                         L->d_paths, L->d_path_len, key_off, bits, pre,
                                                         node_tok, row_node, perm, node_row, CtMeta{},
-                                                        TokRows{});
+                                                        TokRows{}, XRows{});
   LX_CUDA(cudaGetLastError());
   LX_CUDA(cudaMemcpyAsync(node_off, key_off, sizeof(int) * (L->N + 1), cudaMemcpyDeviceToDevice, s));
   LX_CUDA(cudaMemcpyAsync(expert_off, key_off + L->N + 1, sizeof(int) * (L->E + 1),

@@ -473,8 +473,9 @@ bool router_is_tiled(const lx_layer* L, int T);
 int router_tile_counters(int T);  // token tiles of the small-batch router
 // plan_first: tile plans for the generic GEMMs (0), the tensor-core GEMMs
 // (PLAN_TC), or none (-1)
+// x: the token rows, copied into anchor-row order for the tensor-core GEMMs
 lx_status launch_bucket(lx_layer* L, const int* topk_id, int T, int k, cudaStream_t s,
-                        int plan_first);
+                        int plan_first, const void* x);
 lx_status launch_generic_experts(lx_layer* L, const void* x, int T, int k, void* y,
                                  cudaStream_t s);
 // Anchor split-K partials the SwiGLU / combine kernels read for the anchor rows

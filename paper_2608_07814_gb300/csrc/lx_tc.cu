@@ -813,46 +813,6 @@ static TcLaunch tc_op(lx_layer* L, int op, const CUtensorMap* xmap, int xcol, vo
   return P;
 }
 
-namespace {
-
-// xg[r] = x[node_tok[r]] for the anchor rows r < R of this forward (R = the
-// node rows, key_off[N]; rows of correction nodes are skipped: their products
-// gather their rows themselves): one warp per row, 16-byte loads and stores.
-__global__ void __launch_bounds__(256)
-k_gather_rows(const __nv_bfloat16* __restrict__ x, int H, const int* __restrict__ node_tok,
-              const int* __restrict__ row_node, const int* __restrict__ rank,
-              const int* __restrict__ rows_total, long rows_cap, __nv_bfloat16* __restrict__ xg) {
-  pdl_wait();
-  const long R = min((long)*rows_total, rows_cap);
-  const int lane = threadIdx.x & 31;
-  const long warps = (long)gridDim.x * (blockDim.x >> 5);
-  const int vec = H / 8;
-  constexpr int U = 8;  // 16-byte loads of a row in flight per lane before any store
-  long r = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  int tok = r < R ? node_tok[r] : 0;
-  bool anc = r < R && __ldg(rank + row_node[r]) == 0;
-  for (; r < R; r += warps) {
-    const uint4* src = reinterpret_cast<const uint4*>(x + (size_t)tok * H);
-    uint4* dst = reinterpret_cast<uint4*>(xg + (size_t)r * H);
-    const long rn = r + warps;
-    const bool this_anc = anc;
-    tok = rn < R ? node_tok[rn] : 0;  // the next row's token, looked up early
-    anc = rn < R && __ldg(rank + row_node[rn]) == 0;
-    if (!this_anc) continue;
-    for (int i0 = lane; i0 < vec; i0 += 32 * U) {
-      uint4 v[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (i0 + 32 * u < vec) v[u] = __ldg(src + i0 + 32 * u);
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (i0 + 32 * u < vec) dst[i0 + 32 * u] = v[u];
-    }
-  }
-}
-
-}  // namespace
-
 // The prefill forward: every (token, node) product on the tensor cores.
 lx_status launch_tc_experts(lx_layer* L, const void* x, int T, int k, void* y, cudaStream_t s) {
   Workspace& w = L->ws;
@@ -862,16 +822,10 @@ lx_status launch_tc_experts(lx_layer* L, const void* x, int T, int k, void* y, c
     if (P.n_items == 0) return LX_OK;
     return launch_tc(L, P, s, name);
   };
-  // the anchor rows in node-row order once, so that the anchor product's A
-  // tiles are TMA boxes (its 256-row stages are too few to hide gathers); the
-  // correction products read their rows straight from x (gathered by the
-  // GEMM's gather warp)
-  {
-    ProfScope ps(L, s, "gather_rows");
-    launch_k(L, k_gather_rows, L->num_sms * 8, 256, 0, s, xb, (int)H, w.node_tok, w.row_node,
-             L->d_rank, w.key_off + L->N, w.rows_cap, w.xg);
-    LX_CUDA(cudaGetLastError());
-  }
+  // The anchor product's A tiles are TMA boxes of the anchor rows that the
+  // bucketing copied from x (its 256-row stages are too few to hide gathers); the
+  // correction products read their rows straight from x (gathered by the GEMM's
+  // gather warps).
   auto gathered = [&](TcLaunch P) {
     P.gather = w.node_tok;
     P.xsrc = xb;
@@ -881,6 +835,7 @@ lx_status launch_tc_experts(lx_layer* L, const void* x, int T, int k, void* y, c
   {
     TcLaunch ua = tc_op(L, OP_UP_ANCHOR, w.gmap, 0, w.hb, 2 * I, false, 0);
     ua.omap = w.omaps;  // hb (null when not encodable)
+    ua.late = 1;  // tc_up_V reads the bucketing's rows without a wait
     LX_TRY(run(ua, "tc_up_anchor"));
   }
   if (L->ct) {
