@@ -269,6 +269,10 @@ struct TcLaunch {
   // the concatenated children) written and reads them without a wait
   int late;
   int ready;
+  // K blocks before a tile's last at which a CTA claims its next tile, so that the
+  // tiles go to the CTAs that finish first; 0: one tile ahead, for tiles so short
+  // that claiming and decoding the next takes as long
+  int claim;
   // optional TMA map of out (bf16, 32 x 32 boxes, 64-byte swizzle): 256-row
   // tiles store whole 32-row blocks with TMA (row_map null)
   const CUtensorMap* omap;

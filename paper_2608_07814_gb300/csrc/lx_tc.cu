@@ -220,10 +220,12 @@ k_tc_gemm(const __grid_constant__ TcLaunch P) {
       __syncwarp();  // lane 0's acquire orders the scheduler's write before every lane's read
       const TcTile t = qslot[q];
       __syncwarp();
-      if (lane == 0) mbar_arrive(qempty0 + 8 * q);
       ++qi;
       if (t.BN < 0) break;  // no tile left
       const int nkb = (t.K + TC_BK - 1) / TC_BK;
+      // the K block at which the next tile is asked for (-1: at once)
+      const int ask = P.claim ? max(nkb - P.claim, 0) : -1;
+      if (lane == 0 && ask < 0) mbar_arrive(qempty0 + 8 * q);
       const int rt0 = (t.grp * t.Ng + t.row0) / 64;  // first 64-row weight tile
       const int nbox = (t.BN + 63) / 64;
       // K concatenation: k-blocks from kb_own on read child cj's k-block ckb;
@@ -291,6 +293,7 @@ k_tc_gemm(const __grid_constant__ TcLaunch P) {
             }
           }
         }
+        if (lane == 0 && good && kb == ask) mbar_arrive(qempty0 + 8 * q);
         if (kb >= kb_own && ++ckb == cnkb) {  // every lane walks the children alike
           ckb = 0;
           ++cj;
@@ -428,23 +431,30 @@ k_tc_gemm(const __grid_constant__ TcLaunch P) {
     uint32_t qi = 0;
     bool ok = true;
     while (true) {
-      int cur = lane == 0 ? atomicAdd(P.ctr, 1) : 0;
+      // late claims: a tile is claimed only when the producer asks for it;
+      // otherwise it is claimed and decoded before the producer has taken the last
+      const uint32_t q = qi % TC_QN;
+      int good = 1, cur = 0;
+      if (lane == 0) {
+        if (P.claim) good = mbar_wait(qempty0 + 8 * q, ((qi / TC_QN) & 1) ^ 1, abort_flag, P.wait_cycles);
+        if (good) cur = atomicAdd(P.ctr, 1);
+      }
+      if (!__shfl_sync(0xffffffffu, good, 0)) {
+        ok = false;
+        break;
+      }
       cur = __shfl_sync(0xffffffffu, cur, 0);
       TcTile t;
       if (cur < total) tc_decode_warp<BM>(P, cur, t);
       else t.BN = -1;
-      const uint32_t q = qi % TC_QN;
-      int good = 1;
       if (lane == 0) {
-        good = mbar_wait(qempty0 + 8 * q, ((qi / TC_QN) & 1) ^ 1, abort_flag, P.wait_cycles)
-                   ? 1 : 0;
+        if (!P.claim) good = mbar_wait(qempty0 + 8 * q, ((qi / TC_QN) & 1) ^ 1, abort_flag, P.wait_cycles);
         if (good) {
           qslot[q] = t;
           mbar_arrive(qfull0 + 8 * q);
         }
       }
-      good = __shfl_sync(0xffffffffu, good, 0);
-      if (!good) {
+      if (!__shfl_sync(0xffffffffu, good, 0)) {
         ok = false;
         break;
       }
@@ -807,6 +817,12 @@ static TcLaunch tc_op(lx_layer* L, int op, const CUtensorMap* xmap, int xcol, vo
   P.gather = nullptr;
   P.xsrc = nullptr;
   P.ldx = 0;
+  // Late claims from 20 K blocks of 128 rows on (a tile of more than about 6 us;
+  // claiming and decoding the next takes about 3).  With every tile claimed one
+  // ahead, a CTA in a long tile held another that idle SMs could have taken:
+  // forwards of 1031 tokens 218 -> 201 us, 1536 243 -> 226, tree 2048 291 -> 281,
+  // 8192 572 -> 573.  Late claims for the short tiles too: tree 312.
+  P.claim = P.shape.k_const / TC_BK * (P.bm / 128) >= 20 ? 10 : 0;
   P.late = 0;
   P.ready = 0;
   P.omap = nullptr;
