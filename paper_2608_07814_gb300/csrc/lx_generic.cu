@@ -32,17 +32,15 @@ namespace {
 //
 // bf16 weights: mma.sync m16n8k16, the weights as the 16-row operand and the
 // rows as the 8-column one; empty 8-row groups of a ragged tile are skipped.
-// An fp32 activation is split into three bf16 parts (eight significant bits each,
-// together all 24), so every product is exact,
-// and each 64-deep chunk is summed by the tensor core from zero and added to
-// the fp32 sum with an ordinary rounded addition: the tensor core's own
-// accumulation spans 64 products only.
+// An fp32 activation is split into three bf16 parts (eight significant bits
+// each, together all 24), so every product is exact, and each 64-deep chunk is
+// summed by the tensor core from zero and added to the fp32 sum with an ordinary
+// rounded addition: the tensor core's own accumulation spans 64 products only.
 // fp32 weights: fused multiply-adds in ascending K (4 x 4 outputs a thread).
 // Measured on the Qwen3-30B-A3B-shaped layer with rank 32 at 96 tokens, whole
-// forward: 1669 us with a
-// scalar-load, single-buffered form, 195 us with this one (212 before the first
-// tile of a launch was looked up, and its weights requested, ahead of the wait for
-// the preceding one); the tiny fp32 layer
+// forward: 1669 us with a scalar-load, single-buffered form, 195 us with this
+// one (212 before the first tile of a launch was looked up, and its weights
+// requested, ahead of the wait for the preceding one); the tiny fp32 layer
 // (d_model 64, 256 tokens) 74.6 -> 30.6 us.
 // ---------------------------------------------------------------------------
 constexpr int GG_THREADS = 128;
