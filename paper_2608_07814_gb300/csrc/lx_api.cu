@@ -169,7 +169,6 @@ static lx_status ensure_workspace(lx_layer* L, int T, int k, cudaStream_t s) {
       {(void**)&w.blk_pre, sizeof(int) * keys * bucket_blocks(cT)},
       {(void**)&w.key_off, sizeof(int) * (keys + 2)},
       {(void**)&w.node_tok, sizeof(int) * cT * ck * D},
-      {(void**)&w.row_node, sizeof(int) * cT * ck * D},
       {(void**)&w.node_row, sizeof(int) * cT * ck * D},
       {(void**)&w.perm, sizeof(int) * cT * ck},
       {(void**)&w.trow, L->stream_ok ? sizeof(int) * TOK_ROWS * (size_t)cT : 0},

@@ -267,7 +267,7 @@ struct XRows {
 // The rows of every assignment, one warp per token (lane s = top-k slot s):
 // its position in its expert's bucket (perm), the rows of the nodes on its
 // path (node_row; the (token, node) pairs shared by several slots write the
-// same node_tok / row_node values), and, for flat layers on the fused
+// same node_tok values), and, for flat layers on the fused
 // tensor-core path, the per-cluster-row tables: for each anchor row a of the
 // token, al_g[a] = {dominant's gate, gates of child slots 0, 1, ...} (0 where
 // not selected; slots whose experts share a node add up, in slot order) and
@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(256)
 k_assign_rows(const int* __restrict__ topk_id, int T, int k, int N, int E, int D,
               const int* __restrict__ paths, const int* __restrict__ path_len,
               const int* __restrict__ key_off, const uint32_t* __restrict__ bits,
-              const int* __restrict__ pre, int* __restrict__ node_tok, int* __restrict__ row_node,
+              const int* __restrict__ pre, int* __restrict__ node_tok,
               int* __restrict__ perm, int* __restrict__ node_row, const CtMeta cm, const TokRows tr,
               const XRows gr) {
   pdl_wait();
@@ -309,7 +309,6 @@ k_assign_rows(const int* __restrict__ topk_id, int T, int k, int N, int E, int D
       const int n = paths[e * LX_MAX_DEPTH + l];
       row = key_off[n] + rank_before(bits, pre, N + E, n, t);
       node_tok[row] = t;
-      row_node[row] = n;
       if (l == 0) n0 = n;
       if (l == len - 1) arow = row;
     }
@@ -432,7 +431,7 @@ k_bucket_small(const float* __restrict__ logits, const int* __restrict__ ids_in,
                int E, int N, int D, const int* __restrict__ paths,
                const int* __restrict__ path_len, const int* __restrict__ rank,
                int* __restrict__ topk_id, float* __restrict__ topk_w, int* __restrict__ key_off_g,
-               int* __restrict__ node_tok, int* __restrict__ row_node, int* __restrict__ node_row,
+               int* __restrict__ node_tok, int* __restrict__ node_row,
                int* __restrict__ perm, int* __restrict__ tile_off, int max_items, PlanArgs pa,
                const int* __restrict__ anchors, int n_anchor, const int* __restrict__ corrs,
                int n_corr, int blk, int* __restrict__ act, int* __restrict__ act_n,
@@ -539,7 +538,6 @@ k_bucket_small(const float* __restrict__ logits, const int* __restrict__ ids_in,
         const int n = spaths[e * LX_MAX_DEPTH + l];
         row = off[n] + rank_of(n, t);
         node_tok[row] = t;   // (t, n) pairs shared by several slots write the same values
-        row_node[row] = n;
       }
       node_row[(size_t)a * D + l] = row;
     }
@@ -599,7 +597,7 @@ lx_status launch_bucket_small(lx_layer* L, const float* logits, const int* ids_i
   ProfScope ps(L, s, logits ? "topk_bucket_small" : "bucket_small");
   launch_k(L, k_bucket_small, 1, SB_THREADS, smem, s, logits, ids_in, T, k, L->E, L->N, L->max_depth,
                                              L->d_paths, L->d_path_len, L->d_rank, topk_id, topk_w,
-                                             w.key_off, w.node_tok, w.row_node, w.node_row, w.perm,
+                                             w.key_off, w.node_tok, w.node_row, w.perm,
                                              w.tile_off, op_max_items(L), pa, L->d_anchors,
                                              L->n_anchor, L->d_corrs, L->n_corr,
                                              stream_item_rows(T), w.act, w.act_n, w.sctr,
@@ -667,7 +665,7 @@ lx_status launch_bucket(lx_layer* L, const int* topk_id, int T, int k, cudaStrea
     ProfScope ps(L, s, "bucket_rows");
     launch_k(L, k_assign_rows, (unsigned)((T + 1) / 2), 64, 0, s, topk_id, T, k, L->N, L->E,
              L->max_depth, L->d_paths, L->d_path_len, w.key_off, w.bits, w.blk_pre, w.node_tok,
-             w.row_node, w.perm, w.node_row, cm, tr, gr);
+             w.perm, w.node_row, cm, tr, gr);
     LX_CUDA(cudaGetLastError());
   }
   return LX_OK;
@@ -754,8 +752,7 @@ extern "C" lx_status lx_bucket_noalloc(lx_layer* L, const int32_t* topk_id, int3
   int* cnt = reinterpret_cast<int*>(p += round256(sizeof(uint32_t) * BK_WORDS * (size_t)keys * nblk));
   int* pre = reinterpret_cast<int*>(p += round256(sizeof(int) * (size_t)keys * nblk));
   int* key_off = reinterpret_cast<int*>(p += round256(sizeof(int) * (size_t)keys * nblk));
-  int* row_node = reinterpret_cast<int*>(p += b_off);
-  const size_t used = (size_t)(p - static_cast<char*>(base)) + b_rown;
+  const size_t used = (size_t)(p - static_cast<char*>(base)) + b_off;
   if (used > (size_t)LX_NOALLOC_SCRATCH_BYTES)
     return fail(LX_ERR_SHAPE, "lx_bucket_noalloc: scratch layout exceeds the fixed array");
 
@@ -770,7 +767,7 @@ extern "C" lx_status lx_bucket_noalloc(lx_layer* L, const int32_t* topk_id, int3
   LX_CUDA(cudaGetLastError());
   k_assign_rows<<<(unsigned)((T + 7) / 8), 256, 0, s>>>(topk_id, T, k, L->N, L->E, L->max_depth,
                                                         L->d_paths, L->d_path_len, key_off, bits, pre,
-                                                        node_tok, row_node, perm, node_row, CtMeta{},
+                                                        node_tok, perm, node_row, CtMeta{},
                                                         TokRows{}, XRows{});
   LX_CUDA(cudaGetLastError());
   LX_CUDA(cudaMemcpyAsync(node_off, key_off, sizeof(int) * (L->N + 1), cudaMemcpyDeviceToDevice, s));

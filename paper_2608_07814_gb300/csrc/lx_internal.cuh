@@ -301,7 +301,6 @@ struct Workspace {
   int* blk_pre = nullptr;    // [token blocks][N+E] the number in earlier blocks
   int* key_off = nullptr;    // [N+1 + E+1]: node_off then expert_off
   int* node_tok = nullptr;   // [T*k*D]
-  int* row_node = nullptr;   // [T*k*D]
   int* node_row = nullptr;   // [T*k*D]
   int* perm = nullptr;       // [T*k]
   int* trow = nullptr;       // [T][TOK_ROWS] a token's distinct rows (tensor-core path)
