@@ -399,10 +399,14 @@ LX_API lx_status lx_permute_neurons(int32_t dtype, int32_t d_model, int32_t d_ff
  * Solver: Y = R Omega, Q = orth(Y); power_iters times Q = orth(R orth(R^T Q));
  * then the SVD of Bs = Q^T R: Z = R^T Q is orthonormalised too, Z = Z2 M^T with
  * M the l x l triangular factor, and the small SVD of M (one-sided Jacobi)
- * gives Bs's.  orth is CholeskyQR run twice (float64 Gram sums, fp32 Cholesky;
- * the first pass is shifted by 1e-6 of the largest Gram diagonal); the
- * products with R are fp32 (CUDA cores); singular values are float64 Rayleigh
- * quotients.  The sign of each factor column is fixed so that the
+ * gives Bs's.  orth is CholeskyQR (the Gram summed in compensated fp32 pairs to
+ * float64 accuracy, fp32 Cholesky and inverse; the first pass is shifted by
+ * 1e-6 of the largest Gram diagonal), run twice for the final Q and Z and once
+ * for the bases in between; the products with R accumulate in fp32 (bf16
+ * weights: on the tensor cores, X split exactly into three bf16 parts); the
+ * Jacobi is fp32 and rotates every pair of columns further than 1e-6 from
+ * orthogonal until a sweep rotates none (30 sweeps at most); M and the
+ * singular values (Rayleigh quotients) are summed in float64.  The sign of each factor column is fixed so that the
  * largest-magnitude entry of U's column is positive.  Singular values at or
  * below 1e-6 of the largest give zero U and V columns.  The call is latency
  * bound (one-CTA stages): independent projections run concurrently when given

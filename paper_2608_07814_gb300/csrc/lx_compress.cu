@@ -11,25 +11,27 @@
 //               formed on load; fp32 weights), R^T (columns of the same), or an
 //               fp32 matrix (the bases times the small factors).
 //   k_gram      G = X^T X to float64 accuracy (exact fp32 products, error-free
-//               two-sum accumulation on the fp32 pipes), stored in float64.
+//               two-sum accumulation on the fp32 pipes), stored as the unevaluated
+//               fp32 pairs of four interleaved row sets.
 //   k_chol32    one CTA: Cholesky G + s I = L L^T (fp32 in shared memory,
 //               blocked by 16 columns; a small relative shift in the first
 //               pass keeps rank-deficient bases factorable).
-//   k_trsm      X L^-T by blocked substitution, so that its columns are
-//               orthonormal (CholeskyQR).
-//   k_trmm      M = L1 L2, the triangular factor of R^T Q = Z2 M^T.
+//   k_tri_inverse
+//               L^-T, a CTA per 16 columns of the inverse; X L^-T then has
+//               orthonormal columns (CholeskyQR).
+//   k_trmm      M = L1 L2 (float64 sums), the triangular factor of R^T Q = Z2 M^T.
 //   k_jacobi_cluster
 //               one-sided Jacobi SVD of M, M W = U S, over a thread-block
-//               cluster (fp32 rotations, column blocks exchanged through
-//               distributed shared memory).
+//               cluster (fp32 rotations, columns handed on through distributed
+//               shared memory).
 //   k_ritz      sigma_j = |M w_j| / |w_j| in float64 (Rayleigh quotients).
 //   k_finish    the r largest sigma and the fp32 matrices that turn the bases
 //               into the split factors.
 //   k_sign      each factor column's largest-magnitude entry of U made
 //               positive (U and V negated together).
-// The Gram sums, M and the Rayleigh quotients reach float64 accuracy by
-// compensated fp32 arithmetic: this GPU's float64 rate is a small fraction of
-// its fp32 rate.
+// The Gram sums reach float64 accuracy by compensated fp32 arithmetic (this
+// GPU's float64 rate is a small fraction of its fp32 rate); M and the Rayleigh
+// quotients are summed in float64.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -151,36 +153,20 @@ k_cgemm(const TW* __restrict__ Wm, const TW* __restrict__ Wd, const float* __res
 // Rump and Oishi, 2005), so G = hi + lo is as accurate as a dot product in
 // twice the fp32 precision: within 2^-24 |G| + (n 2^-24)^2 sum |x y| of the
 // exact sum, far below the fp32 rounding the Cholesky applies to it.  Four
-// such pairs per thread take the rows of a chunk in turn (independent chains)
-// and are added pairwise at the end; each 64-row chunk is staged in shared
-// memory while the next one is already loading into registers.  16 x 16
-// outputs per CTA; only the tiles on or below the diagonal are computed (the
-// Cholesky reads the lower triangle alone).  The triangle's tiles alone (45 at
-// L = 136) leave most SMs idle and each runs n serial steps, so the rows are
-// cut into up to GR_SPLITS ranges (blockIdx.z) of 256 or more, whose pairs the
-// Cholesky adds in order: 26.9 -> 19.1 us a launch at L = 136 (n = 768 and 2048).
-// The issue rate bounds it, so the ranges are counted by the rows of the SM with
-// the most CTAs (gram_parts): n = 2048 takes 3 (135 CTAs, one an SM, 683 rows
-// each) before 4 (180 CTAs, two on some SMs): 28.0 -> 24.4 us.
-constexpr int GR_SPLITS = 4;
+// such pairs (independent chains) take the rows in turn
+// (rows 4 t + c are chain c's) and are added pairwise at the end.  A CTA takes
+// 16 x 16 outputs and one of the chains (blockIdx.z), so that the tiles on or
+// below the diagonal (45 at L = 136; the Cholesky reads the lower triangle
+// alone) make 180 CTAs, and the Cholesky adds the chains in the same order as
+// one thread with all four would: 26.9 us a launch with one, 20.1 so (L = 136,
+// mean over n = 768 and 2048).  The issue rate bounds it.  Ranges of
+// consecutive rows in place of the chains cost the same and round differently.
+// Each chunk of 64 chain rows is staged in shared memory while the next one is
+// already loading into registers.
 constexpr int GR_T = 16;
 constexpr int GR_KC = 64;
 constexpr int GR_CH = 4;
 static_assert(GR_KC * GR_T % (GR_T * GR_T) == 0, "whole staged values per thread");
-
-// row ranges of a Gram of n rows and L columns
-static int gram_parts(int n, int L, int sms) {
-  const int t = (L + GR_T - 1) / GR_T, tiles = t * (t + 1) / 2;
-  int best = 1, cost = 0x7fffffff;
-  for (int p = 1; p <= std::min(GR_SPLITS, std::max(1, n / 256)); ++p) {
-    const int c = (tiles * p + sms - 1) / sms * ((n + p - 1) / p);
-    if (c < cost) {
-      cost = c;
-      best = p;
-    }
-  }
-  return best;
-}
 
 struct DF {
   float hi, lo;
@@ -196,31 +182,30 @@ __device__ __forceinline__ void df_add(DF& d, float p, float e) {
 }
 
 __global__ void __launch_bounds__(GR_T * GR_T)
-k_gram(const float* __restrict__ X, int n_all, int L, int span, float2* __restrict__ Gp) {
+k_gram(const float* __restrict__ X, int n, int L, float2* __restrict__ Gp) {
   constexpr int PER = GR_KC * GR_T / (GR_T * GR_T);  // staged values per thread and side
   __shared__ float Xi[GR_KC][GR_T], Xj[GR_KC][GR_T];
   if (blockIdx.x > blockIdx.y) return;  // strictly above the diagonal
-  const int n_lo = blockIdx.z * span, n = min(n_all, n_lo + span);
-  float2* G = Gp + (size_t)blockIdx.z * L * L;
+  const int z = blockIdx.z;
+  const int nz = n > z ? (n - z + GR_CH - 1) / GR_CH : 0;  // rows of this chain
+  float2* G = Gp + (size_t)z * L * L;
   const int ti = threadIdx.x / GR_T, tj = threadIdx.x % GR_T;
   const int i0 = blockIdx.y * GR_T, j0 = blockIdx.x * GR_T;
-  DF acc[GR_CH];
-#pragma unroll
-  for (int c = 0; c < GR_CH; ++c) acc[c] = DF{0.f, 0.f};
+  DF acc{0.f, 0.f};
   // the next chunk's rows are loaded into registers while this one is summed
   float ri[PER], rj[PER];
   auto fetch = [&](int m0) {
 #pragma unroll
     for (int e = 0; e < PER; ++e) {
       const int q = threadIdx.x + e * GR_T * GR_T;
-      const int mr = q / GR_T, c = q % GR_T;
-      const bool okm = m0 + mr < n;
-      ri[e] = (okm && i0 + c < L) ? X[(size_t)(m0 + mr) * L + i0 + c] : 0.f;
-      rj[e] = (okm && j0 + c < L) ? X[(size_t)(m0 + mr) * L + j0 + c] : 0.f;
+      const int mr = m0 + q / GR_T, c = q % GR_T;
+      const size_t at = ((size_t)GR_CH * mr + z) * L;
+      ri[e] = (mr < nz && i0 + c < L) ? X[at + i0 + c] : 0.f;
+      rj[e] = (mr < nz && j0 + c < L) ? X[at + j0 + c] : 0.f;
     }
   };
-  fetch(n_lo);
-  for (int m0 = n_lo; m0 < n; m0 += GR_KC) {
+  fetch(0);
+  for (int m0 = 0; m0 < nz; m0 += GR_KC) {
 #pragma unroll
     for (int e = 0; e < PER; ++e) {
       const int q = threadIdx.x + e * GR_T * GR_T;
@@ -228,29 +213,31 @@ k_gram(const float* __restrict__ X, int n_all, int L, int span, float2* __restri
       Xj[q / GR_T][q % GR_T] = rj[e];
     }
     __syncthreads();
-    if (m0 + GR_KC < n) fetch(m0 + GR_KC);
-#pragma unroll
-    for (int mr = 0; mr < GR_KC; mr += GR_CH) {
-#pragma unroll
-      for (int c = 0; c < GR_CH; ++c) {
-        const float x = Xi[mr + c][ti], y = Xj[mr + c][tj];
-        const float p = __fmul_rn(x, y);
-        df_add(acc[c], p, __fmaf_rn(x, y, -p));
-      }
+    if (m0 + GR_KC < nz) fetch(m0 + GR_KC);
+#pragma unroll 16
+    for (int mr = 0; mr < GR_KC; ++mr) {
+      const float x = Xi[mr][ti], y = Xj[mr][tj];
+      const float p = __fmul_rn(x, y);
+      df_add(acc, p, __fmaf_rn(x, y, -p));
     }
     __syncthreads();
   }
-  // (chain 0 + chain 1) + (chain 2 + chain 3), each pair added as hi + lo
-  DF s01 = acc[0], s23 = acc[2];
-  df_add(s01, acc[1].hi, acc[1].lo);
-  df_add(s23, acc[3].hi, acc[3].lo);
-  df_add(s01, s23.hi, s23.lo);
-  if (i0 + ti < L && j0 + tj < L)
-    G[(size_t)(i0 + ti) * L + j0 + tj] = make_float2(s01.hi, s01.lo);
+  if (i0 + ti < L && j0 + tj < L) G[(size_t)(i0 + ti) * L + j0 + tj] = make_float2(acc.hi, acc.lo);
 }
 
-// One CTA (L <= 256).  Cholesky of G + s I in fp32 (the row ranges' pairs of G
-// added in order and rounded once; s = shift_rel * max diag(G)) in a
+// (chain 0 + chain 1) + (chain 2 + chain 3) of a Gram entry, each pair added as
+// hi + lo
+__device__ __forceinline__ DF gram_sum(const float2 (&g)[GR_CH]) {
+  DF s01{g[0].x, g[0].y}, s23{g[2].x, g[2].y};
+  df_add(s01, g[1].x, g[1].y);
+  df_add(s23, g[3].x, g[3].y);
+  df_add(s01, s23.hi, s23.lo);
+  return s01;
+}
+static_assert(GR_CH == 4, "gram_sum adds four chains");
+
+// One CTA (L <= 256).  Cholesky of G + s I in fp32 (the chains of G added in
+// order and rounded once; s = shift_rel * max diag(G)) in a
 // packed lower triangle in shared memory (L (L + 1) / 2 floats, row i from
 // i (i + 1) / 2), pivots floored at 1e-30, blocked by 16 columns (right-looking).
 // One SM's latency bounds it, so each part keeps its chain in registers: warp 0
@@ -259,22 +246,24 @@ k_gram(const float* __restrict__ X, int n_all, int L, int span, float2* __restri
 // (vector loads of a transposed copy), and the trailing triangle takes the
 // panel's rank-16 update with a warp on four rows, lanes along the columns.
 // The factor goes to Lout [L][L] (zero above the diagonal) and the inverses of
-// its 16 x 16 diagonal blocks to Dinv [blocks][16][16], which is all that the
-// solve below needs.  A zero Gram gives Lout = Dinv = 0.  Measured at L = 136:
-// 152 us with in-place shared-memory steps and the whole inverse formed here,
-// 42 us now.
+// its 16 x 16 diagonal blocks to Dinv [blocks][16][16], from which the kernel
+// below forms the rest of the inverse.  A zero Gram gives Lout = Dinv = 0.  The
+// roots and reciprocals are the correctly rounded ones: a Newton step on the
+// fast reciprocal root shortens the diagonal's chain by 6 us at the cost of up to
+// an ulp.  Measured at L = 136: 152 us with in-place shared-memory steps and
+// the whole inverse formed here, 47 us now.
 constexpr int CH_THREADS = 512;  // 16 warps: at most 16 diagonal blocks
 constexpr int CH_B = 16;  // block width
 __device__ __forceinline__ int tri_off(int i) { return i * (i + 1) / 2; }
 inline int ch_ldp(int L) { return (L + 127) / 128 * 128; }  // panel copy: whole column chunks
 
 __global__ void __launch_bounds__(CH_THREADS, 1)
-k_chol32(const float2* __restrict__ Gp, int parts, int L, int ldp, float shift_rel,
-         float* __restrict__ Lout, float* __restrict__ Dinv) {
+k_chol32(const float2* __restrict__ Gp, int L, int ldp, float shift_rel, float* __restrict__ Lout,
+         float* __restrict__ Dinv) {
   extern __shared__ __align__(16) float Ls[];
   float* Pt = Ls + ((tri_off(L) + 3) & ~3);          // [CH_B][ldp] panel, transposed
   __shared__ __align__(16) float sD[2][CH_B][CH_B];  // by block parity: sD[c][i] = l_ic of the diagonal block
-  __shared__ float s_md;
+  __shared__ double s_md;
   __shared__ float s_rdiag[256];  // reciprocals of the factor's diagonal
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = CH_THREADS / 32;
   const int nb = (L + CH_B - 1) / CH_B;
@@ -283,7 +272,7 @@ k_chol32(const float2* __restrict__ Gp, int parts, int L, int ldp, float shift_r
   const int nfold = (L + 1) / 2 * (L + 1);
   constexpr int U = 5;
   for (int e0 = tid; e0 < nfold; e0 += U * CH_THREADS) {
-    float2 g[U][GR_SPLITS];
+    float2 g[U][GR_CH];
     int at[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -293,33 +282,38 @@ k_chol32(const float2* __restrict__ Gp, int parts, int L, int ldp, float shift_r
       const bool ok = e < nfold && (low || 2 * q != L - 1);  // (an odd L's middle row once)
       at[u] = ok ? tri_off(i) + c : -1;
 #pragma unroll
-      for (int z = 0; z < GR_SPLITS; ++z)
-        g[u][z] = ok && z < parts ? Gp[(size_t)z * L * L + i * L + c] : make_float2(0.f, 0.f);
+      for (int z = 0; z < GR_CH; ++z)
+        g[u][z] = ok ? Gp[(size_t)z * L * L + i * L + c] : make_float2(0.f, 0.f);
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      DF t{g[u][0].x, g[u][0].y};
-#pragma unroll
-      for (int z = 1; z < GR_SPLITS; ++z) df_add(t, g[u][z].x, g[u][z].y);
+      // (hi + lo rounded to fp32 at once and by way of float64 is the same: near
+      // a midpoint of two fp32 values the float64 sum is exact)
+      const DF t = gram_sum(g[u]);
       if (at[u] >= 0) Ls[at[u]] = __fadd_rn(t.hi, t.lo);
     }
   }
-  __syncthreads();
-  if (warp == 0) {
-    float md = 0.f;
-    for (int i = lane; i < L; i += 32) md = fmaxf(md, Ls[tri_off(i) + i]);
+  if (warp == 0) {  // the largest diagonal entry
+    double md = 0.0;
+    for (int i = lane; i < L; i += 32) {
+      float2 g[GR_CH];
 #pragma unroll
-    for (int o = 16; o; o >>= 1) md = fmaxf(md, __shfl_xor_sync(0xffffffffu, md, o));
+      for (int z = 0; z < GR_CH; ++z) g[z] = Gp[(size_t)z * L * L + (size_t)i * L + i];
+      const DF t = gram_sum(g);
+      md = fmax(md, (double)t.hi + (double)t.lo);
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) md = fmax(md, __shfl_xor_sync(0xffffffffu, md, o));
     if (lane == 0) s_md = md;
   }
   __syncthreads();
-  const float md = s_md;
-  if (!(md > 0.f)) {
+  const double md = s_md;
+  if (!(md > 0.0)) {
     for (int e = tid; e < L * L; e += CH_THREADS) Lout[e] = 0.f;
     for (int e = tid; e < nb * CH_B * CH_B; e += CH_THREADS) Dinv[e] = 0.f;
     return;
   }
-  const float shift = (float)((double)shift_rel * (double)md);
+  const float shift = (float)(shift_rel * md);
   for (int i = tid; i < L; i += CH_THREADS) Ls[tri_off(i) + i] += shift;  // (float) g_ii + shift
   __syncthreads();
   // ---- factorization.  Warp 0 factors the diagonal block; while the other
@@ -331,11 +325,7 @@ k_chol32(const float2* __restrict__ Gp, int parts, int L, int ldp, float shift_r
     float(*D)[CH_B] = sD[kb & 1];
 #pragma unroll
     for (int j = 0; j < CH_B; ++j) {
-      // rd = 1 / sqrt(p), d = sqrt(p): the fast reciprocal root and a Newton
-      // step each (the IEEE root and division double this chain's latency)
-      const float p = fmaxf(__shfl_sync(0xffffffffu, a[j], j), 1e-30f);
-      const float r0 = rsqrtf(p), rd = fmaf(r0, fmaf(-0.5f * p * r0, r0, 0.5f), r0);
-      const float d0 = p * rd, d = fmaf(fmaf(-d0, d0, p), 0.5f * rd, d0);
+      const float d = sqrtf(fmaxf(__shfl_sync(0xffffffffu, a[j], j), 1e-30f)), rd = 1.f / d;
       const float l = lane == j ? d : lane > j ? a[j] * rd : 0.f;
       a[j] = l;
       if (lane == 0 && j < bw) s_rdiag[j0 + j] = rd;
@@ -484,157 +474,160 @@ __device__ __forceinline__ uint32_t os_smem(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// Y = X L^-T for X [n][l] fp32 (the second half of a CholeskyQR pass): row by
-// row, block column k of Y is (X_k - sum_{j < k} Y_j L_kj^T) Dinv_k^T, so the
-// factor's inverse is never formed and half of the products of a full GEMM are
-// left out.  One CTA takes TS_ROWS rows against the whole factor in shared
-// memory (block rows of 16, each as long as it is, four words of padding so
-// that eight rows read at once fall on distinct banks); thread (row, c) owns
-// column c of a block.  Instruction latency of its few warps bounds it: at
-// l = 136 16.8 us with two columns a thread and copies of 4 bytes, 9.7 so (the
-// GEMM with the formed inverse took 13, but forming it 80 of the Cholesky's 152).
-constexpr int TS_ROWS = 16;
-constexpr int TS_THREADS = CH_B * TS_ROWS;
-__host__ __device__ inline int ts_off(int kb) { return CH_B * (8 * kb * (kb + 1) + 4 * kb); }
-__host__ __device__ inline int ts_ldy(int nb) { return nb * CH_B + 4; }
+// T = L^-T (T[k][n] = X[n][k], X = L^-1) from the factor and its inverted
+// diagonal blocks.  CTA kb forms the 16 columns of X from 16 kb on, block row by
+// block row: S = sum of L_{ib,m} X_m over the earlier rows (ascending), X_ib =
+// -Dinv_ib S; a thread holds one of the 16 x 16 sums.  The block columns do not
+// depend on one another, so the inverse takes nb CTAs instead of more of the
+// Cholesky's one (where it took 80 us at L = 136); the chain of nb block rows of
+// the first bounds it: 10.9 us.  The next block row of L is on its way meanwhile.
+constexpr int TI_THREADS = CH_B * CH_B;
+__host__ __device__ inline int ti_ld(int nb) { return nb * CH_B + 4; }
 
-__global__ void __launch_bounds__(TS_THREADS)
-k_trsm(const float* __restrict__ X, const float* __restrict__ Lf, const float* __restrict__ Dinv,
-       int n, int L, int vec, float* __restrict__ Y) {
-  extern __shared__ __align__(16) float ts[];
-  const int nb = (L + CH_B - 1) / CH_B, ldy = ts_ldy(nb);
-  float* Lb = ts;                       // block row kb at ts_off(kb), rows of 16 (kb + 1) + 4
-  float* Ys = ts + ts_off(nb);          // [TS_ROWS][ldy]
-  float* Ss = Ys + TS_ROWS * ldy;       // [TS_ROWS][CH_B + 4]
-  float* Ds = Ss + TS_ROWS * (CH_B + 4);  // [nb][CH_B][CH_B + 4]
-  const int tid = threadIdx.x, row0 = blockIdx.x * TS_ROWS;
-  // every copy in flight at once: 16 bytes each where the rows allow it
-  auto cp4 = [](float* dst, const float* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(os_smem(dst)), "l"(src) : "memory");
-  };
-  auto cp16 = [](float* dst, const float* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(os_smem(dst)), "l"(src) : "memory");
-  };
-  if (L % 4 == 0 && vec) {
-    for (int r = tid >> 4; r < L; r += TS_THREADS / 16) {
-      const int kb = r / CH_B, ld = CH_B * (kb + 1) + 4;
-      float* dst = Lb + ts_off(kb) + (r - kb * CH_B) * ld;
-      for (int c = 4 * (tid & 15); c < CH_B * kb; c += 64) cp16(dst + c, Lf + (size_t)r * L + c);
-    }
-    for (int r = tid >> 4; r < TS_ROWS; r += TS_THREADS / 16)
-      for (int c = 4 * (tid & 15); c < nb * CH_B; c += 64) {
-        if (row0 + r < n && c < L) cp16(Ys + r * ldy + c, X + (size_t)(row0 + r) * L + c);
-        else *reinterpret_cast<float4*>(Ys + r * ldy + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+__global__ void __launch_bounds__(TI_THREADS)
+k_tri_inverse(const float* __restrict__ Lf, const float* __restrict__ Dinv, int L, float* __restrict__ T) {
+  extern __shared__ __align__(16) float ti[];
+  const int nb = (L + CH_B - 1) / CH_B, ld = ti_ld(nb);
+  float* X = ti;                        // [rows from j0 on][CH_B]
+  float* Lr = X + nb * CH_B * CH_B;     // [2][CH_B][ld]: block rows of L, columns from j0 on
+  float* Dr = Lr + 2 * CH_B * ld;       // [2][CH_B][CH_B + 4]: their inverted diagonal blocks
+  float* S = Dr + 2 * CH_B * (CH_B + 4);  // [CH_B][CH_B]
+  const int tid = threadIdx.x, rr = tid / CH_B, cc = tid % CH_B;
+  const int kb = blockIdx.x, j0 = kb * CH_B;
+  auto fetch = [&](int ib) {
+    if (ib < nb) {
+      const int i0 = ib * CH_B, w = i0 - j0;
+      float* dst = Lr + (ib & 1) * CH_B * ld;
+      if (L % 4 == 0) {
+        for (int q = tid; q < CH_B * w / 4; q += TI_THREADS) {
+          const int r = q / (w / 4), c = 4 * (q - r * (w / 4));
+          if (i0 + r < L)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(os_smem(dst + r * ld + c)),
+                         "l"(Lf + (size_t)(i0 + r) * L + j0 + c)
+                         : "memory");
+        }
+      } else {
+        for (int q = tid; q < CH_B * w; q += TI_THREADS) {
+          const int r = q / w, c = q - r * w;
+          if (i0 + r < L)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(os_smem(dst + r * ld + c)),
+                         "l"(Lf + (size_t)(i0 + r) * L + j0 + c)
+                         : "memory");
+        }
       }
-  } else {
-    for (int r = tid >> 5; r < L; r += TS_THREADS / 32) {
-      const int kb = r / CH_B, ld = CH_B * (kb + 1) + 4;
-      float* dst = Lb + ts_off(kb) + (r - kb * CH_B) * ld;
-      for (int c = tid & 31; c < CH_B * kb; c += 32) cp4(dst + c, Lf + (size_t)r * L + c);
-    }
-    for (int r = tid >> 5; r < TS_ROWS; r += TS_THREADS / 32)
-      for (int c = tid & 31; c < nb * CH_B; c += 32) {
-        if (row0 + r < n && c < L) cp4(Ys + r * ldy + c, X + (size_t)(row0 + r) * L + c);
-        else Ys[r * ldy + c] = 0.f;
+      if (tid < CH_B * CH_B / 4) {
+        const int r = tid / (CH_B / 4), c = 4 * (tid % (CH_B / 4));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                         os_smem(Dr + (ib & 1) * CH_B * (CH_B + 4) + r * (CH_B + 4) + c)),
+                     "l"(Dinv + (i0 + r) * CH_B + c)
+                     : "memory");
       }
-  }
-  for (int e = 4 * tid; e < nb * CH_B * CH_B; e += 4 * TS_THREADS)
-    cp16(Ds + (e / CH_B) * (CH_B + 4) + e % CH_B, Dinv + e);
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  __syncthreads();
-  const int c = tid % CH_B, r = tid / CH_B;
-  float* yr = Ys + r * ldy;
-  float* sr = Ss + r * (CH_B + 4);
-  for (int kb = 0; kb < nb; ++kb) {
-    const int j0 = kb * CH_B, ld = CH_B * (kb + 1) + 4;
-    const float* l0 = Lb + ts_off(kb) + c * ld;
-    float s0[4] = {};
-    if (j0 + c < L) {  // a factor row that exists
+    }
+  };
+  fetch(kb + 1);
+  X[rr * CH_B + cc] = Dinv[(j0 + rr) * CH_B + cc];
+  for (int ib = kb + 1; ib < nb; ++ib) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();  // block row ib has landed; the last one's buffers are free
+    fetch(ib + 1);
+    const int i0 = ib * CH_B;
+    const float* l = Lr + (ib & 1) * CH_B * ld + rr * ld;
+    float acc = 0.f;
+    if (i0 + rr < L) {
 #pragma unroll 4
-      for (int j = 0; j < j0; j += 4) {
-        const float4 y = *reinterpret_cast<const float4*>(yr + j);
-        const float4 a = *reinterpret_cast<const float4*>(l0 + j);
-        s0[0] = fmaf(y.x, a.x, s0[0]);
-        s0[1] = fmaf(y.y, a.y, s0[1]);
-        s0[2] = fmaf(y.z, a.z, s0[2]);
-        s0[3] = fmaf(y.w, a.w, s0[3]);
+      for (int q = 0; q < i0 - j0; q += 4) {
+        const float4 a = *reinterpret_cast<const float4*>(l + q);
+        const float* x = X + q * CH_B + cc;
+        acc = fmaf(a.x, x[0], acc);
+        acc = fmaf(a.y, x[CH_B], acc);
+        acc = fmaf(a.z, x[2 * CH_B], acc);
+        acc = fmaf(a.w, x[3 * CH_B], acc);
       }
     }
-    sr[c] = yr[j0 + c] - ((s0[0] + s0[1]) + (s0[2] + s0[3]));
-    __syncwarp();  // a row's sixteen threads are in one warp
-    const float* d0 = Ds + (j0 + c) * (CH_B + 4);
-    float t0 = 0.f;
+    S[rr * CH_B + cc] = acc;
+    __syncthreads();
+    const float* d = Dr + (ib & 1) * CH_B * (CH_B + 4) + rr * (CH_B + 4);
+    acc = 0.f;
 #pragma unroll
     for (int p = 0; p < CH_B; p += 4) {
-      const float4 s = *reinterpret_cast<const float4*>(sr + p);
-      const float4 a = *reinterpret_cast<const float4*>(d0 + p);
-      t0 = fmaf(s.w, a.w, fmaf(s.z, a.z, fmaf(s.y, a.y, fmaf(s.x, a.x, t0))));
+      const float4 a = *reinterpret_cast<const float4*>(d + p);
+      acc = fmaf(a.x, S[p * CH_B + cc], acc);
+      acc = fmaf(a.y, S[(p + 1) * CH_B + cc], acc);
+      acc = fmaf(a.z, S[(p + 2) * CH_B + cc], acc);
+      acc = fmaf(a.w, S[(p + 3) * CH_B + cc], acc);
     }
-    yr[j0 + c] = t0;
-    __syncwarp();
+    X[(i0 - j0 + rr) * CH_B + cc] = -acc;
   }
   __syncthreads();
-  for (int q = tid >> 5; q < TS_ROWS; q += TS_THREADS / 32)
-    for (int cc = tid & 31; cc < L; cc += 32)
-      if (row0 + q < n) Y[(size_t)(row0 + q) * L + cc] = Ys[q * ldy + cc];
+  for (int k = tid >> 5; k < CH_B && j0 + k < L; k += TI_THREADS / 32)
+    for (int n = tid & 31; n < L; n += 32)
+      T[(size_t)(j0 + k) * L + n] = n >= j0 + k ? X[(n - j0) * CH_B + k] : 0.f;
 }
 
 // Mt (column-major, Mt[j][i] = M[i][j]) of M = L1 L2 for lower-triangular
-// L1, L2 [L][L] (fp32, sums to float64 accuracy).  CTA i, thread j.
-__global__ void k_trmm(const float* __restrict__ L1, const float* __restrict__ L2, int L,
-                       float* __restrict__ Mt) {
+// L1, L2 [L][L] (fp32, float64 sums).  CTA i, thread j.  The float64 pipe bounds
+// it (a multiply-add and a widening, 16 cycles a warp each: row i of L1 is widened
+// once).  Thirty-two loads are in flight, and a warp's lanes walk the same k from
+// its first column on, so that a load reads one row piece: 29 us at
+// L = 136 (8 with compensated fp32 pairs, which hold 48 bits of the sum).
+__global__ void __launch_bounds__(256)
+k_trmm(const float* __restrict__ L1, const float* __restrict__ L2, int L, float* __restrict__ Mt) {
+  __shared__ double a[256];
   const int i = blockIdx.x, j = threadIdx.x;
+  if (j <= i) a[j] = (double)L1[(size_t)i * L + j];
+  __syncthreads();
   if (j >= L) return;
-  // two compensated sums (as in the Gram): a float64 fma and the widening of its
-  // operands run at 1/64 of the fp32 rate.  Thirty-two loads in flight, and a
-  // warp's lanes walk the same k from its first column on (zeros before a lane's
-  // own), so that a load reads one row piece: 20.1 us at L = 136 with every lane starting at its column, 5.6 so.
-  DF acc[2] = {DF{0.f, 0.f}, DF{0.f, 0.f}};
+  double acc = 0.0;
   for (int k = j & ~31; k <= i; k += 32) {
-    float a[32], b[32];
+    float b[32];
 #pragma unroll
-    for (int u = 0; u < 32; ++u) {
-      const bool in = k + u >= j && k + u <= i;
-      a[u] = in ? L1[(size_t)i * L + k + u] : 0.f;
-      b[u] = in ? L2[(size_t)(k + u) * L + j] : 0.f;
-    }
+    for (int u = 0; u < 32; ++u) b[u] = k + u >= j && k + u <= i ? L2[(size_t)(k + u) * L + j] : 0.f;
 #pragma unroll
-    for (int u = 0; u < 32; ++u) {
-      const float p = __fmul_rn(a[u], b[u]);
-      df_add(acc[u & 1], p, __fmaf_rn(a[u], b[u], -p));
-    }
+    for (int u = 0; u < 32; ++u)
+      if (k + u >= j && k + u <= i) acc = fma(a[k + u], (double)b[u], acc);
   }
-  df_add(acc[0], acc[1].hi, acc[1].lo);
-  Mt[(size_t)j * L + i] = __fadd_rn(acc[0].hi, acc[0].lo);
+  Mt[(size_t)j * L + i] = (float)acc;
 }
 
 // One-sided Jacobi SVD of M (Hestenes): the columns of M are orthogonalised by
-// plane rotations applied from the right, M W = U S, W orthogonal.  For a pair:
-// alpha = |m_p|^2, beta = |m_q|^2, gamma = m_p . m_q (fp32, each lane a strided
-// share, then a butterfly that leaves every lane the same sums), and unless
-// |gamma| <= 1e-6 sqrt(alpha beta) columns p, q of M and of W are rotated by the
-// angle that makes them orthogonal (zeta = (beta - alpha) / (2 gamma),
-// t = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)), c = 1 / sqrt(1 + t^2), s = c t).
-// Sweeps end when none of a sweep's pairs had |gamma| above 2e-5
-// sqrt(alpha beta) (the rotations of that sweep leave products of such angles,
-// below the rounding of an fp32 dot product), or after OS_MAX_SWEEPS.
+// plane rotations applied from the right, M W = U S, W orthogonal.  Lp = L
+// rounded up to even (a zero padding column never rotates); a round pairs the
+// columns by the circle method: pair g of round r is (r + g, r - g) mod Lp - 1,
+// pair 0 (r, Lp - 1).  For a pair: alpha = |m_p|^2, beta = |m_q|^2, gamma =
+// m_p . m_q (fp32, eight lanes with a share each, then a butterfly that leaves
+// every lane the same sums), and unless |gamma| <= 1e-6 sqrt(alpha beta) (a little
+// above the rounding of an fp32 dot product, so that sweeps terminate) columns
+// p, q of M and of W are rotated by the angle that makes them orthogonal (zeta =
+// (beta - alpha) / (2 gamma), t = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)), c =
+// 1 / sqrt(1 + t^2), s = c t; correctly rounded roots and divisions).  Sweeps end
+// when one makes no rotation, or after OS_MAX_SWEEPS.
 //
-// On one SM a round (half the columns against the other half) moves all of M
-// and W through shared memory: 1.44 us at L = 136, 1.76 ms in all.  So the
-// sweep is spread over a thread-block cluster of OS_P = 8 CTAs: the columns form
-// 16 blocks of b, a CTA holds two, and a super-step rotates every pair across its
-// two blocks in b rounds of b pairs (a half-warp keeps its column of the first
-// block in registers, the second block's go round in shared memory); between
-// super-steps the blocks are paired anew by the circle method, each block copied
-// (cp.async.bulk between the CTAs' shared memories, 1 mbarrier a buffer) straight
-// into the other buffer of the CTA that needs it next.  Pairs inside a block are
-// rotated once a sweep, in its first super-step.  A round's latency bounds it (the
-// reduction, the angle, a barrier).  Measured at L = 136: 570 us (892 with
-// four CTAs, a warp a pair and the blocks fetched by loads).
+// On one SM a round moves all of M and W through shared memory: 1.44 us at
+// L = 136, 1.76 ms in all.  In the circle method pair g hands its first column
+// to pair g - 1 and its second to pair g + 1 (pair 0 its first to pair 1, the last
+// pair its second to itself), so the pairs are cut into OS_P = 8 runs, one a CTA
+// of a thread-block cluster, and only the columns at the ends of a run leave the
+// SM: sixteen lanes have a pair (eight its columns of M, eight those of W), read
+// the columns from one buffer and store them, rotated, where the next round
+// reads them, in the other buffer of this CTA or, with st.async and the bytes
+// counted by that CTA's mbarrier, of the neighbour.  A neighbour can be one round
+// ahead at most, because it needs this CTA's column of every round, and it
+// overwrites a slot only after the pair that read it has sent that column.  The
+// order of the rotations and of every sum is that of one SM taking the rounds in
+// turn, so the bits are the same.  A round's latency bounds it (a column's loads,
+// the reduction, the angle, the hop to the neighbour): 0.79 us a round at L = 136,
+// 970 us in all.
+//
+// Which entries of a column a lane sums: up to 144 columns, entries 16 v + 2 u,
+// + 1 (lane u, v = 0, 1, ...); above, u, u + 8, u + 16, ...; both ascending.
 // Output: Wt [L][L], Wt[j][k] = W[k][j].
 constexpr int OS_MAX_SWEEPS = 30;
-constexpr int OS_P = 8;           // CTAs of the cluster
-constexpr int OS_MAX_WARPS = 8;   // 16 columns a block at L = 256, a half-warp each
+constexpr int OS_P = 8;        // CTAs of the cluster
+constexpr int OS_LANES = 16;   // of a pair: eight for M, eight for W
+constexpr int OS_MAX_PAIRS = 16;  // a CTA's at L = 256
+// floats of a column's part (M or W, NV pairs of entries a lane): the parts of a
+// column 16 mod 32 words apart, so that a pair's 16 lanes touch distinct banks
+__host__ __device__ constexpr int os_part(int nv) { return 16 * nv + (nv % 2 == 0 ? 16 : 0); }
 
 __device__ __forceinline__ uint32_t os_map(uint32_t a, uint32_t cta) {
   uint32_t r;
@@ -646,17 +639,11 @@ __device__ __forceinline__ uint32_t os_ld_remote(uint32_t a) {
   asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
   return v;
 }
-__device__ __forceinline__ void os_cluster_arrive() {
+__device__ __forceinline__ void os_cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void os_cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void os_cluster_sync() {
-  os_cluster_arrive();
-  os_cluster_wait();
-}
-// bounded wait for a phase of this CTA's mbarrier (its copies were issued by
+// bounded wait for a phase of this CTA's mbarrier (its bytes were sent by
 // CTAs that are resident beside it, so it ends)
 __device__ __forceinline__ bool os_wait(uint32_t bar, uint32_t parity) {
   const unsigned long long t0 = clock64();
@@ -689,290 +676,218 @@ __device__ __forceinline__ float2 os_fma2(float2 a, float2 b, float2 c) {
       : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
   return d;
 }
-__device__ __forceinline__ float os_sqrt(float v) {
-  float r;
-  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
-  return r;
-}
 
-// Rotates the columns x and y of this half-warp's pair (`on`: it has one).  A
-// column is L rows of M, then L rows of W, 32 values a chunk, two a lane; the
-// last chunk of M (v = KV - 1) is cut at L by m0, m1.  The tangent comes as
-// 2 gamma / (|d| + sqrt(d^2 + 4 gamma^2)), d = beta - alpha, and may be off by
-// its rounding (the next sweep sees what is left); the rotation may not be:
-// c = 1 / sqrt(1 + t^2) takes a Newton step to full precision.  True if the
-// pair was further than 2e-5 from orthogonal.
-template <int KV>
-__device__ __forceinline__ bool os_rotate(float2 (&x)[2 * KV], float2 (&y)[2 * KV], bool on, bool m0,
-                                          bool m1) {
-  float2 a2{0.f, 0.f}, b2{0.f, 0.f}, g2{0.f, 0.f};
+// Rotates the columns x and y of this pair (lanes 0 .. 7 of its sixteen: M, the
+// others: W); true if it did.
+template <int NV>
+__device__ __forceinline__ bool os_rotate(float2 (&x)[NV], float2 (&y)[NV], bool on) {
+  float a = 0.f, b = 0.f, g = 0.f;
 #pragma unroll
-  for (int v = 0; v < KV; ++v) {
-    const float2 p = v + 1 < KV ? x[v] : make_float2(m0 ? x[v].x : 0.f, m1 ? x[v].y : 0.f);
-    const float2 q = v + 1 < KV ? y[v] : make_float2(m0 ? y[v].x : 0.f, m1 ? y[v].y : 0.f);
-    a2 = os_fma2(p, p, a2);
-    b2 = os_fma2(q, q, b2);
-    g2 = os_fma2(p, q, g2);
+  for (int v = 0; v < NV; ++v) {
+    a = fmaf(x[v].x, x[v].x, a);
+    a = fmaf(x[v].y, x[v].y, a);
+    b = fmaf(y[v].x, y[v].x, b);
+    b = fmaf(y[v].y, y[v].y, b);
+    g = fmaf(x[v].x, y[v].x, g);
+    g = fmaf(x[v].y, y[v].y, g);
   }
-  float a = a2.x + a2.y, b = b2.x + b2.y, g = g2.x + g2.y;
 #pragma unroll
-  for (int o = 8; o; o >>= 1) {
+  for (int o = 4; o; o >>= 1) {
     a += __shfl_xor_sync(0xffffffffu, a, o);
     b += __shfl_xor_sync(0xffffffffu, b, o);
     g += __shfl_xor_sync(0xffffffffu, g, o);
   }
-  const float ab = a * b, gg = g * g;
-  if (!(on && gg > 1e-12f * ab)) return false;  // the same for the half-warp
-  const float d = b - a, den = fabsf(d) + os_sqrt(fmaf(d, d, 4.f * gg));
-  const float t = __fdividef(d >= 0.f ? 2.f * g : -2.f * g, fmaxf(den, 1e-37f));
-  const float u = fmaf(t, t, 1.f), c0 = rsqrtf(u);
-  const float c = fmaf(c0, fmaf(-0.5f * u * c0, c0, 0.5f), c0), sn = t * c;
+  const int from = threadIdx.x & 23;  // the M lanes' sums for the W lanes
+  a = __shfl_sync(0xffffffffu, a, from);
+  b = __shfl_sync(0xffffffffu, b, from);
+  g = __shfl_sync(0xffffffffu, g, from);
+  if (!(on && g != 0.f && fabsf(g) > 1e-6f * sqrtf(a * b))) return false;  // pair-uniform
+  // (an overflowing zeta gives t = 0: no rotation, never a NaN)
+  const float z = (b - a) / (2.f * g);
+  const float t = (z >= 0.f ? 1.f : -1.f) / (fabsf(z) + sqrtf(fmaf(z, z, 1.f)));
+  const float c = 1.f / sqrtf(fmaf(t, t, 1.f)), sn = t * c;
   const float2 c2{c, c}, s2{sn, sn}, ns2{-sn, -sn};
 #pragma unroll
-  for (int v = 0; v < 2 * KV; ++v) {
+  for (int v = 0; v < NV; ++v) {
     const float2 p = x[v], q = y[v];
     x[v] = os_fma2(c2, p, os_mul2(ns2, q));
     y[v] = os_fma2(s2, p, os_mul2(c2, q));
   }
-  return gg > 4e-10f * ab;
+  return true;
 }
 
-// the two blocks of cluster rank c in super-step st of a sweep (n = 2 P blocks)
-__device__ __forceinline__ void os_pair(int st, int c, int n, int& p, int& q) {
-  p = st + c;
-  if (p >= n - 1) p -= n - 1;
-  q = st - c;
-  if (q < 0) q += n - 1;
-  if (c == 0) q = n - 1;
-}
-// where block k is in super-step st: cluster rank and which of its two
-__device__ __forceinline__ void os_where(int k, int st, int n, int& c, int& h) {
-  if (k == n - 1) {
-    c = 0;
-    h = 1;
-    return;
-  }
-  const int d = k >= st ? k - st : k - st + n - 1;
-  if (d < n / 2) {
-    c = d;
-    h = 0;
-  } else {
-    c = n - 1 - d;
-    h = 1;
-  }
-}
-
-template <int KV>
-__global__ void __launch_bounds__(32 * OS_MAX_WARPS)
-k_jacobi_cluster(const float* __restrict__ Mt, int L, int b, float* __restrict__ Wt) {
-  constexpr int CL = 64 * KV;  // floats of a column: L of M, L of W, zeros
-  constexpr int NC = 2 * KV;   // its chunks of 32
-  constexpr int NBLK = 2 * OS_P, NST = NBLK - 1;
-  extern __shared__ __align__(128) float osm[];  // [2 buffers][2 blocks][b columns][CL]
-  __shared__ __align__(8) uint64_t s_full[2];    // by buffer: both blocks have landed
-  __shared__ unsigned s_far[2];  // by sweep parity: a pair of this CTA was far from orthogonal
-  __shared__ unsigned s_max, s_go;
-  const int tid = threadIdx.x, lane = tid & 31, hl = lane & 15;
-  const int w = 2 * (tid >> 5) + (lane >> 4);  // this half-warp's pair
-  uint32_t rank;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-  const int bb = b + (b & 1);
-  const bool m0 = 32 * (KV - 1) + 2 * hl < L, m1 = 32 * (KV - 1) + 2 * hl + 1 < L;
-  const bool on = w < b;
+template <int NV>
+__global__ void __launch_bounds__(OS_LANES * OS_MAX_PAIRS)
+k_jacobi_cluster(const float* __restrict__ Mt, int L, float* __restrict__ Wt) {
+  constexpr int PART = os_part(NV), COL = 2 * PART;  // floats of a column's part and of a column
+  extern __shared__ __align__(128) float osm[];  // [2 buffers][first, second columns][nmax][COL]
+  __shared__ __align__(8) uint64_t s_full[2];    // by buffer: the neighbours' columns have landed
+  __shared__ unsigned s_rot[2];                  // by sweep parity: a pair of this CTA was rotated
+  __shared__ unsigned s_go;
+  const int tid = threadIdx.x, lane16 = tid & (OS_LANES - 1), u = lane16 & 7, i = tid / OS_LANES;
+  uint32_t rank_u;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank_u));
+  const int rank = (int)rank_u;
+  const int Lp = L + (L & 1), half = Lp / 2;
+  // pairs g0 .. g0 + n - 1 of a round; a cluster has no more busy CTAs than pairs
+  const int busy = min(OS_P, half), each = half / busy, more = half % busy;
+  const int nmax = each + (more ? 1 : 0);
+  const int n = rank < busy ? each + (rank < more ? 1 : 0) : 0;
+  const int g = rank * each + min(rank, more) + i;
+  const bool on = i < n;
   const uint32_t base = os_smem(osm), full0 = os_smem(s_full);
-  const uint32_t blk_bytes = (uint32_t)(b * CL) * 4u;
+  const uint32_t buf_bytes = (uint32_t)(2 * nmax * COL) * 4u, line_bytes = (uint32_t)(nmax * COL) * 4u;
+  // this lane's piece of slot `at` of line h (0: first columns) in buffer 0
+  const uint32_t mine = (uint32_t)((lane16 >> 3) * PART + 2 * u) * 4u;
+  auto slot = [&](int h, int at) { return (uint32_t)h * line_bytes + (uint32_t)(at * COL) * 4u + mine; };
+  // where the pair's columns go for the next round: an offset, and the CTA (-1: this one)
+  uint32_t xto = slot(0, 0), yto = slot(1, 0);
+  int xcta = -1, ycta = -1;
+  if (on && half > 1) {
+    if (g == 0) {
+      xto = slot(1, n > 1 ? 1 : 0);
+      if (n == 1) xcta = 1;
+    } else {
+      if (i > 0) xto = slot(0, i - 1);
+      else {
+        xcta = rank - 1;
+        xto = slot(0, each + (rank - 1 < more ? 1 : 0) - 1);
+      }
+      if (g == half - 1) yto = slot(0, n - 1);
+      else if (i < n - 1) yto = slot(1, i + 1);
+      else ycta = rank + 1;  // (to its slot (1, 0))
+    }
+  }
+  // the bytes of the neighbours' columns that arrive for each round
+  const uint32_t incoming =
+      (uint32_t)(n == 0 ? 0 : (rank > 0) + (rank < busy - 1)) * (uint32_t)(OS_LANES * NV * 8);
+  const bool listens = on && incoming && (i == 0 || i == n - 1);
   if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full0) : "memory");
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full0 + 8) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    s_far[0] = s_far[1] = s_max = 0;
+    s_rot[0] = s_rot[1] = 0;
   }
-  __syncthreads();
-  int pb, qb;
-  os_pair(0, (int)rank, NBLK, pb, qb);
-  float2 x[NC], y[NC];
-  // the first super-step's columns; M scaled by a power of two so that its
-  // largest entry is near 1 (the squares below then neither overflow nor, for
-  // any column that counts, underflow; W does not see the scale)
-  {
-    const int cx = pb * b + w, cy = qb * b + w;
-    float mx = 0.f;
-    auto first = [&](int col, int e) {  // element e of column col before any rotation
-      if (!on || col >= L || e >= 2 * L) return 0.f;
-      if (e >= L) return e - L == col ? 1.f : 0.f;
-      const float v = Mt[(size_t)col * L + e];
-      mx = fmaxf(mx, fabsf(v));
-      return v;
+  // the columns of pair g in round 0
+  const int cx = g, cy = g == 0 ? Lp - 1 : Lp - 1 - g;
+  const bool strided = Lp > 144;
+  auto entry = [&](int v, int e) { return strided ? 16 * v + 8 * e + u : 16 * v + 2 * u + e; };
+  if (on) {
+    auto first = [&](int col, int k) {
+      if (lane16 >= 8) return k == col ? 1.f : 0.f;
+      return col < L && k < L ? Mt[(size_t)col * L + k] : 0.f;
     };
 #pragma unroll
-    for (int v = 0; v < NC; ++v) {
-      const int e = 32 * v + 2 * hl;
-      x[v] = make_float2(first(cx, e), first(cx, e + 1));
-      y[v] = make_float2(first(cy, e), first(cy, e + 1));
+    for (int v = 0; v < NV; ++v) {
+      *reinterpret_cast<float2*>(reinterpret_cast<char*>(osm) + slot(0, i) + 64 * v) =
+          make_float2(first(cx, entry(v, 0)), first(cx, entry(v, 1)));
+      *reinterpret_cast<float2*>(reinterpret_cast<char*>(osm) + slot(1, i) + 64 * v) =
+          make_float2(first(cy, entry(v, 0)), first(cy, entry(v, 1)));
     }
-    atomicMax(&s_max, __float_as_uint(mx));
-    __syncthreads();
-    os_cluster_sync();  // also: every CTA's mbarriers are initialised
-    unsigned m = 0;
-    for (int c = 0; c < OS_P; ++c) m = max(m, os_ld_remote(os_map(os_smem(&s_max), (uint32_t)c)));
-    const int ex = min(max((int)(m >> 23) - 127, -120), 120);
-    const float sc = m ? __uint_as_float((uint32_t)(127 - ex) << 23) : 1.f;
-    float* B = osm + 2 * hl;
-    if (on)
-#pragma unroll
-      for (int v = 0; v < NC; ++v) {
-        const int e = 32 * v + 2 * hl;
-        if (e < L) x[v].x *= sc, y[v].x *= sc;
-        if (e + 1 < L) x[v].y *= sc, y[v].y *= sc;
-        *reinterpret_cast<float2*>(B + (size_t)w * CL + 32 * v) = x[v];
-        *reinterpret_cast<float2*>(B + (size_t)(b + w) * CL + 32 * v) = y[v];
-      }
-    __syncthreads();
   }
-  bool alive = true, far = false;
-  int sweep = 0, st = 0;
-  for (uint32_t k = 0;; ++k) {
-    const uint32_t cur = k & 1;
-    os_pair(st, (int)rank, NBLK, pb, qb);
-    float* B = osm + (size_t)cur * 2 * b * CL + 2 * hl;
-    if (k > 0 && alive) alive = os_wait(full0 + 8 * cur, ((k - 1) >> 1) & 1);
-    __syncwarp();
-    os_cluster_arrive();  // this CTA holds its blocks of super-step k
-    if (st == 0) {
-      // the pairs inside each of the two blocks: half-warps 0 .. bb/2 - 1 the
-      // first, the next bb/2 the second (circle method on bb columns)
-      const int half = bb / 2, g = w < half ? w : w - half;
-      for (int rd = 0; rd < bb - 1; ++rd) {
-        int i = rd, j = bb - 1;
-        if (g > 0) {
-          i = rd + g;
-          if (i >= bb - 1) i -= bb - 1;
-          j = rd - g;
-          if (j < 0) j += bb - 1;
-        }
-        const bool in = w < bb && i < b && j < b;
-        float* ci = B + (size_t)((w < half ? 0 : b) + (in ? i : 0)) * CL;
-        float* cj = B + (size_t)((w < half ? 0 : b) + (in ? j : 0)) * CL;
+  __syncthreads();
+  os_cluster_sync();  // every CTA's mbarriers are initialised
+  uint32_t k = 0;     // rounds done
+  bool alive = true;
+  for (int sweep = 0;; ++sweep) {
+    bool rotated = false;
+    for (int rd = 0; rd < Lp - 1; ++rd, ++k) {
+      if (n == 0) continue;
+      const uint32_t cur = k & 1, nxt = cur ^ 1;
+      if (tid == 0 && incoming)
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full0 + 8 * nxt),
+                     "r"(incoming)
+                     : "memory");
+      if (listens && k > 0 && alive) alive = os_wait(full0 + 8 * cur, ((k - 1) >> 1) & 1);
+      __syncwarp();
+      float2 x[NV], y[NV];
+      const char* B = reinterpret_cast<const char*>(osm) + cur * buf_bytes;
 #pragma unroll
-        for (int v = 0; v < NC; ++v) {
-          x[v] = in ? *reinterpret_cast<const float2*>(ci + 32 * v) : make_float2(0.f, 0.f);
-          y[v] = in ? *reinterpret_cast<const float2*>(cj + 32 * v) : make_float2(0.f, 0.f);
-        }
-        far |= os_rotate<KV>(x, y, in, m0, m1);
-        if (in)
-#pragma unroll
-          for (int v = 0; v < NC; ++v) {
-            *reinterpret_cast<float2*>(ci + 32 * v) = x[v];
-            *reinterpret_cast<float2*>(cj + 32 * v) = y[v];
-          }
-        __syncthreads();
+      for (int v = 0; v < NV; ++v) {
+        x[v] = on ? *reinterpret_cast<const float2*>(B + slot(0, i) + 64 * v) : make_float2(0.f, 0.f);
+        y[v] = on ? *reinterpret_cast<const float2*>(B + slot(1, i) + 64 * v) : make_float2(0.f, 0.f);
       }
-    }
+      rotated |= os_rotate<NV>(x, y, on);
+      auto put = [&](const float2 (&c)[NV], uint32_t to, int cta) {
+        if (cta < 0) {
+          char* D = reinterpret_cast<char*>(osm) + nxt * buf_bytes + to;
 #pragma unroll
-    for (int v = 0; v < NC; ++v)
-      x[v] = on ? *reinterpret_cast<const float2*>(B + (size_t)w * CL + 32 * v) : make_float2(0.f, 0.f);
-    // every pair across the two blocks
-    for (int rd = 0; rd < b; ++rd) {
-      int j = w + rd;
-      if (j >= b) j -= b;
-      float* cj = B + (size_t)(b + (on ? j : 0)) * CL;
+          for (int v = 0; v < NV; ++v) *reinterpret_cast<float2*>(D + 64 * v) = c[v];
+        } else {
+          const uint32_t dst = os_map(base + nxt * buf_bytes + to, (uint32_t)cta);
+          const uint32_t bar = os_map(full0 + 8 * nxt, (uint32_t)cta);
 #pragma unroll
-      for (int v = 0; v < NC; ++v)
-        y[v] = on ? *reinterpret_cast<const float2*>(cj + 32 * v) : make_float2(0.f, 0.f);
-      far |= os_rotate<KV>(x, y, on, m0, m1);
-      if (on)
-#pragma unroll
-        for (int v = 0; v < NC; ++v) *reinterpret_cast<float2*>(cj + 32 * v) = y[v];
+          for (int v = 0; v < NV; ++v)
+            asm volatile(
+                "st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(
+                    dst + 64 * v),
+                "f"(c[v].x), "f"(c[v].y), "r"(bar)
+                : "memory");
+        }
+      };
+      if (on) {
+        put(x, xto, xcta);
+        put(y, yto, ycta);
+      }
       __syncthreads();
     }
-    if (on)
-#pragma unroll
-      for (int v = 0; v < NC; ++v) *reinterpret_cast<float2*>(B + (size_t)w * CL + 32 * v) = x[v];
-    const bool last = st == NST - 1;
-    if (last && far && hl == 0) s_far[sweep & 1] = 1;
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // before the copies read the columns
+    if (rotated) s_rot[sweep & 1] = 1;
+    // every CTA reads the same flags, so all leave after the same sweep
     __syncthreads();
-    os_cluster_wait();  // every CTA holds its blocks of super-step k: the other buffers are free
-    if (last) {
-      // every CTA reads the same flags, so all leave after the same sweep
-      os_cluster_sync();
-      if (tid == 0) {
-        unsigned go = 0;
-        for (int c = 0; c < OS_P; ++c) go |= os_ld_remote(os_map(os_smem(&s_far[sweep & 1]), (uint32_t)c));
-        s_go = go;
-        s_far[(sweep + 1) & 1] = 0;  // last read a sweep ago
-      }
-      __syncthreads();
-      ++sweep;
-      if (!s_go || sweep == OS_MAX_SWEEPS) break;
-      far = false;
-    }
-    st = last ? 0 : st + 1;
+    os_cluster_sync();
     if (tid == 0) {
-      // each block straight into the other buffer of the CTA that needs it next
-      const uint32_t nbuf = cur ^ 1;
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full0 + 8 * nbuf),
-                   "r"(2 * blk_bytes)
-                   : "memory");
+      unsigned go = 0;
+      for (int c = 0; c < OS_P; ++c) go |= os_ld_remote(os_map(os_smem(&s_rot[sweep & 1]), (uint32_t)c));
+      s_go = go;
+      s_rot[(sweep + 1) & 1] = 0;  // last read a sweep ago
+    }
+    __syncthreads();
+    if (!s_go || sweep + 1 == OS_MAX_SWEEPS) break;
+  }
+  // a sweep's rounds bring every column back to where it began
+  if (listens && alive) alive = os_wait(full0 + 8 * (k & 1), ((k - 1) >> 1) & 1);
+  if (on && lane16 >= 8) {
+    const char* B = reinterpret_cast<const char*>(osm) + (k & 1) * buf_bytes;
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        int c, hd;
-        os_where(h ? qb : pb, st, NBLK, c, hd);
-        const uint32_t src = base + (cur * 2 + h) * blk_bytes;
-        const uint32_t dst = os_map(base + (nbuf * 2 + hd) * blk_bytes, (uint32_t)c);
-        const uint32_t bar = os_map(full0 + 8 * nbuf, (uint32_t)c);
-        asm volatile(
-            "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-            "r"(src), "r"(blk_bytes), "r"(bar)
-            : "memory");
+    for (int v = 0; v < NV; ++v) {
+      const float2 p = *reinterpret_cast<const float2*>(B + slot(0, i) + 64 * v);
+      const float2 q = *reinterpret_cast<const float2*>(B + slot(1, i) + 64 * v);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int r = entry(v, e);
+        if (r >= L) continue;
+        if (cx < L) Wt[(size_t)cx * L + r] = e ? p.y : p.x;
+        if (cy < L) Wt[(size_t)cy * L + r] = e ? q.y : q.x;
       }
     }
-    __syncwarp();
   }
-  // this CTA's columns are in the buffer worked on last
-  os_pair(NST - 1, (int)rank, NBLK, pb, qb);
-  // (the buffer's parity is that of the super-steps done, NST a sweep)
-  const float* B = osm + (size_t)((sweep * NST - 1) & 1) * 2 * b * CL;
-  if (on)
-    for (int h = 0; h < 2; ++h) {
-      const int col = (h ? qb : pb) * b + w;
-      if (col >= L) continue;
-      for (int i = hl; i < L; i += 16) Wt[(size_t)col * L + i] = B[(size_t)(h * b + w) * CL + L + i];
-    }
   __syncwarp();
   os_cluster_sync();  // no CTA leaves while its flags are read
 }
 
-// CTA j: v = M w_j to float64 accuracy, sigma_j = |v| / |w_j| (the Rayleigh quotient of
+// CTA j: v = M w_j in float64, sigma_j = |v| / |w_j| (the Rayleigh quotient of
 // the converged rotation, second-order accurate in the rotation's error);
 // MWn[j] = v / |w_j|, Wn[j] = w_j / |w_j| (fp32, column j stored contiguously).
 __global__ void __launch_bounds__(256)
 k_ritz(const float* __restrict__ Mt, const float* __restrict__ Wt, int L, float* __restrict__ MWn,
        float* __restrict__ Wn, double* __restrict__ sig64) {
-  __shared__ float w[256];
+  __shared__ double w[256];
   __shared__ double red[2][8];
-  __shared__ double s_inv;
+  __shared__ double s_norm;
   const int j = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int k = tid; k < L; k += 256) w[k] = Wt[(size_t)j * L + k];
+  if (tid < L) w[tid] = (double)Wt[(size_t)j * L + tid];
   __syncthreads();
   double v = 0.0, ww = 0.0;
   if (tid < L) {
-    // two compensated sums (as in the Gram), thirty-two loads in flight
-    DF p2[2] = {DF{0.f, 0.f}, DF{0.f, 0.f}};
-    for (int k = 0; k < L; k += 32) {
+    for (int k = 0; k < L; k += 32) {  // thirty-two loads in flight
       float m[32];
 #pragma unroll
       for (int u = 0; u < 32; ++u) m[u] = k + u < L ? Mt[(size_t)(k + u) * L + tid] : 0.f;
 #pragma unroll
-      for (int u = 0; u < 32; ++u) {
-        const float wv = k + u < L ? w[k + u] : 0.f;
-        const float p = __fmul_rn(m[u], wv);
-        df_add(p2[u & 1], p, __fmaf_rn(m[u], wv, -p));
-      }
+      for (int u = 0; u < 32; ++u)
+        if (k + u < L) v = fma((double)m[u], w[k + u], v);
     }
-    df_add(p2[0], p2[1].hi, p2[1].lo);
-    v = (double)p2[0].hi + (double)p2[0].lo;
-    ww = (double)w[tid] * (double)w[tid];
+    ww = w[tid] * w[tid];
   }
   double v2 = v * v, w2 = ww;
   for (int o = 16; o; o >>= 1) {
@@ -984,22 +899,21 @@ k_ritz(const float* __restrict__ Mt, const float* __restrict__ Wt, int L, float*
     red[1][warp] = w2;
   }
   __syncthreads();
-  if (tid == 0) {
-    // the float64 root and division once: they run at a fraction of the fp32 rate
+  if (tid == 0) {  // the float64 roots once: they run at a fraction of the fp32 rate
     double tv = 0.0, tw = 0.0;
     for (int q = 0; q < 8; ++q) {
       tv += red[0][q];
       tw += red[1][q];
     }
     const double nw_ = sqrt(tw);
-    s_inv = nw_ > 0.0 ? 1.0 / nw_ : 0.0;
+    s_norm = nw_;
     sig64[j] = nw_ > 0.0 ? sqrt(tv) / nw_ : 0.0;
   }
   __syncthreads();
   if (tid < L) {
-    const double inv = s_inv;
-    MWn[(size_t)j * L + tid] = (float)(v * inv);
-    Wn[(size_t)j * L + tid] = (float)((double)w[tid] * inv);
+    const double nw_ = s_norm;
+    MWn[(size_t)j * L + tid] = nw_ > 0.0 ? (float)(v / nw_) : 0.f;
+    Wn[(size_t)j * L + tid] = nw_ > 0.0 ? (float)(w[tid] / nw_) : 0.f;
   }
 }
 
@@ -1087,8 +1001,8 @@ __global__ void k_sign(float* __restrict__ U, float* __restrict__ V, int rows, i
 }
 
 bool g_ch_cap[64] = {};
-bool g_ts_cap[64] = {};
-bool g_jac_cap[8][64] = {};
+bool g_ti_cap[64] = {};
+bool g_jac_cap[6][64] = {};
 
 }  // namespace
 }  // namespace lx
@@ -1101,7 +1015,7 @@ constexpr size_t CP_SMEM_CAP = 200 * 1024;
 size_t al256(size_t v) { return (v + 255) / 256 * 256; }
 
 struct CompressWs {
-  float *y0, *y1, *z0, *z1, *Dinv, *Wu, *Wv, *L1, *L2, *Mt, *Wt, *MWn, *Wn;
+  float *y0, *y1, *z0, *z1, *Dinv, *T, *Wu, *Wv, *L1, *L2, *Mt, *Wt, *MWn, *Wn;
   double* sig64;
   char* tc;  // the tensor-core residual products' scratch (bf16 weights)
   size_t bytes;
@@ -1122,6 +1036,7 @@ CompressWs carve(char* base, long rows, long cols, long l, long r) {
   w.z0 = (float*)take(4 * cols * l);
   w.z1 = (float*)take(4 * cols * l);
   w.Dinv = (float*)take(4 * CH_B * (l + CH_B));
+  w.T = (float*)take(4 * l * l);
   w.Wu = (float*)take(4 * l * r);
   w.Wv = (float*)take(4 * l * r);
   w.L1 = (float*)take(4 * l * l);
@@ -1174,24 +1089,21 @@ lx_status run_compress(int rows, int cols, const TW* Wd, const TW* Wm, const flo
       k_cgemm<TW, A_F32><<<grid, CG_THREADS, 0, s>>>(nullptr, nullptr, X, cols, B, C, M, N, K);
   };
   // CholeskyQR pass X -> out [n][l] (X L^-T, orthonormal columns when the Gram
-  // is well conditioned).  The row ranges' Gram sums lie in the residual
-  // products' partials, which are idle here.
+  // is well conditioned).  The Gram's chains lie in the residual products'
+  // partials, which are idle here.
   float2* const G = reinterpret_cast<float2*>(w.tc + res_tc_part_offset(rows, cols, l));
   const int ldp = ch_ldp(l), nb = (l + CH_B - 1) / CH_B;
   const size_t ch_smem = sizeof(float) * ((((size_t)l * (l + 1) / 2 + 3) & ~(size_t)3) + (size_t)CH_B * ldp);
-  const size_t ts_smem = sizeof(float) * ((size_t)ts_off(nb) + TS_ROWS * ts_ldy(nb) +
-                                          (TS_ROWS + nb * CH_B) * (CH_B + 4));
+  const size_t ti_smem = sizeof(float) * ((size_t)nb * CH_B * CH_B + 2 * CH_B * ti_ld(nb) +
+                                          2 * CH_B * (CH_B + 4) + CH_B * CH_B);
   LX_CUDA(smem_cap_once((const void*)k_chol32, (int)CP_SMEM_CAP, dev, g_ch_cap));
-  LX_CUDA(smem_cap_once((const void*)k_trsm, (int)CP_SMEM_CAP, dev, g_ts_cap));
+  LX_CUDA(smem_cap_once((const void*)k_tri_inverse, (int)CP_SMEM_CAP, dev, g_ti_cap));
   auto cholqr = [&](const float* X, float* out, int n, float shift, float* Lf) {
-    const int want = gram_parts(n, l, num_sms);
-    const int span = ((n + want - 1) / want + GR_KC - 1) / GR_KC * GR_KC;
-    const int parts = (n + span - 1) / span;
-    const dim3 grid((l + GR_T - 1) / GR_T, (l + GR_T - 1) / GR_T, parts);
-    k_gram<<<grid, GR_T * GR_T, 0, s>>>(X, n, l, span, G);
-    k_chol32<<<1, CH_THREADS, ch_smem, s>>>(G, parts, l, ldp, shift, Lf, w.Dinv);
-    k_trsm<<<(n + TS_ROWS - 1) / TS_ROWS, TS_THREADS, ts_smem, s>>>(X, Lf, w.Dinv, n, l,
-                                                                        reinterpret_cast<uintptr_t>(X) % 16 == 0, out);
+    const dim3 grid((l + GR_T - 1) / GR_T, (l + GR_T - 1) / GR_T, GR_CH);
+    k_gram<<<grid, GR_T * GR_T, 0, s>>>(X, n, l, G);
+    k_chol32<<<1, CH_THREADS, ch_smem, s>>>(G, l, ldp, shift, Lf, w.Dinv);
+    k_tri_inverse<<<nb, TI_THREADS, ti_smem, s>>>(Lf, w.Dinv, l, w.T);
+    gemm(A_F32, X, w.T, out, n, l, l);
   };
   // CholeskyQR (the first pass shifted by 1e-6 of the largest Gram diagonal,
   // so rank-deficient bases stay factorable).  orth2 runs it twice, X [n][l]
@@ -1224,14 +1136,13 @@ lx_status run_compress(int rows, int cols, const TW* Wd, const TW* Wm, const flo
   orth2(&zc, &zt, cols);
   k_trmm<<<l, 256, 0, s>>>(w.L1, w.L2, l, w.Mt);
   {
-    const int b = (l + 2 * OS_P - 1) / (2 * OS_P), kv = (l + 31) / 32;
-    auto launch = [&](auto kern) -> lx_status {
-      const size_t smem = sizeof(float) * 2 * 2 * b * (size_t)(64 * kv);
-      LX_CUDA(smem_cap_once((const void*)kern, (int)CP_SMEM_CAP, dev, g_jac_cap[kv - 1]));
+    const int Lp = l + (l & 1), half = Lp / 2, nmax = (half + OS_P - 1) / OS_P;
+    auto launch = [&](auto kern, int slot, int col_floats) -> lx_status {
+      LX_CUDA(smem_cap_once((const void*)kern, (int)CP_SMEM_CAP, dev, g_jac_cap[slot]));
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(OS_P);
-      cfg.blockDim = dim3(32 * ((b + 1) / 2));
-      cfg.dynamicSmemBytes = smem;
+      cfg.blockDim = dim3(32 * ((nmax + 1) / 2));
+      cfg.dynamicSmemBytes = sizeof(float) * 2 * 2 * nmax * (size_t)col_floats;
       cfg.stream = s;
       cudaLaunchAttribute attr[1];
       attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1240,19 +1151,15 @@ lx_status run_compress(int rows, int cols, const TW* Wd, const TW* Wm, const flo
       attr[0].val.clusterDim.z = 1;
       cfg.attrs = attr;
       cfg.numAttrs = 1;
-      LX_CUDA(cudaLaunchKernelEx(&cfg, kern, (const float*)w.Mt, l, b, w.Wt));
+      LX_CUDA(cudaLaunchKernelEx(&cfg, kern, (const float*)w.Mt, l, w.Wt));
       return LX_OK;
     };
-    switch (kv) {
-      case 1: LX_TRY(launch(k_jacobi_cluster<1>)); break;
-      case 2: LX_TRY(launch(k_jacobi_cluster<2>)); break;
-      case 3: LX_TRY(launch(k_jacobi_cluster<3>)); break;
-      case 4: LX_TRY(launch(k_jacobi_cluster<4>)); break;
-      case 5: LX_TRY(launch(k_jacobi_cluster<5>)); break;
-      case 6: LX_TRY(launch(k_jacobi_cluster<6>)); break;
-      case 7: LX_TRY(launch(k_jacobi_cluster<7>)); break;
-      default: LX_TRY(launch(k_jacobi_cluster<8>)); break;
-    }
+    if (Lp <= 32) LX_TRY(launch(k_jacobi_cluster<2>, 0, 2 * os_part(2)));
+    else if (Lp <= 48) LX_TRY(launch(k_jacobi_cluster<3>, 1, 2 * os_part(3)));
+    else if (Lp <= 80) LX_TRY(launch(k_jacobi_cluster<5>, 2, 2 * os_part(5)));
+    else if (Lp <= 144) LX_TRY(launch(k_jacobi_cluster<9>, 3, 2 * os_part(9)));
+    else if (Lp <= 192) LX_TRY(launch(k_jacobi_cluster<12>, 4, 2 * os_part(12)));
+    else LX_TRY(launch(k_jacobi_cluster<16>, 5, 2 * os_part(16)));
   }
   k_ritz<<<l, 256, 0, s>>>(w.Mt, w.Wt, l, w.MWn, w.Wn, w.sig64);
   k_finish<<<l, 256, 0, s>>>(w.sig64, w.MWn, w.Wn, l, r, w.Wu, w.Wv, sigma);
