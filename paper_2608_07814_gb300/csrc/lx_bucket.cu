@@ -27,7 +27,7 @@ constexpr int BK_WORDS = BK_TOK / 32;  // bitmap words of a key in a block
 // five at 8192 tokens and 256 keys, 25 for these three); word w belongs to warp
 // w alone, so the shared-memory atomics meet only inside a warp.
 __global__ void __launch_bounds__(BK_TOK)
-k_mark_bits(const int* __restrict__ topk_id, int T, int k, int N, int E,
+k_mark_bits(const int* topk_id, int T, int k, int N, int E,
             const int* __restrict__ paths, uint32_t* __restrict__ bits, int* __restrict__ cnt) {
   extern __shared__ __align__(16) uint32_t sb[];
   const int keys = N + E, tid = threadIdx.x;
@@ -42,7 +42,7 @@ k_mark_bits(const int* __restrict__ topk_id, int T, int k, int N, int E,
       int e[U];
       int4 p[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) e[u] = s0 + u < k ? topk_id[(size_t)t * k + s0 + u] : -1;
+      for (int u = 0; u < U; ++u) e[u] = s0 + u < k ? ld_dep(topk_id + (size_t)t * k + s0 + u) : -1;
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         if (e[u] >= E) e[u] = -1;  // invalid ids are ignored
@@ -73,15 +73,14 @@ k_mark_bits(const int* __restrict__ topk_id, int T, int k, int N, int E,
 static_assert(BK_WORDS == 8 && LX_MAX_DEPTH == 4, "two 16-byte pieces a key, one a path");
 
 // number of tokens before t that have the key (pre: those of earlier blocks)
-__device__ __forceinline__ int rank_before(const uint32_t* __restrict__ bits, const int* __restrict__ pre,
-                                           int keys, int key, int t) {
+__device__ __forceinline__ int rank_before(const uint32_t* bits, const int* pre, int keys, int key, int t) {
   const size_t row = (size_t)(t / BK_TOK) * keys + key;
-  const uint4 a = __ldcg(reinterpret_cast<const uint4*>(bits) + 2 * row);
-  const uint4 b = __ldcg(reinterpret_cast<const uint4*>(bits) + 2 * row + 1);
+  const uint4 a = ld_dep(reinterpret_cast<const uint4*>(bits) + 2 * row);
+  const uint4 b = ld_dep(reinterpret_cast<const uint4*>(bits) + 2 * row + 1);
   const uint32_t v[BK_WORDS] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
   const int w = (t % BK_TOK) >> 5;
   const uint32_t below = (1u << (t & 31)) - 1u;
-  int r = __ldcg(pre + row);
+  int r = ld_dep(pre + row);
 #pragma unroll
   for (int j = 0; j < BK_WORDS; ++j) r += __popc(v[j] & (j < w ? 0xffffffffu : j == w ? below : 0u));
   return r;
@@ -188,7 +187,7 @@ inline size_t op_smem(int keys, int N) { return sizeof(int) * ((size_t)keys + 2 
 // before the wait for the preceding kernel; the plans, one after another over
 // the whole CTA, had made this 9.8 us at 8192 tokens (6.6 now).
 __global__ void __launch_bounds__(OP_THREADS)
-k_offsets_plan(const int* __restrict__ cnt, int nblk, int N, int E, int* __restrict__ pre,
+k_offsets_plan(const int* cnt, int nblk, int N, int E, int* __restrict__ pre,
                int* __restrict__ key_off, const int* __restrict__ rank, int* __restrict__ tile_off,
                int max_items, PlanArgs pa, const int* __restrict__ anchors, int n_anchor,
                const int* __restrict__ corrs, int n_corr, int blk, int* __restrict__ act,
@@ -209,7 +208,7 @@ k_offsets_plan(const int* __restrict__ cnt, int nblk, int N, int E, int* __restr
     for (int b0 = 0; b0 < nblk; b0 += 16) {
       int v[16];
 #pragma unroll
-      for (int u = 0; u < 16; ++u) v[u] = b0 + u < nblk ? cnt[(size_t)(b0 + u) * keys + key] : 0;
+      for (int u = 0; u < 16; ++u) v[u] = b0 + u < nblk ? ld_dep(cnt + (size_t)(b0 + u) * keys + key) : 0;
 #pragma unroll
       for (int u = 0; u < 16; ++u)
         if (b0 + u < nblk) {
@@ -280,10 +279,9 @@ struct XRows {
 // without it, of the 256-expert layer's 4096 592 -> 575.  Two tokens a CTA, so
 // that a batch of hundreds spreads over the SMs.
 __global__ void __launch_bounds__(256)
-k_assign_rows(const int* __restrict__ topk_id, int T, int k, int N, int E, int D,
+k_assign_rows(const int* topk_id, int T, int k, int N, int E, int D,
               const int* __restrict__ paths, const int* __restrict__ path_len,
-              const int* __restrict__ key_off, const uint32_t* __restrict__ bits,
-              const int* __restrict__ pre, int* __restrict__ node_tok,
+              const int* key_off, const uint32_t* bits, const int* pre, int* __restrict__ node_tok,
               int* __restrict__ perm, int* __restrict__ node_row, const CtMeta cm, const TokRows tr,
               const XRows gr) {
   pdl_wait();
@@ -291,13 +289,13 @@ k_assign_rows(const int* __restrict__ topk_id, int T, int k, int N, int E, int D
   const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (t >= T) return;
   const size_t a = (size_t)t * k + lane;
-  int e = lane < k ? topk_id[a] : -1, len = 0;
+  int e = lane < k ? ld_dep(topk_id + a) : -1, len = 0;
   if (e < 0 || e >= E) e = -1;
   const unsigned twins = __match_any_sync(0xffffffffu, e);
   if (e >= 0) {
     len = path_len[e];
     if (lane == __ffs(twins) - 1)  // a repeated id counts once, with its first slot
-      perm[key_off[N + 1 + e] + rank_before(bits, pre, N + E, N + e, t)] = (int)a;
+      perm[ld_dep(key_off + N + 1 + e) + rank_before(bits, pre, N + E, N + e, t)] = (int)a;
   }
   int arow = -1;  // the anchor's row: the last level
   int r0 = -1, r1 = -1, n0 = -1, ev = -1;  // ev: entry `lane` = slot lane / D, level lane % D
@@ -307,7 +305,7 @@ k_assign_rows(const int* __restrict__ topk_id, int T, int k, int N, int E, int D
     int row = -1;
     if (l < len) {
       const int n = paths[e * LX_MAX_DEPTH + l];
-      row = key_off[n] + rank_before(bits, pre, N + E, n, t);
+      row = ld_dep(key_off + n) + rank_before(bits, pre, N + E, n, t);
       node_tok[row] = t;
       if (l == 0) n0 = n;
       if (l == len - 1) arow = row;
@@ -346,7 +344,7 @@ k_assign_rows(const int* __restrict__ topk_id, int T, int k, int N, int E, int D
       uint4 v[U];
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if (i0 + 32 * u < gr.vec) v[u] = __ldg(src + i0 + 32 * u);
+        if (i0 + 32 * u < gr.vec) v[u] = ld_dep(src + i0 + 32 * u);
       for (unsigned b = lead; b; b &= b - 1) {
         uint4* dst = gr.xg + (size_t)__shfl_sync(0xffffffffu, arow, __ffs(b) - 1) * gr.vec;
 #pragma unroll
@@ -427,7 +425,7 @@ __host__ __device__ inline size_t sb_smem(int T, int k, int keys, int E, int N) 
 }
 
 __global__ void __launch_bounds__(SB_THREADS)
-k_bucket_small(const float* __restrict__ logits, const int* __restrict__ ids_in, int T, int k,
+k_bucket_small(const float* logits, const int* ids_in, int T, int k,
                int E, int N, int D, const int* __restrict__ paths,
                const int* __restrict__ path_len, const int* __restrict__ rank,
                int* __restrict__ topk_id, float* __restrict__ topk_w, int* __restrict__ key_off_g,
@@ -464,7 +462,7 @@ k_bucket_small(const float* __restrict__ logits, const int* __restrict__ ids_in,
   }
   pdl_wait();
   if (!logits)  // the given ids (written by the preceding kernel)
-    for (int i = tid; i < T * k; i += nth) ids[i] = ids_in[i];
+    for (int i = tid; i < T * k; i += nth) ids[i] = ld_dep(ids_in + i);
   // 1. routing (or the given ids)
   if (logits) {
     for (int t = warp; t < T; t += nw) {

@@ -365,9 +365,8 @@ __device__ __forceinline__ void store4<__nv_bfloat16>(__nv_bfloat16* p, float4 v
 
 template <typename TZ>
 __global__ void __launch_bounds__(SW_T)
-k_swiglu_aggregate(const int* __restrict__ topk_id, const float* __restrict__ topk_w,
-                   const int* __restrict__ node_row, int T, int k, int D,
-                   const float* __restrict__ h, int I, TZ* __restrict__ z) {
+k_swiglu_aggregate(const float* topk_w, const int* node_row, int T, int k, int D, const float* h, int I,
+                   TZ* __restrict__ z) {
   pdl_wait();
   extern __shared__ float4 zacc[];  // [distinct rows][SW_T]
   __shared__ int rows[LX_MAX_K * LX_MAX_DEPTH], lrow[LX_MAX_K * LX_MAX_DEPTH];
@@ -376,8 +375,8 @@ k_swiglu_aggregate(const int* __restrict__ topk_id, const float* __restrict__ to
   __shared__ int nd_s;
   const int kD = k * D;
   for (int t = blockIdx.x; t < T; t += gridDim.x) {
-    for (int j = threadIdx.x; j < kD; j += blockDim.x) rows[j] = node_row[(size_t)t * kD + j];
-    for (int j = threadIdx.x; j < k; j += blockDim.x) gw[j] = topk_w[(size_t)t * k + j];
+    for (int j = threadIdx.x; j < kD; j += blockDim.x) rows[j] = ld_dep(node_row + (size_t)t * kD + j);
+    for (int j = threadIdx.x; j < k; j += blockDim.x) gw[j] = ld_dep(topk_w + (size_t)t * k + j);
     __syncthreads();
     // distinct rows, numbered in order of first appearance (entry j owns the
     // number of first appearances before it)
@@ -419,8 +418,8 @@ k_swiglu_aggregate(const int* __restrict__ topk_id, const float* __restrict__ to
           for (int l = 0; l < D; ++l) {
             const int r = rows[sl * D + l];
             if (r < 0) continue;
-            const float4 a = *reinterpret_cast<const float4*>(h + (size_t)r * 2 * I + i);
-            const float4 b = *reinterpret_cast<const float4*>(h + (size_t)r * 2 * I + I + i);
+            const float4 a = ld_dep(reinterpret_cast<const float4*>(h + (size_t)r * 2 * I + i));
+            const float4 b = ld_dep(reinterpret_cast<const float4*>(h + (size_t)r * 2 * I + I + i));
             pg.x += a.x; pg.y += a.y; pg.z += a.z; pg.w += a.w;
             pu.x += b.x; pu.y += b.y; pu.z += b.z; pu.w += b.w;
           }
@@ -445,14 +444,13 @@ k_swiglu_aggregate(const int* __restrict__ topk_id, const float* __restrict__ to
 // each thread owns four columns and issues four rows' loads at a time.
 template <typename TY>
 __global__ void __launch_bounds__(256)
-k_combine(const int* __restrict__ node_row, int k, int D, const float* __restrict__ ypart, int H,
-          TY* __restrict__ y, int T) {
+k_combine(const int* node_row, int k, int D, const float* ypart, int H, TY* __restrict__ y, int T) {
   pdl_wait();
   __shared__ int raw_s[LX_MAX_K * LX_MAX_DEPTH];
   __shared__ int rows_s[LX_MAX_K * LX_MAX_DEPTH];
   __shared__ int nrows_s;
   for (int t = blockIdx.x; t < T; t += gridDim.x) {
-    for (int j = threadIdx.x; j < k * D; j += blockDim.x) raw_s[j] = node_row[(long)t * k * D + j];
+    for (int j = threadIdx.x; j < k * D; j += blockDim.x) raw_s[j] = ld_dep(node_row + (long)t * k * D + j);
     __syncthreads();
     // distinct rows in ascending order: each first occurrence takes the rank
     // of its value among the distinct values
@@ -491,14 +489,14 @@ k_combine(const int* __restrict__ node_row, int k, int D, const float* __restric
         float4 v[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-          v[u] = *reinterpret_cast<const float4*>(ypart + (size_t)rows_s[q + u] * H + c);
+          v[u] = ld_dep(reinterpret_cast<const float4*>(ypart + (size_t)rows_s[q + u] * H + c));
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           acc.x += v[u].x; acc.y += v[u].y; acc.z += v[u].z; acc.w += v[u].w;
         }
       }
       for (; q < m; ++q) {
-        const float4 v = *reinterpret_cast<const float4*>(ypart + (size_t)rows_s[q] * H + c);
+        const float4 v = ld_dep(reinterpret_cast<const float4*>(ypart + (size_t)rows_s[q] * H + c));
         acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
       }
       store4<TY>(y + (size_t)t * H + c, acc);
@@ -576,19 +574,19 @@ template <int CPL>
 __device__ __forceinline__ Cols<CPL> ld_cols(const float* p) {
   Cols<CPL> r;
   if constexpr (CPL == 8) {
-    const float4 f = __ldg(reinterpret_cast<const float4*>(p));
-    const float4 g = __ldg(reinterpret_cast<const float4*>(p + 4));
+    const float4 f = ld_dep(reinterpret_cast<const float4*>(p));
+    const float4 g = ld_dep(reinterpret_cast<const float4*>(p + 4));
     r.v[0] = f.x; r.v[1] = f.y; r.v[2] = f.z; r.v[3] = f.w;
     r.v[4] = g.x; r.v[5] = g.y; r.v[6] = g.z; r.v[7] = g.w;
   } else if constexpr (CPL == 4) {
-    const float4 f = __ldg(reinterpret_cast<const float4*>(p));
+    const float4 f = ld_dep(reinterpret_cast<const float4*>(p));
     r.v[0] = f.x; r.v[1] = f.y; r.v[2] = f.z; r.v[3] = f.w;
   } else if constexpr (CPL == 2) {
-    const float2 f = __ldg(reinterpret_cast<const float2*>(p));
+    const float2 f = ld_dep(reinterpret_cast<const float2*>(p));
     r.v[0] = f.x; r.v[1] = f.y;
   } else {
 #pragma unroll
-    for (int i = 0; i < CPL; ++i) r.v[i] = __ldg(p + i);
+    for (int i = 0; i < CPL; ++i) r.v[i] = ld_dep(p + i);
   }
   return r;
 }
@@ -596,7 +594,7 @@ template <int CPL>
 __device__ __forceinline__ Cols<CPL> ld_cols(const __nv_bfloat16* p) {
   Cols<CPL> r;
   if constexpr (CPL == 8) {
-    const uint4 u = __ldg(reinterpret_cast<const uint4*>(p));
+    const uint4 u = ld_dep(reinterpret_cast<const uint4*>(p));
     const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -604,15 +602,15 @@ __device__ __forceinline__ Cols<CPL> ld_cols(const __nv_bfloat16* p) {
       r.v[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
     }
   } else if constexpr (CPL == 4) {
-    const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+    const uint2 u = ld_dep(reinterpret_cast<const uint2*>(p));
     r.v[0] = __uint_as_float(u.x << 16); r.v[1] = __uint_as_float(u.x & 0xFFFF0000u);
     r.v[2] = __uint_as_float(u.y << 16); r.v[3] = __uint_as_float(u.y & 0xFFFF0000u);
   } else if constexpr (CPL == 2) {
-    const uint32_t u = __ldg(reinterpret_cast<const unsigned int*>(p));
+    const uint32_t u = ld_dep(reinterpret_cast<const unsigned int*>(p));
     r.v[0] = __uint_as_float(u << 16); r.v[1] = __uint_as_float(u & 0xFFFF0000u);
   } else {
 #pragma unroll
-    for (int i = 0; i < CPL; ++i) r.v[i] = __bfloat162float(p[i]);
+    for (int i = 0; i < CPL; ++i) r.v[i] = __bfloat162float(ld_dep(p + i));
   }
   return r;
 }
@@ -625,13 +623,13 @@ template <int CPL>
 __device__ __forceinline__ RawB<CPL> ld_raw(const __nv_bfloat16* p) {
   RawB<CPL> r;
   if constexpr (CPL == 4) {
-    const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+    const uint2 u = ld_dep(reinterpret_cast<const uint2*>(p));
     r.w[0] = u.x;
     r.w[1] = u.y;
   } else if constexpr (CPL == 2) {
-    r.w[0] = __ldg(reinterpret_cast<const unsigned int*>(p));
+    r.w[0] = ld_dep(reinterpret_cast<const unsigned int*>(p));
   } else {
-    r.w[0] = (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(p));
+    r.w[0] = (uint32_t)ld_dep(reinterpret_cast<const unsigned short*>(p));
   }
   return r;
 }
@@ -684,8 +682,8 @@ __device__ __forceinline__ void add_cols(Cols<CPL>& a, const Cols<CPL>& b) {
 
 template <typename TH, typename TZ, int D, bool SPLIT, int CPL>
 __global__ void __launch_bounds__(WT_WARPS * 32, (sizeof(TH) == 2 && CPL >= 4 && D <= 2) ? 3 : 2)
-k_swiglu_warp(const float* __restrict__ topk_w, const int* __restrict__ node_row, int T, int k,
-              const TH* __restrict__ h, int I, TZ* __restrict__ z, int cols_per_item,
+k_swiglu_warp(const float* topk_w, const int* node_row, int T, int k, const TH* h, int I,
+              TZ* __restrict__ z, int cols_per_item,
               const SplitParts hs) {
   extern __shared__ float zsm[];  // bf16 path: [warp][k slots][32 lanes * CPL] activations
   __shared__ WarpRows wrs[WT_WARPS];
@@ -696,13 +694,14 @@ k_swiglu_warp(const float* __restrict__ topk_w, const int* __restrict__ node_row
   const long items = (long)T * per_tok;
   long it = (long)blockIdx.x * WT_WARPS + warp;
   // The routing tables (node rows, gates) come from the routing and bucketing
-  // kernels, at least two launches before this one: the first item's rows are
-  // found before the wait for the preceding kernel (a small batch has one item a
-  // warp, and the search is a chain of shuffles).
+  // kernels, and the x-side products between them and this launch trigger only after
+  // their wait for the bucketing: the first item's rows are found before the wait
+  // for the preceding kernel (a small batch has one item a warp, and the search is
+  // a chain of shuffles).
   if (it < items) {
     const int t = (int)(it / per_tok);
-    warp_token_rows(lane < kD ? node_row[(size_t)t * kD + lane] : -1, kD, D, wr);
-    if (lane < k) wr.g[lane] = topk_w[(size_t)t * k + lane];
+    warp_token_rows(lane < kD ? ld_dep(node_row + (size_t)t * kD + lane) : -1, kD, D, wr);
+    if (lane < k) wr.g[lane] = ld_dep(topk_w + (size_t)t * k + lane);
     __syncwarp();
   }
   pdl_wait();
@@ -711,8 +710,8 @@ k_swiglu_warp(const float* __restrict__ topk_w, const int* __restrict__ node_row
     const int c_begin = (int)(it % per_tok) * cols_per_item;
     const int c_end = min(I, c_begin + cols_per_item);
     if (!first) {
-      warp_token_rows(lane < kD ? node_row[(size_t)t * kD + lane] : -1, kD, D, wr);
-      if (lane < k) wr.g[lane] = topk_w[(size_t)t * k + lane];
+      warp_token_rows(lane < kD ? ld_dep(node_row + (size_t)t * kD + lane) : -1, kD, D, wr);
+      if (lane < k) wr.g[lane] = ld_dep(topk_w + (size_t)t * k + lane);
       __syncwarp();
     }
     const int nd = wr.nd;
@@ -858,8 +857,8 @@ k_swiglu_warp(const float* __restrict__ topk_w, const int* __restrict__ node_row
 // anchor row split into K ranges contributes its partials in split order)
 template <typename TP, typename TY, int CPL, bool SPLIT>
 __global__ void __launch_bounds__(WT_WARPS * 32, 2)
-k_combine_warp(const int* __restrict__ node_row, int k, int D, const TP* __restrict__ ypart,
-               int H, TY* __restrict__ y, int T, int cols_per_item, const SplitParts ys) {
+k_combine_warp(const int* node_row, int k, int D, const TP* ypart, int H, TY* __restrict__ y,
+               int T, int cols_per_item, const SplitParts ys) {
   __shared__ WarpRows wrs[WT_WARPS];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   WarpRows& wr = wrs[warp];
@@ -867,16 +866,17 @@ k_combine_warp(const int* __restrict__ node_row, int k, int D, const TP* __restr
   const int per_tok = (H + cols_per_item - 1) / cols_per_item;
   const long items = (long)T * per_tok;
   long it = (long)blockIdx.x * WT_WARPS + warp;
-  // node rows come from the bucketing, several launches before this one: the
-  // first item's rows are found before the wait for the preceding kernel
+  // node rows come from the bucketing, and the x-side products in between trigger
+  // only after their wait for it: the first item's rows are found before the wait
+  // for the preceding kernel
   if (it < items)
-    warp_token_rows(lane < kD ? node_row[(size_t)(it / per_tok) * kD + lane] : -1, kD, D, wr);
+    warp_token_rows(lane < kD ? ld_dep(node_row + (size_t)(it / per_tok) * kD + lane) : -1, kD, D, wr);
   pdl_wait();
   for (bool first = true; it < items; it += (long)gridDim.x * WT_WARPS, first = false) {
     const int t = (int)(it / per_tok);
     const int c_begin = (int)(it % per_tok) * cols_per_item;
     const int c_end = min(H, c_begin + cols_per_item);
-    if (!first) warp_token_rows(lane < kD ? node_row[(size_t)t * kD + lane] : -1, kD, D, wr);
+    if (!first) warp_token_rows(lane < kD ? ld_dep(node_row + (size_t)t * kD + lane) : -1, kD, D, wr);
     const int nd = wr.nd;
     for (int c = c_begin + CPL * lane; c < c_end; c += 32 * CPL) {
       Cols<CPL> acc;
@@ -960,11 +960,12 @@ __device__ __forceinline__ uint32_t pack2(float2 v) {
 
 // y[t] = sum of ypart over t's listed rows in ascending row order
 __global__ void __launch_bounds__(256, 6)
-k_combine_tok(const int* __restrict__ trow, int max_rows, const __nv_bfloat16* __restrict__ ypart, int H,
+k_combine_tok(const int* trow, int max_rows, const __nv_bfloat16* ypart, int H,
               __nv_bfloat16* __restrict__ y) {
   const int4* rows = reinterpret_cast<const int4*>(trow + (size_t)blockIdx.x * TOK_ROWS);
-  // (the list comes from the bucketing, several launches before this one)
-  int4 r = __ldg(rows);
+  // (the list comes from the bucketing, and tc_up_anchor in between triggers only
+  // after its wait for it)
+  int4 r = ld_dep(rows);
   pdl_wait();
   for (int c = 8 * threadIdx.x; c < H; c += 8 * blockDim.x) {
     float2 acc[4];
@@ -976,8 +977,8 @@ k_combine_tok(const int* __restrict__ trow, int max_rows, const __nv_bfloat16* _
       uint4 v[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u)
-        if (rr[u] >= 0) v[u] = *reinterpret_cast<const uint4*>(ypart + (size_t)rr[u] * H + c);
-      if (d + 4 < max_rows) q = __ldg(rows + d / 4 + 1);
+        if (rr[u] >= 0) v[u] = ld_dep(reinterpret_cast<const uint4*>(ypart + (size_t)rr[u] * H + c));
+      if (d + 4 < max_rows) q = ld_dep(rows + d / 4 + 1);
 #pragma unroll
       for (int u = 0; u < 4; ++u)
         if (rr[u] >= 0) {
@@ -996,13 +997,12 @@ k_combine_tok(const int* __restrict__ trow, int max_rows, const __nv_bfloat16* _
 // gate and up values are loaded once (six rows in flight) and added to the slots
 // whose path holds the row, rows ascending; then the acts, then the rows' z.
 __global__ void __launch_bounds__(256, 2)
-k_swiglu_tok(const float* __restrict__ topk_w, const int* __restrict__ trow,
-             const uint8_t* __restrict__ tmask, int k, const __nv_bfloat16* __restrict__ h, int I,
-             __nv_bfloat16* __restrict__ z) {
+k_swiglu_tok(const float* topk_w, const int* trow, const uint8_t* tmask, int k, const __nv_bfloat16* h,
+             int I, __nv_bfloat16* __restrict__ z) {
   __shared__ int srow[TOK_ROWS], smask[TOK_ROWS];
   __shared__ float sg[WT_SLOTS];
   const int t = blockIdx.x, tid = threadIdx.x;
-  if (tid < TOK_ROWS) {
+  if (tid < TOK_ROWS) {  // (ahead of the wait: as in k_combine_tok)
     srow[tid] = trow[(size_t)t * TOK_ROWS + tid];
     smask[tid] = tmask[(size_t)t * TOK_ROWS + tid];
     if (tid < WT_SLOTS) sg[tid] = tid < k ? topk_w[(size_t)t * k + tid] : 0.f;
@@ -1020,8 +1020,8 @@ k_swiglu_tok(const float* __restrict__ topk_w, const int* __restrict__ trow,
       for (int q = 0; q < U; ++q)
         if (d0 + q < nd) {
           const __nv_bfloat16* hp = h + (size_t)srow[d0 + q] * 2 * I + c;
-          g[q] = *reinterpret_cast<const uint2*>(hp);
-          u[q] = *reinterpret_cast<const uint2*>(hp + I);
+          g[q] = ld_dep(reinterpret_cast<const uint2*>(hp));
+          u[q] = ld_dep(reinterpret_cast<const uint2*>(hp + I));
         }
 #pragma unroll
       for (int q = 0; q < U; ++q) {
@@ -1194,7 +1194,7 @@ lx_status launch_swiglu(lx_layer* L, int T, int k, bool bf16, cudaStream_t s, Sp
   const size_t smem = sizeof(float4) * SW_T * k * L->max_depth;
   static bool done_f[64] = {};
   LX_CUDA(smem_cap_once((const void*)k_swiglu_aggregate<float>, 200 * 1024, L->device, done_f));
-  launch_k(L, k_swiglu_aggregate<float>, grid, SW_T, smem, s, w.topk_id, w.topk_w, w.node_row, T,
+  launch_k(L, k_swiglu_aggregate<float>, grid, SW_T, smem, s, w.topk_w, w.node_row, T,
            k, L->max_depth, w.h, L->I, w.z);
   LX_CUDA(cudaGetLastError());
   return LX_OK;

@@ -426,12 +426,24 @@ inline cudaError_t smem_cap_once(const void* func, int bytes, int device, bool (
   return e;
 }
 
-// Kernel launch with programmatic dependent launch: the next kernel of the
-// stream may be scheduled while this one drains, and every kernel of the
-// library starts with griddepcontrol.wait (pdl_wait), which returns once its
-// predecessor has completed and its writes are visible.  Off while profiling,
-// so that the per-kernel events time one kernel each.  Launch errors surface
-// through cudaGetLastError at the call site.
+// Kernel launch with programmatic dependent launch: a kernel of the stream may
+// start once every CTA of its predecessor has let it (griddepcontrol.
+// launch_dependents, here "trigger") or ended.  Every launch passes
+// griddepcontrol.wait before it ends, which returns once its predecessor has
+// completed and its writes are visible, so launches complete in order.  Most
+// kernels wait first of all and trigger then (pdl_wait); some trigger at their
+// start and wait only where they need the predecessor's output.
+//   Before its own wait a kernel may read the layer's constants, and what a
+// launch W wrote if some launch between the two triggers only after its own wait:
+// this kernel cannot have started before that trigger, and by then W was complete.
+// A launch that triggers at its start does not count, however many of them lie in
+// between.
+//   What an earlier launch wrote is never read through the read-only path (__ldg,
+// or a const __restrict__ parameter of a kernel launched so): the compiler may move
+// such a load above the wait.  Those parameters are plain pointers, read with ld_dep
+// where the order of the loads against other stores matters.
+//   Off while profiling, so that the per-kernel events time one kernel each.
+// Launch errors surface through cudaGetLastError at the call site.
 template <typename... KArgs, typename... Args>
 inline void launch_k(const lx_layer* L, void (*kern)(KArgs...), dim3 grid, dim3 block,
                      size_t smem, cudaStream_t s, Args... args) {
@@ -453,6 +465,28 @@ inline void launch_k(const lx_layer* L, void (*kern)(KArgs...), dim3 grid, dim3 
 __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// A load of what an earlier launch wrote: stays behind the wait above it (volatile
+// asm statements keep their order) but is free to move across ordinary stores.
+template <typename T>
+__device__ __forceinline__ T ld_dep(const T* p) {
+  static_assert(sizeof(T) == 2 || sizeof(T) == 4 || sizeof(T) == 8 || sizeof(T) == 16, "one load");
+  union {
+    T v;
+    unsigned short h;
+    uint32_t w[sizeof(T) >= 4 ? sizeof(T) / 4 : 1];
+  } u;
+  const size_t a = __cvta_generic_to_global(p);
+  if constexpr (sizeof(T) == 2) asm volatile("ld.global.u16 %0, [%1];" : "=h"(u.h) : "l"(a));
+  else if constexpr (sizeof(T) == 4) asm volatile("ld.global.u32 %0, [%1];" : "=r"(u.w[0]) : "l"(a));
+  else if constexpr (sizeof(T) == 8)
+    asm volatile("ld.global.v2.u32 {%0,%1}, [%2];" : "=r"(u.w[0]), "=r"(u.w[1]) : "l"(a));
+  else
+    asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(u.w[0]), "=r"(u.w[1]), "=r"(u.w[2]), "=r"(u.w[3])
+                 : "l"(a));
+  return u.v;
 }
 
 // Launch-time timing helper: records events around a launch when profiling.

@@ -82,7 +82,7 @@ __device__ __forceinline__ void load8<__nv_bfloat16>(const __nv_bfloat16* p, flo
 
 template <typename T>
 __global__ void __launch_bounds__(RT_THREADS)
-k_router_logits(const T* __restrict__ x, const T* __restrict__ W, const float* __restrict__ bias,
+k_router_logits(const T* x, const T* __restrict__ W, const float* __restrict__ bias,
                 int Ttok, int E, int H, int experts_per_cta, float* __restrict__ logits,
                 int* __restrict__ tile_cnt, int k, int* __restrict__ topk_id,
                 float* __restrict__ topk_w) {
@@ -242,7 +242,7 @@ __device__ __forceinline__ void rtt_load_tile(const __nv_bfloat16* x, int t0, in
 }
 
 __global__ void __launch_bounds__(RTT_THREADS, 1)
-k_router_tiled(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ W,
+k_router_tiled(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ W,
                const float* __restrict__ bias, int Ttok, int E, int H,
                float* __restrict__ logits, int k, int* __restrict__ topk_id,
                float* __restrict__ topk_w) {
@@ -399,8 +399,7 @@ constexpr int RS_WARPS = 8;
 // 50 and 67 us at 8192 tokens (the loads do not bound it).
 template <int EPL, int U>
 __global__ void __launch_bounds__(RS_WARPS * 32, U == 8 ? 3 : 4)
-k_router_screen(const float* __restrict__ part, int splits, int Epad,
-                const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ W,
+k_router_screen(const float* part, int splits, int Epad, const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ W,
                 const float* __restrict__ bias, int T, int E, int H, float wmax, int k,
                 int* __restrict__ topk_id, float* __restrict__ topk_w) {
   extern __shared__ __align__(16) unsigned char smem[];
