@@ -245,13 +245,19 @@ LX_API lx_status lx_read_profile(lx_layer* layer, lx_kernel_time* out, int32_t c
  * `site` waits for a condition that nothing fulfils -- LX_WAIT_STREAM_DEP: one
  * arrival more than the streaming producer tiles make; LX_WAIT_TC_MMA: a
  * barrier that only the abort path arrives on, before the tensor-core MMA
- * issuer's first tile -- so that it runs out after the bound.  LX_WAIT_NONE
+ * issuer's first tile; LX_WAIT_ROUTER: the same in the screened route's product
+ * (bf16, larger batches) -- so that it runs out after the bound.  LX_WAIT_NONE
  * turns the hook off.  Errors: LX_ERR_ARG (NULL layer, unknown site).
  *
  * lx_clear_device_error: zeroes the device error word (stream-ordered on the
  * legacy default stream; synchronises the device).  Errors: LX_ERR_ARG.
  */
-typedef enum { LX_WAIT_NONE = 0, LX_WAIT_STREAM_DEP = 1, LX_WAIT_TC_MMA = 2 } lx_wait_site;
+typedef enum {
+  LX_WAIT_NONE = 0,
+  LX_WAIT_STREAM_DEP = 1,
+  LX_WAIT_TC_MMA = 2,
+  LX_WAIT_ROUTER = 3
+} lx_wait_site;
 LX_API lx_status lx_set_wait_limit(lx_layer* layer, uint64_t cycles);
 LX_API lx_status lx_inject_unmet_wait(lx_layer* layer, int32_t site);
 LX_API lx_status lx_clear_device_error(lx_layer* layer);

@@ -834,7 +834,8 @@ extern "C" lx_status lx_set_wait_limit(lx_layer* L, uint64_t cycles) {
 
 extern "C" lx_status lx_inject_unmet_wait(lx_layer* L, int32_t site) {
   if (!L) return fail(LX_ERR_ARG, "layer is NULL");
-  if (site != LX_WAIT_NONE && site != LX_WAIT_STREAM_DEP && site != LX_WAIT_TC_MMA)
+  if (site != LX_WAIT_NONE && site != LX_WAIT_STREAM_DEP && site != LX_WAIT_TC_MMA &&
+      site != LX_WAIT_ROUTER)
     return fail(LX_ERR_ARG, "unknown wait site");
   L->unmet_wait = site;
   return LX_OK;

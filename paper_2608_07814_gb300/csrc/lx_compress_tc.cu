@@ -41,6 +41,8 @@ struct ResLaunch {
   int M, Npad, kb_seg, kb_split, n_kb;  // 64-wide K blocks: per segment, per CTA, in all
   float* part;        // [gridDim.z][splits][M][Npad]: blockIdx.z takes B rows z Npad ..
   unsigned long long wait_cycles;
+  int* err;           // error word (LX_ERR_TIMEOUT on a wait that gave up), or null
+  int unmet;          // test hook: the MMA issuer first waits for what nothing fulfils
 };
 
 __global__ void __launch_bounds__(RM_THREADS, 1) k_res_mma(const __grid_constant__ ResLaunch P) {
@@ -101,8 +103,8 @@ __global__ void __launch_bounds__(RM_THREADS, 1) k_res_mma(const __grid_constant
   } else if (warp == 1) {
     if (lane == 0) {
       const uint32_t idesc = instr_desc(RM_BM, P.Npad);
-      bool ok = true;
-      for (int i = 0; i < nkb; ++i) {
+      bool ok = !P.unmet || mbar_wait(done, 0, abort_flag, P.wait_cycles);
+      for (int i = 0; ok && i < nkb; ++i) {
         const uint32_t s = i % RM_STAGES;
         if (!mbar_wait(full0 + 8 * s, (i / RM_STAGES) & 1, abort_flag, P.wait_cycles)) {
           ok = false;
@@ -126,7 +128,13 @@ __global__ void __launch_bounds__(RM_THREADS, 1) k_res_mma(const __grid_constant
     // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 (tile rows)
     const int q = warp & 3;
     int ok = 1;
-    if (lane == 0) ok = (mbar_wait(done, 0, abort_flag, P.wait_cycles) && !*abort_flag) ? 1 : 0;
+    if (lane == 0) {
+      // (an aborted issuer commits `done` too: only then is its TMEM idle.  It may
+      // have waited for the bound by then, so this wait has twice that.)
+      ok = mbar_wait(done, 0, nullptr, 2 * P.wait_cycles) ? 1 : 0;
+      if (!ok) *abort_flag = 1;
+      else if (*abort_flag) ok = 0;
+    }
     ok = __shfl_sync(0xffffffffu, ok, 0);  // warp-uniform: the TMEM loads are warp-wide
     __syncwarp();
     tc_fence_after();
@@ -163,6 +171,7 @@ __global__ void __launch_bounds__(RM_THREADS, 1) k_res_mma(const __grid_constant
   }
   tc_fence_before();
   __syncthreads();
+  if (threadIdx.x == RM_THREADS - 1 && P.err && *abort_flag) atomicExch(P.err, LX_ERR_TIMEOUT);
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256)
@@ -335,6 +344,8 @@ lx_status tc_splitk_gemm(lx_layer* L, const CUtensorMap& a, const CUtensorMap& b
   splits = (P.n_kb + P.kb_split - 1) / P.kb_split;
   P.part = part;
   P.wait_cycles = wait_limit(L);
+  P.err = L->ws.err;
+  P.unmet = L->unmet_wait == LX_WAIT_ROUTER;
   const int b_bytes = Npad * 64 * 2;
   const int smem = RM_STAGES * (RM_A_BYTES + ((b_bytes + 1023) & ~1023)) + 8 * (2 * RM_STAGES + 3) + 1024;
   LX_CUDA(smem_cap_once((const void*)k_res_mma, 227 * 1024, L->device, g_rm_cap));

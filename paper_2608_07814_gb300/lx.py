@@ -33,7 +33,7 @@ EXPORTS = [
     "lx_compress_workspace", "lx_compress_factor", "lx_set_wait_limit", "lx_inject_unmet_wait",
     "lx_clear_device_error",
 ]
-LX_WAIT_NONE, LX_WAIT_STREAM_DEP, LX_WAIT_TC_MMA = 0, 1, 2
+LX_WAIT_NONE, LX_WAIT_STREAM_DEP, LX_WAIT_TC_MMA, LX_WAIT_ROUTER = range(4)
 LX_NOALLOC_SCRATCH_BYTES = 16 << 20
 
 
