@@ -256,11 +256,25 @@ typedef enum {
   LX_WAIT_NONE = 0,
   LX_WAIT_STREAM_DEP = 1,
   LX_WAIT_TC_MMA = 2,
-  LX_WAIT_ROUTER = 3
+  LX_WAIT_ROUTER = 3,
+  LX_WAIT_CALL_PRODUCT = 4,
+  LX_WAIT_CALL_JACOBI = 5
 } lx_wait_site;
 LX_API lx_status lx_set_wait_limit(lx_layer* layer, uint64_t cycles);
 LX_API lx_status lx_inject_unmet_wait(lx_layer* layer, int32_t site);
 LX_API lx_status lx_clear_device_error(lx_layer* layer);
+
+/*
+ * The calls without a layer (lx_compress_factor, lx_align_cost) have bounded waits
+ * too (default bound), and no error word of a layer: when one gives up, every value
+ * that the call writes is NaN.
+ * lx_inject_unmet_wait_call (test hook): in the calling thread's next such call,
+ * waits have the bound `cycles` (0: the default) and the one at `site` runs out --
+ * LX_WAIT_CALL_PRODUCT: in the tensor-core products (bf16; lx_align_cost also needs
+ * d_model a multiple of 256); LX_WAIT_CALL_JACOBI: in lx_compress_factor's Jacobi (l
+ * above 2); LX_WAIT_NONE: none.  Errors: LX_ERR_ARG (another site).
+ */
+LX_API lx_status lx_inject_unmet_wait_call(int32_t site, uint64_t cycles);
 
 /*
  * Size of the fixed device array that lx_bucket_noalloc uses as scratch.  The
@@ -349,8 +363,11 @@ LX_API lx_status lx_coact_npmi(const uint64_t* coact, int32_t E, int64_t n_token
  *   dom_gate, dom_up, mem_gate, mem_up: device [I][H]; dom_down, mem_down:
  *          device [H][I] (row-major, the x W^T storage of lx_load_compressed_layer);
  *   cost:  device [I][I] fp32 out.  Every pointer 16-byte aligned.
- * Stream-ordered; no allocation.  Errors: LX_ERR_ARG (dtype, NULL, alignment),
- * LX_ERR_SHAPE (sizes).
+ * Stream-ordered.  bf16 with d_model a multiple of 256 takes scratch from the
+ * device's stream-ordered memory pool (cudaMallocAsync) and gives it back on the
+ * stream; the other forms allocate nothing.  If a bounded wait of the tensor-core
+ * products gives up, the cost is NaN.  Errors: LX_ERR_ARG (dtype, NULL, alignment),
+ * LX_ERR_SHAPE (sizes), LX_ERR_CUDA (no scratch).
  */
 LX_API lx_status lx_align_cost(int32_t dtype, int32_t d_model, int32_t d_ff,
                                const void* dom_gate, const void* dom_up, const void* dom_down,
@@ -415,8 +432,9 @@ LX_API lx_status lx_permute_neurons(int32_t dtype, int32_t d_model, int32_t d_ff
  * singular values (Rayleigh quotients) are summed in float64.  The sign of each factor column is fixed so that the
  * largest-magnitude entry of U's column is positive.  Singular values at or
  * below 1e-6 of the largest give zero U and V columns.  The call is latency
- * bound (one-CTA stages): independent projections run concurrently when given
- * their own streams and workspaces.
+ * bound (stages of one to eight CTAs): independent projections run concurrently
+ * when given their own streams and workspaces.  If one of its bounded waits gives
+ * up, U, V and s are NaN.
  *   dtype:      LX_F32 or LX_BF16 of w_dom / w_mem
  *   rows, cols: the projection's [out][in] shape, multiples of 8 (gate / up:
  *               [I][H], down: [H][I]); w_dom, w_mem device, 16-byte aligned

@@ -320,11 +320,13 @@ struct AlignPackArgs {
   const __nv_bfloat16* d[2];
   __nv_bfloat16* cat[2];
   float* npart[2];  // [H / AP_HB][I]
+  int* err;         // the call's error word, zeroed here
 };
 __global__ void __launch_bounds__(256) k_align_pack(const AlignPackArgs A, int H, int I) {
   __shared__ __align__(16) __nv_bfloat16 blk[AP_HB][34];
   const int x = blockIdx.z, i0 = blockIdx.x * 32, hb = blockIdx.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (blockIdx.x + blockIdx.y + blockIdx.z + threadIdx.x == 0) *A.err = 0;
   const long K = 3L * H;
   const __nv_bfloat16* g = A.g[x];
   const __nv_bfloat16* u = A.u[x];
@@ -401,12 +403,13 @@ __global__ void __launch_bounds__(256) k_align_pack(const AlignPackArgs A, int H
 
 // cost[i][j] = na[i] + nb[j] - 2 sum_s part[z][s][i][j - z Npad], z = j / Npad
 // (the K ranges in ascending order), na / nb the sums of the nhb norm
-// partials [nhb][I] in range order
+// partials [nhb][I] in range order; NaN where a wait of the products gave up (err)
 __global__ void k_align_finish(const float* __restrict__ part, int splits, int I, int Npad,
                                const float* __restrict__ npa, const float* __restrict__ npb,
-                               int nhb, float* __restrict__ cost) {
+                               int nhb, const int* __restrict__ err, float* __restrict__ cost) {
   // four consecutive columns per thread (I and Npad are multiples of 4)
   const long total = (long)I * I / 4;
+  const float bad = *err ? NAN : 0.f;
   for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (long)gridDim.x * blockDim.x) {
     const int i = (int)(4 * e / I), j = (int)(4 * e % I), z = j / Npad, jj = j % Npad;
@@ -427,7 +430,7 @@ __global__ void k_align_finish(const float* __restrict__ part, int splits, int I
       const float4 v = p[sp * st];
       dot.x += v.x; dot.y += v.y; dot.z += v.z; dot.w += v.w;
     }
-    float a = 0.f;
+    float a = bad;
     float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int r = 0; r < nhb; ++r) {
       a += npa[(size_t)r * I + i];
@@ -518,7 +521,7 @@ namespace {
 // stream-ordered allocator (packed operands, norms, split-K partials), freed on
 // the stream after the last kernel.
 lx_status align_cost_tc(int H, int I, const void* dg, const void* du, const void* dd,
-                        const void* mg, const void* mu, const void* md, float* cost,
+                        const void* mg, const void* mu, const void* md, float* cost, CallWaits waits,
                         cudaStream_t s) {
   using B = __nv_bfloat16;
   int dev = 0, sms = 0;
@@ -532,14 +535,16 @@ lx_status align_cost_tc(int H, int I, const void* dg, const void* du, const void
   const size_t b_cat = al((size_t)I * K * 2), b_nrm = al((size_t)nhb * I * 4);
   const size_t b_part = al((size_t)nz * RES_TC_MAX_SPLITS * I * Npad * 4);
   char* ws = nullptr;
-  LX_CUDA(cudaMallocAsync((void**)&ws, 2 * b_cat + 2 * b_nrm + b_part, s));
+  LX_CUDA(cudaMallocAsync((void**)&ws, 2 * b_cat + 2 * b_nrm + b_part + 256, s));
   B* A = reinterpret_cast<B*>(ws);
   B* Bm = reinterpret_cast<B*>(ws + b_cat);
   float* na = reinterpret_cast<float*>(ws + 2 * b_cat);
   float* nb = reinterpret_cast<float*>(ws + 2 * b_cat + b_nrm);
   float* part = reinterpret_cast<float*>(ws + 2 * b_cat + 2 * b_nrm);
+  waits.err = reinterpret_cast<int*>(ws + 2 * b_cat + 2 * b_nrm + b_part);
   lx_status st = LX_OK;
   AlignPackArgs pa;
+  pa.err = waits.err;
   pa.g[0] = static_cast<const B*>(dg);
   pa.u[0] = static_cast<const B*>(du);
   pa.d[0] = static_cast<const B*>(dd);
@@ -560,12 +565,12 @@ lx_status align_cost_tc(int H, int I, const void* dg, const void* du, const void
     st = fail(LX_ERR_CUDA, "cuTensorMapEncodeTiled(alignment operands) failed");
   int splits = 1;
   if (st == LX_OK)
-    st = tc_splitk_gemm_chunks(ma, mb, I, Npad, nz, (int)K, part, RES_TC_MAX_SPLITS, &splits, sms,
+    st = tc_splitk_gemm_chunks(ma, mb, I, Npad, nz, (int)K, part, RES_TC_MAX_SPLITS, &splits, waits, sms,
                                dev, s);
   if (st == LX_OK) {
     const long total = (long)I * I;
     k_align_finish<<<(unsigned)std::min<long>((total / 4 + 255) / 256, 8L * sms), 256, 0, s>>>(
-        part, splits, I, Npad, na, nb, nhb, cost);
+        part, splits, I, Npad, na, nb, nhb, waits.err, cost);
     e = cudaGetLastError();
     if (e != cudaSuccess) st = cuda_fail(e, "alignment cost");
   }
@@ -588,11 +593,12 @@ extern "C" lx_status lx_align_cost(int32_t dtype, int32_t d_model, int32_t d_ff,
     if (!p) return fail(LX_ERR_ARG, "NULL weight or cost pointer");
     if (!aligned16(p)) return fail(LX_ERR_ARG, "weights and cost must be 16-byte aligned");
   }
+  const CallWaits waits = take_call_waits();
   const int H = d_model, I = d_ff;
   const dim3 grid((I + AC_TILE - 1) / AC_TILE, (I + AC_TILE - 1) / AC_TILE);
   cudaStream_t s = (cudaStream_t)stream;
-  if (dtype == LX_BF16 && H % 256 == 0) return align_cost_tc(H, I, dom_gate, dom_up, dom_down,
-                                                            mem_gate, mem_up, mem_down, cost, s);
+  if (dtype == LX_BF16 && H % 256 == 0)
+    return align_cost_tc(H, I, dom_gate, dom_up, dom_down, mem_gate, mem_up, mem_down, cost, waits, s);
   if (dtype == LX_BF16) {
     using B = __nv_bfloat16;
     k_align_cost_mma<<<grid, AM_THREADS, 0, s>>>((const B*)dom_gate, (const B*)dom_up,

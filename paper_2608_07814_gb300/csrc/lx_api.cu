@@ -841,6 +841,24 @@ extern "C" lx_status lx_inject_unmet_wait(lx_layer* L, int32_t site) {
   return LX_OK;
 }
 
+namespace lx {
+static thread_local CallWaits g_call_waits;
+CallWaits take_call_waits() {
+  const CallWaits w = g_call_waits;
+  g_call_waits = CallWaits{};
+  return w;
+}
+}  // namespace lx
+
+extern "C" lx_status lx_inject_unmet_wait_call(int32_t site, uint64_t cycles) {
+  if (site != LX_WAIT_NONE && site != LX_WAIT_CALL_PRODUCT && site != LX_WAIT_CALL_JACOBI)
+    return fail(LX_ERR_ARG, "unknown wait site");
+  lx::g_call_waits = lx::CallWaits{};
+  lx::g_call_waits.unmet = site;
+  if (cycles) lx::g_call_waits.cycles = cycles;
+  return LX_OK;
+}
+
 extern "C" lx_status lx_clear_device_error(lx_layer* L) {
   if (!L) return fail(LX_ERR_ARG, "layer is NULL");
   if (L->ws.base) {

@@ -618,6 +618,11 @@ k_trmm(const float* __restrict__ L1, const float* __restrict__ L2, int L, float*
 // the reduction, the angle, the hop to the neighbour): 0.79 us a round at L = 136,
 // 970 us in all.
 //
+// Every wait is bounded.  A thread whose wait gave up waits no more and its CTA
+// goes on with what the buffers hold, so that the neighbours get their bytes and
+// every CTA reaches the end of the sweep; the CTAs then read one another's flags and
+// all leave there, with LX_ERR_TIMEOUT in the call's error word.
+//
 // Which entries of a column a lane sums: up to 144 columns, entries 16 v + 2 u,
 // + 1 (lane u, v = 0, 1, ...); above, u, u + 8, u + 16, ...; both ascending.
 // Output: Wt [L][L], Wt[j][k] = W[k][j].
@@ -625,6 +630,8 @@ constexpr int OS_MAX_SWEEPS = 30;
 constexpr int OS_P = 8;        // CTAs of the cluster
 constexpr int OS_LANES = 16;   // of a pair: eight for M, eight for W
 constexpr int OS_MAX_PAIRS = 16;  // a CTA's at L = 256
+constexpr unsigned OS_ROTATED = 1, OS_GAVE_UP = 2;  // flags of a CTA's sweep
+constexpr long long OS_LAND_CYCLES = 1 << 20;  // half a millisecond, for bytes in flight to land
 // floats of a column's part (M or W, NV pairs of entries a lane): the parts of a
 // column 16 mod 32 words apart, so that a pair's 16 lanes touch distinct banks
 __host__ __device__ constexpr int os_part(int nv) { return 16 * nv + (nv % 2 == 0 ? 16 : 0); }
@@ -645,7 +652,7 @@ __device__ __forceinline__ void os_cluster_sync() {
 }
 // bounded wait for a phase of this CTA's mbarrier (its bytes were sent by
 // CTAs that are resident beside it, so it ends)
-__device__ __forceinline__ bool os_wait(uint32_t bar, uint32_t parity) {
+__device__ __forceinline__ bool os_wait(uint32_t bar, uint32_t parity, unsigned long long limit) {
   const unsigned long long t0 = clock64();
   while (true) {
     uint32_t ok;
@@ -657,7 +664,7 @@ __device__ __forceinline__ bool os_wait(uint32_t bar, uint32_t parity) {
         : "r"(bar), "r"(parity)
         : "memory");
     if (ok) return true;
-    if (clock64() - t0 > kDefaultWaitCycles) return false;
+    if (clock64() - t0 > limit) return false;
   }
 }
 __device__ __forceinline__ float2 os_mul2(float2 a, float2 b) {
@@ -718,11 +725,11 @@ __device__ __forceinline__ bool os_rotate(float2 (&x)[NV], float2 (&y)[NV], bool
 
 template <int NV>
 __global__ void __launch_bounds__(OS_LANES * OS_MAX_PAIRS)
-k_jacobi_cluster(const float* __restrict__ Mt, int L, float* __restrict__ Wt) {
+k_jacobi_cluster(const float* __restrict__ Mt, int L, float* __restrict__ Wt, const CallWaits waits) {
   constexpr int PART = os_part(NV), COL = 2 * PART;  // floats of a column's part and of a column
   extern __shared__ __align__(128) float osm[];  // [2 buffers][first, second columns][nmax][COL]
   __shared__ __align__(8) uint64_t s_full[2];    // by buffer: the neighbours' columns have landed
-  __shared__ unsigned s_rot[2];                  // by sweep parity: a pair of this CTA was rotated
+  __shared__ unsigned s_rot[2];                  // by sweep parity: this CTA's flags
   __shared__ unsigned s_go;
   const int tid = threadIdx.x, lane16 = tid & (OS_LANES - 1), u = lane16 & 7, i = tid / OS_LANES;
   uint32_t rank_u;
@@ -759,9 +766,10 @@ k_jacobi_cluster(const float* __restrict__ Mt, int L, float* __restrict__ Wt) {
     }
   }
   // the bytes of the neighbours' columns that arrive for each round
-  const uint32_t incoming =
-      (uint32_t)(n == 0 ? 0 : (rank > 0) + (rank < busy - 1)) * (uint32_t)(OS_LANES * NV * 8);
+  uint32_t incoming = (uint32_t)(n == 0 ? 0 : (rank > 0) + (rank < busy - 1)) * (uint32_t)(OS_LANES * NV * 8);
   const bool listens = on && incoming && (i == 0 || i == n - 1);
+  // (test hook: the first CTA waits for bytes that nobody sends)
+  if (waits.unmet == LX_WAIT_CALL_JACOBI && rank == 0 && incoming) incoming += 16;
   if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full0) : "memory");
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full0 + 8) : "memory");
@@ -794,11 +802,11 @@ k_jacobi_cluster(const float* __restrict__ Mt, int L, float* __restrict__ Wt) {
     for (int rd = 0; rd < Lp - 1; ++rd, ++k) {
       if (n == 0) continue;
       const uint32_t cur = k & 1, nxt = cur ^ 1;
-      if (tid == 0 && incoming)
+      if (tid == 0 && incoming && alive)  // (thread 0 listens: the phase before is over)
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(full0 + 8 * nxt),
                      "r"(incoming)
                      : "memory");
-      if (listens && k > 0 && alive) alive = os_wait(full0 + 8 * cur, ((k - 1) >> 1) & 1);
+      if (listens && k > 0 && alive) alive = os_wait(full0 + 8 * cur, ((k - 1) >> 1) & 1, waits.cycles);
       __syncwarp();
       float2 x[NV], y[NV];
       const char* B = reinterpret_cast<const char*>(osm) + cur * buf_bytes;
@@ -831,7 +839,7 @@ k_jacobi_cluster(const float* __restrict__ Mt, int L, float* __restrict__ Wt) {
       }
       __syncthreads();
     }
-    if (rotated) s_rot[sweep & 1] = 1;
+    if (rotated || !alive) atomicOr(&s_rot[sweep & 1], (rotated ? OS_ROTATED : 0u) | (alive ? 0u : OS_GAVE_UP));
     // every CTA reads the same flags, so all leave after the same sweep
     __syncthreads();
     os_cluster_sync();
@@ -842,10 +850,17 @@ k_jacobi_cluster(const float* __restrict__ Mt, int L, float* __restrict__ Wt) {
       s_rot[(sweep + 1) & 1] = 0;  // last read a sweep ago
     }
     __syncthreads();
-    if (!s_go || sweep + 1 == OS_MAX_SWEEPS) break;
+    if (s_go & OS_GAVE_UP) alive = false;  // the same in every CTA
+    if (s_go != OS_ROTATED || sweep + 1 == OS_MAX_SWEEPS) break;
   }
   // a sweep's rounds bring every column back to where it began
-  if (listens && alive) alive = os_wait(full0 + 8 * (k & 1), ((k - 1) >> 1) & 1);
+  if (listens && alive) alive = os_wait(full0 + 8 * (k & 1), ((k - 1) >> 1) & 1, waits.cycles);
+  if (!alive) {
+    atomicExch(waits.err, LX_ERR_TIMEOUT);
+    const long long t0 = clock64();
+    while (clock64() - t0 < OS_LAND_CYCLES) {
+    }
+  }
   if (on && lane16 >= 8) {
     const char* B = reinterpret_cast<const char*>(osm) + (k & 1) * buf_bytes;
 #pragma unroll
@@ -862,7 +877,7 @@ k_jacobi_cluster(const float* __restrict__ Mt, int L, float* __restrict__ Wt) {
     }
   }
   __syncwarp();
-  os_cluster_sync();  // no CTA leaves while its flags are read
+  os_cluster_sync();  // no CTA leaves while its flags are read or bytes for it are in flight
 }
 
 // CTA j: v = M w_j in float64, sigma_j = |v| / |w_j| (the Rayleigh quotient of
@@ -923,14 +938,22 @@ k_ritz(const float* __restrict__ Mt, const float* __restrict__ Wt, int L, float*
 // and Z2 Wv = V_r S_r^(1/2) (Eq. factors); CTA 0 writes sig [r] fp32.  Every CTA
 // ranks the sigma for itself (non-negative float64 values compare as their
 // bits do), so that no single CTA takes the L r square roots and divisions:
-// 87 us with one CTA, 6.7 us now at L = 136, r = 128.
+// 87 us with one CTA, 6.7 us now at L = 136, r = 128.  All NaN if a wait of the
+// call gave up (err), so that the caller sees it in every factor.
 __global__ void __launch_bounds__(256)
 k_finish(const double* __restrict__ sig64, const float* __restrict__ MWn,
-         const float* __restrict__ Wn, int L, int r, float* __restrict__ Wu,
-         float* __restrict__ Wv, float* __restrict__ sig) {
+         const float* __restrict__ Wn, int L, int r, const int* __restrict__ err,
+         float* __restrict__ Wu, float* __restrict__ Wv, float* __restrict__ sig) {
   __shared__ double sv[256];
   __shared__ int order[256];
   const int tid = threadIdx.x, k = blockIdx.x;
+  if (*err) {
+    if (tid < r) {
+      Wu[(size_t)k * r + tid] = Wv[(size_t)k * r + tid] = NAN;
+      if (k == 0) sig[tid] = NAN;
+    }
+    return;
+  }
   if (tid < L) sv[tid] = sig64[tid];
   __syncthreads();
   if (tid < L) {
@@ -1017,6 +1040,7 @@ size_t al256(size_t v) { return (v + 255) / 256 * 256; }
 struct CompressWs {
   float *y0, *y1, *z0, *z1, *Dinv, *T, *Wu, *Wv, *L1, *L2, *Mt, *Wt, *MWn, *Wn;
   double* sig64;
+  int* err;  // LX_ERR_TIMEOUT if a wait of the call gave up
   char* tc;  // the tensor-core residual products' scratch (bf16 weights)
   size_t bytes;
 };
@@ -1046,6 +1070,7 @@ CompressWs carve(char* base, long rows, long cols, long l, long r) {
   w.MWn = (float*)take(4 * l * l);
   w.Wn = (float*)take(4 * l * l);
   w.sig64 = (double*)take(8 * l);
+  w.err = (int*)take(4);
   w.tc = take(res_tc_workspace(rows, cols, l));
   w.bytes = off;
   return w;
@@ -1062,13 +1087,15 @@ lx_status check_compress(int32_t rows, int32_t cols, int32_t l, int32_t r) {
 template <typename TW>
 lx_status run_compress(int rows, int cols, const TW* Wd, const TW* Wm, const float* omega, int l,
                        int r, int q, float* U, float* V, float* sigma, const CompressWs& w,
-                       int dev, cudaStream_t s) {
+                       CallWaits waits, int dev, cudaStream_t s) {
   int num_sms = 0;
   LX_CUDA(cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev));
   // bf16 weights: the residual products R X and R^T X on the tensor cores
   constexpr bool bf16_w = std::is_same<TW, __nv_bfloat16>::value;
   const bool res_tc = bf16_w && res_tc_fits(rows, cols, l);
   lx_status tc_status = LX_OK;
+  waits.err = w.err;
+  LX_CUDA(cudaMemsetAsync(w.err, 0, sizeof(int), s));
   bool have_wt = false;  // W^T of this call's weights lies in w.tc
   auto gemm = [&](int mode, const float* X, const float* B, float* C, int M, int N, int K) {
     const dim3 grid((N + CG_TILE - 1) / CG_TILE, (M + CG_TILE - 1) / CG_TILE);
@@ -1076,7 +1103,7 @@ lx_status run_compress(int rows, int cols, const TW* Wd, const TW* Wm, const flo
       if (res_tc && (mode == A_RES || mode == A_RES_T)) {
         const lx_status st = res_gemm_tc(mode == A_RES_T, reinterpret_cast<const __nv_bfloat16*>(Wm),
                                          reinterpret_cast<const __nv_bfloat16*>(Wd), rows, cols, B, N,
-                                         C, w.tc, &have_wt, num_sms, dev, s);
+                                         C, w.tc, &have_wt, waits, num_sms, dev, s);
         if (st != LX_OK) tc_status = st;
         return;
       }
@@ -1151,7 +1178,7 @@ lx_status run_compress(int rows, int cols, const TW* Wd, const TW* Wm, const flo
       attr[0].val.clusterDim.z = 1;
       cfg.attrs = attr;
       cfg.numAttrs = 1;
-      LX_CUDA(cudaLaunchKernelEx(&cfg, kern, (const float*)w.Mt, l, w.Wt));
+      LX_CUDA(cudaLaunchKernelEx(&cfg, kern, (const float*)w.Mt, l, w.Wt, (const CallWaits)waits));
       return LX_OK;
     };
     if (Lp <= 32) LX_TRY(launch(k_jacobi_cluster<2>, 0, 2 * os_part(2)));
@@ -1162,7 +1189,7 @@ lx_status run_compress(int rows, int cols, const TW* Wd, const TW* Wm, const flo
     else LX_TRY(launch(k_jacobi_cluster<16>, 5, 2 * os_part(16)));
   }
   k_ritz<<<l, 256, 0, s>>>(w.Mt, w.Wt, l, w.MWn, w.Wn, w.sig64);
-  k_finish<<<l, 256, 0, s>>>(w.sig64, w.MWn, w.Wn, l, r, w.Wu, w.Wv, sigma);
+  k_finish<<<l, 256, 0, s>>>(w.sig64, w.MWn, w.Wn, l, r, w.err, w.Wu, w.Wv, sigma);
   gemm(A_F32, yc, w.Wu, U, rows, r, l);   // U_r S^(1/2)
   gemm(A_F32, zc, w.Wv, V, cols, r, l);   // V_r S^(1/2)
   k_sign<<<r, 256, 0, s>>>(U, V, rows, cols, r);
@@ -1197,12 +1224,13 @@ extern "C" lx_status lx_compress_factor(int32_t dtype, int32_t rows, int32_t col
   if ((uintptr_t)workspace & 255u) return fail(LX_ERR_ARG, "workspace must be 256-byte aligned");
   const CompressWs w = carve((char*)workspace, rows, cols, l, r);
   if (workspace_bytes < w.bytes) return fail(LX_ERR_ARG, "workspace too small");
+  const CallWaits waits = take_call_waits();
   int dev = 0;
   LX_CUDA(cudaGetDevice(&dev));
   cudaStream_t s = (cudaStream_t)stream;
   if (dtype == LX_BF16)
     return run_compress(rows, cols, (const __nv_bfloat16*)w_dom, (const __nv_bfloat16*)w_mem,
-                        omega, l, r, power_iters, U, V, sigma, w, dev, s);
+                        omega, l, r, power_iters, U, V, sigma, w, waits, dev, s);
   return run_compress(rows, cols, (const float*)w_dom, (const float*)w_mem, omega, l, r,
-                      power_iters, U, V, sigma, w, dev, s);
+                      power_iters, U, V, sigma, w, waits, dev, s);
 }

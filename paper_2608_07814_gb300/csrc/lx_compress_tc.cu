@@ -41,7 +41,7 @@ struct ResLaunch {
   int M, Npad, kb_seg, kb_split, n_kb;  // 64-wide K blocks: per segment, per CTA, in all
   float* part;        // [gridDim.z][splits][M][Npad]: blockIdx.z takes B rows z Npad ..
   unsigned long long wait_cycles;
-  int* err;           // error word (LX_ERR_TIMEOUT on a wait that gave up), or null
+  int* err;           // error word (LX_ERR_TIMEOUT on a wait that gave up)
   int unmet;          // test hook: the MMA issuer first waits for what nothing fulfils
 };
 
@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(RM_THREADS, 1) k_res_mma(const __grid_constant
   }
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == RM_THREADS - 1 && P.err && *abort_flag) atomicExch(P.err, LX_ERR_TIMEOUT);
+  if (threadIdx.x == RM_THREADS - 1 && *abort_flag) atomicExch(P.err, LX_ERR_TIMEOUT);
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256)
@@ -270,7 +270,7 @@ bool res_tc_fits(long rows, long cols, long l) {
 
 lx_status res_gemm_tc(bool transposed, const __nv_bfloat16* Wm, const __nv_bfloat16* Wd,
                       long rows, long cols, const float* X, long N, float* C, char* ws,
-                      bool* have_wt, int num_sms, int dev, cudaStream_t s) {
+                      bool* have_wt, const CallWaits& waits, int num_sms, int dev, cudaStream_t s) {
   auto al = [](size_t v) { return (v + 255) / 256 * 256; };
   __nv_bfloat16* Wt = reinterpret_cast<__nv_bfloat16*>(ws);  // [2][cols][rows]
   __nv_bfloat16* Bc = reinterpret_cast<__nv_bfloat16*>(ws + al(2 * (size_t)rows * cols * 2));
@@ -310,7 +310,9 @@ lx_status res_gemm_tc(bool transposed, const __nv_bfloat16* Wm, const __nv_bfloa
   P.kb_split = (P.n_kb + splits - 1) / splits;
   splits = (P.n_kb + P.kb_split - 1) / P.kb_split;
   P.part = part;
-  P.wait_cycles = kDefaultWaitCycles;
+  P.wait_cycles = waits.cycles;
+  P.err = waits.err;
+  P.unmet = waits.unmet == LX_WAIT_CALL_PRODUCT;
   const int b_bytes = (int)Npad * 64 * 2;
   const int smem = RM_STAGES * (RM_A_BYTES + ((b_bytes + 1023) & ~1023)) + 8 * (2 * RM_STAGES + 3) + 1024;
   LX_CUDA(smem_cap_once((const void*)k_res_mma, 227 * 1024, dev, g_rm_cap));
@@ -361,7 +363,7 @@ lx_status tc_splitk_gemm(lx_layer* L, const CUtensorMap& a, const CUtensorMap& b
 // nz)); a plain launch (no layer), for the stateless entry points.
 lx_status tc_splitk_gemm_chunks(const CUtensorMap& a, const CUtensorMap& b, int M, int Npad,
                                 int nz, int K, float* part, int max_splits, int* splits_out,
-                                int num_sms, int dev, cudaStream_t s) {
+                                const CallWaits& waits, int num_sms, int dev, cudaStream_t s) {
   ResLaunch P;
   std::memset(&P, 0, sizeof(P));
   P.a_mem = a;
@@ -377,7 +379,9 @@ lx_status tc_splitk_gemm_chunks(const CUtensorMap& a, const CUtensorMap& b, int 
   P.kb_split = (P.n_kb + splits - 1) / splits;
   splits = (P.n_kb + P.kb_split - 1) / P.kb_split;
   P.part = part;
-  P.wait_cycles = kDefaultWaitCycles;
+  P.wait_cycles = waits.cycles;
+  P.err = waits.err;
+  P.unmet = waits.unmet == LX_WAIT_CALL_PRODUCT;
   const int b_bytes = Npad * 64 * 2;
   const int smem = RM_STAGES * (RM_A_BYTES + ((b_bytes + 1023) & ~1023)) + 8 * (2 * RM_STAGES + 3) + 1024;
   LX_CUDA(smem_cap_once((const void*)k_res_mma, 227 * 1024, dev, g_rm_cap));

@@ -549,6 +549,16 @@ bool encode_bf16_2d(CUtensorMap* m, const void* base, long inner, long outer, in
 // (bf16 weights): C [M][N] = R X (transposed = false: M = rows, K = cols) or
 // R^T X (M = cols, K = rows), R = Wm - Wd [rows][cols], X fp32 [K][N]
 constexpr int RES_TC_MAX_SPLITS = 32;
+// the bounded waits of a call without a layer: `err` (device, zeroed by the call)
+// takes LX_ERR_TIMEOUT when one gives up, and the call's last kernels then write
+// NaN results
+struct CallWaits {
+  unsigned long long cycles = kDefaultWaitCycles;
+  int unmet = 0;  // lx_wait_site made to run out (test hook), 0 = none
+  int* err = nullptr;
+};
+// the calling thread's hook of lx_inject_unmet_wait_call, for one call
+CallWaits take_call_waits();
 size_t res_tc_workspace(long rows, long cols, long l);
 // where the K ranges' partials lie in that workspace (RES_TC_MAX_SPLITS x
 // max(rows, cols) x 16-padded l floats)
@@ -556,12 +566,13 @@ size_t res_tc_part_offset(long rows, long cols, long l);
 bool res_tc_fits(long rows, long cols, long l);
 lx_status res_gemm_tc(bool transposed, const __nv_bfloat16* Wm, const __nv_bfloat16* Wd,
                       long rows, long cols, const float* X, long N, float* C, char* ws,
-                      bool* have_wt, int num_sms, int dev, cudaStream_t s);
+                      bool* have_wt, const CallWaits& waits, int num_sms, int dev, cudaStream_t s);
 // split-K tensor-core product part[s][M][Npad] = A . B^T over K range s (see
 // lx_compress_tc.cu); the number of ranges used is returned in splits_out
 lx_status tc_splitk_gemm_chunks(const CUtensorMap& a, const CUtensorMap& b, int M, int Npad,
                                 int nz, int K, float* part, int max_splits, int* splits_out,
-                                int num_sms, int dev, cudaStream_t s);
+                                const CallWaits& waits, int num_sms, int dev,
+                                cudaStream_t s);
 lx_status tc_splitk_gemm(lx_layer* L, const CUtensorMap& a, const CUtensorMap& b, int M, int Npad,
                          int K, float* part, int max_splits, int* splits_out, cudaStream_t s,
                          const char* name);

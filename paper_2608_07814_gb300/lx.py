@@ -31,9 +31,10 @@ EXPORTS = [
     "lx_read_profile", "lx_last_error", "lx_bucket_noalloc", "lx_coact_accumulate",
     "lx_coact_npmi", "lx_align_cost", "lx_lap_solve", "lx_lap_solve_batch", "lx_permute_neurons",
     "lx_compress_workspace", "lx_compress_factor", "lx_set_wait_limit", "lx_inject_unmet_wait",
-    "lx_clear_device_error",
+    "lx_clear_device_error", "lx_inject_unmet_wait_call",
 ]
-LX_WAIT_NONE, LX_WAIT_STREAM_DEP, LX_WAIT_TC_MMA, LX_WAIT_ROUTER = range(4)
+(LX_WAIT_NONE, LX_WAIT_STREAM_DEP, LX_WAIT_TC_MMA, LX_WAIT_ROUTER, LX_WAIT_CALL_PRODUCT,
+ LX_WAIT_CALL_JACOBI) = range(6)
 LX_NOALLOC_SCRATCH_BYTES = 16 << 20
 
 
@@ -90,6 +91,7 @@ def lib() -> ctypes.CDLL:
             "lx_set_profiling": [vp, i32],
             "lx_set_wait_limit": [vp, ctypes.c_uint64],
             "lx_inject_unmet_wait": [vp, i32],
+            "lx_inject_unmet_wait_call": [i32, ctypes.c_uint64],
             "lx_clear_device_error": [vp],
             "lx_read_profile": [vp, ctypes.POINTER(KernelTime), i32, ctypes.POINTER(i32)],
             "lx_bucket_noalloc": [vp, vp, i32, i32, vp, vp, vp, vp, vp, vp],
@@ -318,6 +320,12 @@ def align_cost(dom, mem, stream=None) -> torch.Tensor:
     _check(lib().lx_align_cost(_dtype_code(g), H, I, *[_ptr(t) for t in dom],
                                *[_ptr(t) for t in mem], _ptr(cost), _stream(stream)))
     return cost
+
+
+def inject_unmet_wait_call(site: int, cycles: int = 0) -> None:
+    """Test hook: in this thread's next align_cost / compress_factor the wait at
+    `site` (LX_WAIT_CALL_*) runs out after `cycles` SM clock cycles."""
+    _check(lib().lx_inject_unmet_wait_call(int(site), int(cycles)))
 
 
 def lap_solve(cost: np.ndarray):
