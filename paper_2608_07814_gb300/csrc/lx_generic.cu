@@ -36,6 +36,8 @@ namespace {
 // each, together all 24), so every product is exact, and each 64-deep chunk is
 // summed by the tensor core from zero and added to the fp32 sum with an ordinary
 // rounded addition: the tensor core's own accumulation spans 64 products only.
+// A sum that comes out a NaN is formed again by plain multiply-adds (infinite
+// weights; see the epilogue).
 // fp32 weights: fused multiply-adds in ascending K (4 x 4 outputs a thread).
 // Measured on the Qwen3-30B-A3B-shaped layer with rank 32 at 96 tokens, whole
 // forward: 1669 us with a scalar-load, single-buffered form, 195 us with this
@@ -96,9 +98,10 @@ __device__ __forceinline__ int gg_pos(int u, int m) {
   if constexpr (UNITS == 8) return u ^ (m & 7);
   else return (((u & 3) << 2) | (u >> 2)) ^ ((m & 1) << 2);
 }
-// x = hi + mid + lo exactly, each part the leading eight significant bits of
-// what is left (by truncation: no part overflows), two values packed as bf16;
-// an infinity is hi alone (inf - inf would make it a NaN)
+// x = hi + mid + lo, each part the leading eight significant bits of what is left
+// (by truncation: no part overflows), two values packed as bf16; exact for |x| >=
+// 2^-110 (below, what is under 2^-133, the least bf16, is cut); an infinity is hi
+// alone (inf - inf would make it a NaN)
 __device__ __forceinline__ float gg_rest(float x, float& head) {
   head = __uint_as_float(__float_as_uint(x) & 0xFFFF0000u);
   return fabsf(x) == INFINITY ? 0.f : x - head;
@@ -113,6 +116,13 @@ __device__ __forceinline__ void gg_split(uint32_t xb, uint32_t yb, uint32_t& hi,
   hi = gg_pack(hx, hy);
   mid = gg_pack(mx, my);
   lo = gg_pack(lx_, ly);
+}
+
+// element k of weight row c (stored in rows of K, or tiled 64 x 64)
+template <typename TW>
+__device__ __forceinline__ const TW* gg_weight(const TW* W, bool tiled, int c, int k, int K) {
+  return tiled ? W + (((size_t)(c >> 6) * (K >> 6) + (k >> 6)) * 64 + (c & 63)) * 64 + (k & 63)
+               : W + (size_t)c * K + k;
 }
 
 // One chunk of a tile's tensor-core product: NT groups of eight rows.
@@ -161,6 +171,23 @@ __device__ __forceinline__ void gg_chunk_mma(uint32_t ws, uint32_t as, float (&s
   for (int j = 0; j < NT; ++j)
 #pragma unroll
     for (int c = 0; c < 4; ++c) sum[j][c] += acc[j][c];
+}
+
+// The sums of this thread's fragments that came out NaN, term by term in ascending
+// K: a zero part of a split activation times an infinite weight is a NaN that the
+// plain product is not.  Out of line, so that the kernel's registers do not see it
+// (in line: 199 -> 210 us a forward at rank 32, 96 tokens).
+__device__ __noinline__ void gg_redo_nan(float (&sum)[G_BM / 8][4], const float* const* arow, int rows,
+                                         int cols, bool tiled, const __nv_bfloat16* W, int col0, int K) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int e = 0; e < 4 * (G_BM / 8); ++e) {
+    const int j = e >> 2, c = e & 3;
+    const int m = 8 * j + 2 * (lane & 3) + (c & 1), col = 16 * warp + (lane >> 2) + (c >= 2 ? 8 : 0);
+    if (m >= rows || col >= cols || sum[j][c] == sum[j][c]) continue;
+    float v = 0.f;
+    for (int k = 0; k < K && v == v; ++k) v = fmaf(arow[m][k], to_f32(*gg_weight(W, tiled, col0 + col, k, K)), v);
+    sum[j][c] = v;
+  }
 }
 
 // OPK only names the instantiation (one kernel symbol per product in profiles)
@@ -213,10 +240,7 @@ k_grouped_gemm(const __grid_constant__ GemmLaunch P) {
     // (a rank that is no multiple of eight, bf16, or of four, fp32) element loads
     const bool vec = K % EW == 0 && K % EA == 0 && o.lda % EA == 0;
     const int nch = (K + BK - 1) / BK;
-    auto w_at = [&](int c, int kx) {
-      return o.tiled ? W + ((((size_t)((col0 + c) >> 6) * (K >> 6) + (kx >> 6)) * 64 + ((col0 + c) & 63)) * 64 + (kx & 63))
-                     : W + (size_t)(col0 + c) * K + kx;
-    };
+    auto w_at = [&](int c, int kx) { return gg_weight(W, o.tiled, col0 + c, kx, K); };
     // what: 1 the weights, 2 the rows of A, 3 both
     auto fetch = [&](int ch, int what) {
       if (ch >= nch) return;
@@ -316,6 +340,13 @@ k_grouped_gemm(const __grid_constant__ GemmLaunch P) {
     float* out = o.out + (size_t)row0 * o.ldo + (size_t)grp * Ng + col0;
     if constexpr (C::MMA) {
       const int g = lane >> 2, q = lane & 3;
+      if constexpr (sizeof(TA) == 4) {
+        float nan = 0.f;  // a NaN among the sums of rows that count
+#pragma unroll
+        for (int j = 0; j < G_BM / 8; ++j)
+          if (8 * j < rows) nan += (sum[j][0] + sum[j][1]) + (sum[j][2] + sum[j][3]);
+        if (nan != nan) gg_redo_nan(sum, arow, rows, cols, o.tiled, W, col0, K);
+      }
 #pragma unroll
       for (int j = 0; j < G_BM / 8; ++j)
 #pragma unroll
