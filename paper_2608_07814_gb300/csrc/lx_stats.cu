@@ -3,12 +3,14 @@
 // normalised pointwise mutual information, whose 1 - NPMI is Stage 2's
 // Coact-NPMI clustering distance).
 //
-// Co-activation counts are popcounts: a CTA takes a chunk of tokens, records in
-// shared memory one bit per (expert, token) of the tokens' selected sets, and
-// counts for its slice of the expert pairs the tokens that have both
+// Co-activation counts are popcounts (k_coact_bits): a CTA takes a chunk of tokens,
+// records in shared memory one bit per (expert, token) of the tokens' selected
+// sets, and counts for its slice of the expert pairs the tokens that have both
 // (popc(bits_i & bits_j) over the chunk's words), one 64-bit atomic addition per
-// non-zero pair and chunk.  Integer addition is associative, so the counts do
-// not depend on the order.
+// non-zero pair and chunk.  Its work grows with the square of E; with many experts
+// and few ids a token, a 64-bit atomic addition per pair of the token
+// (k_coact_global) is less (coact_by_bits).  Integer addition is associative, so
+// the counts do not depend on the form or the order.
 #include <algorithm>
 
 #include "lx_internal.cuh"
@@ -17,6 +19,7 @@ namespace lx {
 namespace {
 
 constexpr int CO_THREADS = 512;
+constexpr int CO_WARPS = CO_THREADS / 32;
 constexpr int CO_BIT_BYTES = 128 * 1024;  // bitmaps of a chunk
 constexpr int CO_MAX_WORDS = 64;
 
@@ -25,7 +28,7 @@ constexpr int CO_MAX_WORDS = 64;
 __host__ __device__ inline int co_words(int E, int T) {
   int w = CO_MAX_WORDS;
   while (w > 1 && (size_t)w * E * 4 > CO_BIT_BYTES) w /= 2;
-  const int need = (T + 31) / 32;
+  const int need = T / 32 + (T % 32 != 0);
   return w < need ? w : need;
 }
 
@@ -75,6 +78,39 @@ k_coact_bits(const int* __restrict__ ids, int T, int k, int E, int words,
   }
 }
 
+// One warp per token: lane s holds slot s's id, selected when it is in [0, E) and
+// no lower lane holds the same.
+__global__ void __launch_bounds__(CO_THREADS)
+k_coact_global(const int* __restrict__ ids, int T, int k, int E, unsigned long long* __restrict__ fire,
+               unsigned long long* __restrict__ coact) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (long t = (long)blockIdx.x * CO_WARPS + warp; t < T; t += (long)gridDim.x * CO_WARPS) {
+    const int id = lane < k ? ids[(size_t)t * k + lane] : -1;
+    const bool valid = id >= 0 && id < E;
+    // (invalid lanes never match another lane)
+    const unsigned same = __match_any_sync(0xffffffffu, valid ? id : -1 - lane);
+    const bool mine = valid && lane == __ffs(same) - 1;
+    const unsigned sel = __ballot_sync(0xffffffffu, mine);
+    if (mine && fire) atomicAdd(&fire[id], 1ull);
+    if (!coact) continue;
+    for (unsigned b = sel; b; b &= b - 1) {  // warp-uniform loop over the selected lanes
+      const int other = __shfl_sync(0xffffffffu, id, __ffs(b) - 1);
+      if (mine) atomicAdd(&coact[(size_t)id * E + other], 1ull);
+    }
+  }
+}
+
+// Up to 256 experts the bits won at every size measured (the pairs kept as a
+// histogram in shared memory before: 1.5 to 10 times slower).  Above, one addition a
+// pair costs T k^2, the bits T E^2 / 64 and a flush of up to E^2 a chunk; measured,
+// atomics against bits: E = 1024, k = 8: 2048 tokens 4.6 / 41 us, 65536 50 / 479;
+// E = 512, k = 8: 65536 66 / 140, k = 32: 2048 20 / 36, 65536 466 / 188; E = 384, k =
+// 8: 8192 14 / 25, 65536 88 / 78; E = 768, k = 32: 8192 64 / 48; E = 1024, k = 32:
+// 65536 389 / 518.
+bool coact_by_bits(int T, int k, int E) {
+  return E <= 256 || (E <= 768 && E <= 48 * k && (double)T * k * k >= 4e6);
+}
+
 // p_i = C_ii / n, p_ij = C_ij / n; ln(p_ij / (p_i p_j)) / (-ln p_ij) for
 // 0 < p_ij < 1, -1 for p_ij = 0, +1 for p_ij = 1 (float64).
 __global__ void k_npmi(const unsigned long long* __restrict__ coact, int E,
@@ -116,13 +152,20 @@ extern "C" lx_status lx_coact_accumulate(const int32_t* topk_id, int32_t T, int3
   int dev = 0, sms = 0;
   LX_CUDA(cudaGetDevice(&dev));
   LX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int words = co_words(E, T), chunks = (T + 32 * words - 1) / (32 * words);
+  unsigned long long* f = reinterpret_cast<unsigned long long*>(fire);
+  unsigned long long* c = reinterpret_cast<unsigned long long*>(coact);
+  if (!coact_by_bits(T, k, E)) {
+    const long grid = std::min(((long)T + CO_WARPS - 1) / CO_WARPS, 8L * sms);
+    k_coact_global<<<(unsigned)grid, CO_THREADS, 0, s>>>(topk_id, T, k, E, f, c);
+    LX_CUDA(cudaGetLastError());
+    return LX_OK;
+  }
+  const int words = co_words(E, T), chunks = (int)(((long)T + 32 * words - 1) / (32 * words));
   // enough slices of the pairs for two CTAs an SM, at least a row for each
   const int slices = std::max(1, std::min(E, (2 * sms + chunks - 1) / chunks));
   LX_CUDA(smem_cap_once((const void*)k_coact_bits, CO_BIT_BYTES, dev, g_co_smem_cap));
   k_coact_bits<<<dim3(chunks, std::min(slices, 128)), CO_THREADS, sizeof(unsigned int) * (size_t)words * E, s>>>(
-      topk_id, T, k, E, words, reinterpret_cast<unsigned long long*>(fire),
-      reinterpret_cast<unsigned long long*>(coact));
+      topk_id, T, k, E, words, f, c);
   LX_CUDA(cudaGetLastError());
   return LX_OK;
 }
