@@ -390,15 +390,19 @@ constexpr int RS_WARPS = 8;
 // lower the threshold), and the top-k of the candidates, at most one a lane, by
 // counting for each the candidates ahead of it (independent shuffles).
 // U: 16-byte chunks of a candidate's router row that a lane has in flight (two
-// candidates at a time): 8, whole rows of up to 2048 elements at once, with three
-// CTAs an SM; 4 and four CTAs for longer rows (measured at H = 2560, E = 256, 4096
-// tokens: 41 us, 53 with 8).  Measured, Qwen3-30B-A3B-shaped router: 8192 tokens
-// 49 -> 46 us; a route call of 2048 tokens 35.0 -> 33.0, of 1031 32.6 -> 29.1 (two
-// ordered top-k a token and U = 4 before).  Tried: the candidates of 8 or 16
+// candidates at a time): 8 for rows of 1025 to 2048 elements, which are then whole
+// rows, else 4 (rows of up to 1024 have no more, and twice the predicated loads cost:
+// H = 1024, E = 256, k = 8, 4096 tokens, both launches: 43 us with 8, 36 with 4).  CTAS
+// an SM: three (four leave too few registers for the loads: H = 4096, E = 256, k = 8,
+// 8192 tokens: 105 us, 126 with four), but four where the batch is then one wave and
+// not two (H = 2560, E = 256, k = 8, 4096 tokens: 52, 56 with three).
+// Measured, Qwen3-30B-A3B-shaped router: 8192 tokens 49 -> 46 us; a route call of 2048
+// tokens 35.0 -> 33.0, of 1031 32.6 -> 29.1 (two ordered top-k a token and U = 4
+// before).  Tried: the candidates of 8 or 16
 // tokens gathered per expert, so that a router row is loaded once for all of them:
 // 50 and 67 us at 8192 tokens (the loads do not bound it).
-template <int EPL, int U>
-__global__ void __launch_bounds__(RS_WARPS * 32, U == 8 ? 3 : 4)
+template <int EPL, int U, int CTAS>
+__global__ void __launch_bounds__(RS_WARPS * 32, CTAS)
 k_router_screen(const float* part, int splits, int Epad, const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ W,
                 const float* __restrict__ bias, int T, int E, int H, float wmax, int k,
                 int* __restrict__ topk_id, float* __restrict__ topk_w) {
@@ -613,24 +617,31 @@ static size_t screen_smem(const lx_layer* L) {
   return (size_t)RS_WARPS * ((size_t)L->H * 2 + 4 * (size_t)std::max(L->E, 2 * LX_MAX_K));
 }
 
-// Whether the screened route pays when only ids and gates are asked for.  Its
-// cost hardly depends on the batch below about 1200 tokens (two launches, about
-// 16 us); the full logits' grows with T E H.  Measured route calls (bucketing
-// included), full -> screened: E = 128, H = 2048: T = 257 26.5 -> 28.8 us, 320
-// 29.9 -> 28.2, 512 37.7 -> 29.4, 1031 48.3 -> 29.1; E = 256, H = 2560: T = 200
-// 41.3 -> 41.6, 257 44.3 -> 40.1, 1031 102 -> 45.8.
-static bool screen_pays(const lx_layer* L, int T) {
+// Whether the screened route pays when only ids and gates are asked for: always
+// where the tiled router would run, else by an estimate of both in microseconds, from
+// 256 tokens on.  The full logits grow with T E H (and a little for each row); the
+// screened route's two launches with H and k, below a wave of tokens not with T.
+// Measured on GB300, router kernels alone, full / screened: E = 128, H = 2048, k = 8:
+// T = 300 24 / 29, 512 35 / 27; k = 2: 300 23 / 23; E = 256, H = 2560, k = 8: T = 256 41
+// / 40, 800 92 / 42; E = 64, H = 4096, k = 8: 512 31 / 36, 800 39 / 38; E = 64, H = 7168,
+// k = 8: 256 26 / 45; E = 16, H = 7168, k = 8: 8192 129 / 165, k = 2: 126 / 104; E = 128,
+// H = 7168, k = 8: 512 74 / 52, 8192 740 / 240.
+static bool screen_pays(const lx_layer* L, int T, int k) {
   if (!L->router_screen || screen_smem(L) > 200 * 1024) return false;
-  return router_is_tiled(L, T) || (T >= 256 && (double)T * L->E * L->H >= 80e6);
+  if (router_is_tiled(L, T)) return true;
+  if (T < 256) return false;
+  const double full = 10 + 0.125e-6 * T * L->E * (L->H + 700.0);
+  const double per_kilo = std::max(1.7 + 0.4 * k, 1.2 + 1e-3 * T * (1 + 0.16 * k));
+  return 15.5 + (L->E > 128 ? 5 : 0) + L->H / 1024.0 * per_kilo <= full;
 }
 
-template <int EPL, int U>
+template <int EPL, int U, int CTAS>
 static lx_status launch_screen(lx_layer* L, const void* x, int T, int k, int splits, int Epad, int* topk_id,
                                float* topk_w, cudaStream_t s) {
   static bool done[64] = {};
-  LX_CUDA(smem_cap_once((const void*)k_router_screen<EPL, U>, 200 * 1024, L->device, done));
+  LX_CUDA(smem_cap_once((const void*)k_router_screen<EPL, U, CTAS>, 200 * 1024, L->device, done));
   ProfScope ps(L, s, "router_select");
-  launch_k(L, k_router_screen<EPL, U>, (unsigned)((T + RS_WARPS - 1) / RS_WARPS), RS_WARPS * 32,
+  launch_k(L, k_router_screen<EPL, U, CTAS>, (unsigned)((T + RS_WARPS - 1) / RS_WARPS), RS_WARPS * 32,
            screen_smem(L), s, (const float*)L->ws.rs_part, splits, Epad, (const __nv_bfloat16*)x,
            (const __nv_bfloat16*)L->router_w, (const float*)L->router_bias, T, L->E, L->H, L->router_wmax,
            k, topk_id, topk_w);
@@ -643,7 +654,7 @@ lx_status launch_router(lx_layer* L, const void* x, int T, int k, float* logits,
   if (reinterpret_cast<uintptr_t>(x) % 16)
     return fail(LX_ERR_ARG, "x must be 16-byte aligned");
   const int tiles = (T + RT_TOK - 1) / RT_TOK;
-  if (!need_logits && screen_pays(L, T)) {
+  if (!need_logits && screen_pays(L, T, k)) {
     // screened: approximate logits on the tensor cores, then the candidates'
     // canonical logits and the top-k (the logits buffer is not written)
     CUtensorMap xm;
@@ -654,11 +665,17 @@ lx_status launch_router(lx_layer* L, const void* x, int T, int k, float* logits,
     int splits = 1;
     LX_TRY(tc_splitk_gemm(L, xm, L->router_map, T, Epad, L->H, L->ws.rs_part, RS_MAX_SPLITS,
                           &splits, s, "router_screen"));
+    // (see k_router_screen on its forms)
+    const int ctas = (T + RS_WARPS - 1) / RS_WARPS;
+    const bool four = ctas > 3 * L->num_sms && ctas <= 4 * L->num_sms && 4 * (screen_smem(L) + 1024) <= 228 * 1024;
+    const bool eight = L->H > 1024 && L->H <= 2048;
     if (L->E <= 128)
-      return L->H <= 2048 ? launch_screen<4, 8>(L, x, T, k, splits, Epad, topk_id, topk_w, s)
-                          : launch_screen<4, 4>(L, x, T, k, splits, Epad, topk_id, topk_w, s);
-    return L->H <= 2048 ? launch_screen<8, 8>(L, x, T, k, splits, Epad, topk_id, topk_w, s)
-                        : launch_screen<8, 4>(L, x, T, k, splits, Epad, topk_id, topk_w, s);
+      return eight  ? launch_screen<4, 8, 3>(L, x, T, k, splits, Epad, topk_id, topk_w, s)
+             : four ? launch_screen<4, 4, 4>(L, x, T, k, splits, Epad, topk_id, topk_w, s)
+                    : launch_screen<4, 4, 3>(L, x, T, k, splits, Epad, topk_id, topk_w, s);
+    return eight  ? launch_screen<8, 8, 3>(L, x, T, k, splits, Epad, topk_id, topk_w, s)
+           : four ? launch_screen<8, 4, 4>(L, x, T, k, splits, Epad, topk_id, topk_w, s)
+                  : launch_screen<8, 4, 3>(L, x, T, k, splits, Epad, topk_id, topk_w, s);
   }
   if (router_is_tiled(L, T)) {
     // large batch: persistent register-tiled kernel
