@@ -247,7 +247,8 @@ static_assert(GR_CH == 4, "gram_sum adds four chains");
 // panel's rank-16 update with a warp on four rows, lanes along the columns.
 // The factor goes to Lout [L][L] (zero above the diagonal) and the inverses of
 // its 16 x 16 diagonal blocks to Dinv [blocks][16][16], from which the kernel
-// below forms the rest of the inverse.  A zero Gram gives Lout = Dinv = 0.  The
+// below forms the rest of the inverse (one block is the whole of it: L <= 16 gives
+// T = L^-T here, and that launch is saved).  A zero Gram gives Lout = Dinv = 0.  The
 // roots and reciprocals are the correctly rounded ones: a Newton step on the
 // fast reciprocal root shortens the diagonal's chain by 6 us at the cost of up to
 // an ulp.  Measured at L = 136: 152 us with in-place shared-memory steps and
@@ -259,7 +260,7 @@ inline int ch_ldp(int L) { return (L + 127) / 128 * 128; }  // panel copy: whole
 
 __global__ void __launch_bounds__(CH_THREADS, 1)
 k_chol32(const float2* __restrict__ Gp, int L, int ldp, float shift_rel, float* __restrict__ Lout,
-         float* __restrict__ Dinv) {
+         float* __restrict__ Dinv, float* __restrict__ T) {
   extern __shared__ __align__(16) float Ls[];
   float* Pt = Ls + ((tri_off(L) + 3) & ~3);          // [CH_B][ldp] panel, transposed
   __shared__ __align__(16) float sD[2][CH_B][CH_B];  // by block parity: sD[c][i] = l_ic of the diagonal block
@@ -311,6 +312,7 @@ k_chol32(const float2* __restrict__ Gp, int L, int ldp, float shift_rel, float* 
   if (!(md > 0.0)) {
     for (int e = tid; e < L * L; e += CH_THREADS) Lout[e] = 0.f;
     for (int e = tid; e < nb * CH_B * CH_B; e += CH_THREADS) Dinv[e] = 0.f;
+    for (int e = tid; T && e < L * L; e += CH_THREADS) T[e] = 0.f;
     return;
   }
   const float shift = (float)(shift_rel * md);
@@ -364,6 +366,10 @@ k_chol32(const float2* __restrict__ Gp, int L, int ldp, float shift_rel, float* 
 #pragma unroll
       for (int i = 0; i < CH_B; ++i)
         Dinv[(kb * CH_B + i) * CH_B + lane] = (i < bw && lane <= i) ? x[i] : 0.f;
+    if (T && lane < L)
+#pragma unroll
+      for (int i = 0; i < CH_B; ++i)
+        if (i < L) T[lane * L + i] = lane <= i ? x[i] : 0.f;
   };
   if (warp == 0) {
     float a[CH_B];
@@ -1128,8 +1134,8 @@ lx_status run_compress(int rows, int cols, const TW* Wd, const TW* Wm, const flo
   auto cholqr = [&](const float* X, float* out, int n, float shift, float* Lf) {
     const dim3 grid((l + GR_T - 1) / GR_T, (l + GR_T - 1) / GR_T, GR_CH);
     k_gram<<<grid, GR_T * GR_T, 0, s>>>(X, n, l, G);
-    k_chol32<<<1, CH_THREADS, ch_smem, s>>>(G, l, ldp, shift, Lf, w.Dinv);
-    k_tri_inverse<<<nb, TI_THREADS, ti_smem, s>>>(Lf, w.Dinv, l, w.T);
+    k_chol32<<<1, CH_THREADS, ch_smem, s>>>(G, l, ldp, shift, Lf, w.Dinv, nb == 1 ? w.T : nullptr);
+    if (nb > 1) k_tri_inverse<<<nb, TI_THREADS, ti_smem, s>>>(Lf, w.Dinv, l, w.T);
     gemm(A_F32, X, w.T, out, n, l, l);
   };
   // CholeskyQR (the first pass shifted by 1e-6 of the largest Gram diagonal,
