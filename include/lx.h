@@ -160,10 +160,14 @@ LX_API lx_status lx_bucket(lx_layer* layer, const int32_t* topk_id, int32_t T, i
  * Kernels: bf16 layers whose H, I and ranks are multiples of 64 (with k <= 8,
  * k * max_depth <= 32) take the weight-streaming kernels for T <= 256 and the
  * tcgen05 tensor-core kernels above; every other layer, and LX_PATH_GENERIC,
- * the CUDA-core kernels.  All products accumulate in fp32; on the streaming
- * and tensor-core paths the intermediates that cross device memory (the
- * gate/up pre-activations, x V, the SwiGLU aggregate, z Vd and the down
- * partials) are stored as bf16, on the CUDA-core path as fp32.
+ * the generic kernels.  All products accumulate in fp32; on the streaming and
+ * tensor-core paths the intermediates that cross device memory (the gate/up
+ * pre-activations, x V, the SwiGLU aggregate, z Vd and the down partials) are
+ * stored as bf16, on the generic path as fp32.  There fp32 weights take fused
+ * multiply-adds in ascending K; bf16 weights take mma.sync, an fp32 activation
+ * split into three bf16 parts (exact for |x| >= 2^-110), 64 products at a time
+ * summed by the tensor core and added to an fp32 sum; infinities and NaNs come
+ * out as in plain fp32 arithmetic.
  * Errors: LX_ERR_ARG (k, T, alignment, aliasing, null pointers), LX_ERR_OOM /
  * LX_ERR_CUDA while growing the workspace; a kernel's bounded wait that gave up
  * is reported by lx_layer_info (device_error).
@@ -205,8 +209,8 @@ typedef struct {
 LX_API lx_status lx_layer_info(lx_layer* layer, lx_layer_info_t* info);
 
 /* Execution paths.  LX_PATH_AUTO picks the fastest kernels that support the
- * layer and batch; LX_PATH_GENERIC forces the plain CUDA-core kernels (every
- * dtype and shape). */
+ * layer and batch; LX_PATH_GENERIC forces the generic kernels (every dtype and
+ * shape). */
 typedef enum { LX_PATH_AUTO = 0, LX_PATH_GENERIC = 1 } lx_path;
 LX_API lx_status lx_set_path(lx_layer* layer, int32_t path);
 

@@ -409,9 +409,13 @@ constexpr int SB_THREADS = 1024;
 constexpr int SB_MAX_T = 256;
 constexpr size_t SB_SMEM_LIMIT = 160 * 1024;
 
-// The batches this form takes: those for which a byte pair per (key, token), the
-// ids and the tables fit SB_SMEM_LIMIT (more keys or tokens than that are better
-// spread over the multi-kernel path's CTAs).
+// The batches this form takes: those for which two bytes per (key, token), the ids
+// and the tables fit SB_SMEM_LIMIT, about 81000 (key, token) pairs.  The bits need a
+// fraction of that; the line is where the byte tables of an earlier form ended.
+// Bucketing calls back to back at it and above, one CTA / three launches: 512 keys,
+// 200 tokens 8.5 / 9.6 us, 256 tokens 12.5 / 10.0; 1024 keys, 128 tokens 7.7 / 11.1,
+// 256 tokens 13.4 / 11.4; 2048 keys, 64 tokens 8.7 / 15.4, 256 tokens 16.9 / 15.7: a line
+// by the tokens alone (up to about 200) would be the better one.
 __host__ __device__ inline size_t sb_fit(int T, int k, int keys, int E, int N) {
   const size_t Tp = ((size_t)T + 15) / 16 * 16;
   return (size_t)T * k * 4 + 2 * (size_t)keys * Tp + (size_t)keys * 4 + ((size_t)keys + 2) * 4 +
@@ -544,12 +548,11 @@ k_bucket_small(const float* logits, const int* ids_in, int T, int k,
 
 }  // namespace
 
-// plans 0..N_OPS-1: generic tiles; N_OPS..2*N_OPS-1: streaming tiles
-// Plans for slots [first, first + n_plans): 0 = the generic GEMMs' six ops,
-// PLAN_TC = the tensor-core GEMMs' six ops.
 int bucket_blocks(int T) { return (T + BK_TOK - 1) / BK_TOK; }
 int bucket_words() { return BK_WORDS; }
 
+// Plans for slots [first, first + n_plans): 0 = the generic GEMMs' six ops,
+// PLAN_TC = the tensor-core GEMMs' six ops.
 static PlanArgs make_plans(const lx_layer* L, int n_plans, int first = 0) {
   PlanArgs pa;
   pa.n_plans = n_plans;

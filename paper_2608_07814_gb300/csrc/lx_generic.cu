@@ -1,4 +1,5 @@
-// Generic expert path (CUDA cores, fp32 accumulation, every dtype and shape).
+// Generic expert path (fp32 intermediates and sums, every dtype and shape; bf16
+// weights on mma.sync with exact products, fp32 weights on the CUDA cores).
 //
 // For every node n and every token t in its bucket the shared product is
 // evaluated once (Sec. 5.1):
@@ -48,7 +49,6 @@ namespace {
 constexpr int GG_THREADS = 128;
 constexpr int GG_STAGES = 4;
 constexpr int GG_CTAS_PER_SM = 3;
-constexpr int GG_WBYTES = G_BN * 128;  // weight rows of a chunk, 128 bytes each
 
 struct GemmLaunch {
   GemmArgs op[2];

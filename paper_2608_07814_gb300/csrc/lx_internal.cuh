@@ -123,7 +123,7 @@ __device__ __forceinline__ void warp_topk(const float* lt, int E, int k, int& se
 }
 
 // ---------------------------------------------------------------------------
-// grouped GEMM over node buckets (the generic CUDA-core path)
+// grouped GEMM over node buckets
 // ---------------------------------------------------------------------------
 // Op kinds, indexing the per-op tile plans.
 enum OpKind {

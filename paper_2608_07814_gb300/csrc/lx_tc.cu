@@ -463,7 +463,7 @@ k_tc_gemm(const __grid_constant__ TcLaunch P) {
       // a CTA that starts beside the preceding launch takes one tile and no more
       // before that launch is done: the first CTAs would otherwise hold the tiles
       // of a short launch while the others find none
-      if (!GATHER && qi == 1 && (!P.ready || P.kc_child)) asm volatile("griddepcontrol.wait;" ::: "memory");
+      if (!GATHER && qi == 1) asm volatile("griddepcontrol.wait;" ::: "memory");
     }
     if (!ok && lane == 0) {
       atomicExch(P.err, LX_ERR_TIMEOUT);
@@ -876,7 +876,7 @@ lx_status launch_tc_experts(lx_layer* L, const void* x, int T, int k, void* y, c
     dn.kc_wmaps = L->d_tmaps + (size_t)OP_DN_U * L->N;
     dn.kc_xmap = w.pamap + 2;
     dn.kc_slot = (int)rmax;
-    dn.ready = L->n_corr > 0;  // z was complete before tc_dn_V let this launch start
+    dn.ready = 1;  // z was complete before tc_dn_V let this launch start
     dn.omap = w.omaps ? w.omaps + 1 : nullptr;  // yb
     LX_TRY(run(dn, "tc_dn_anchor_U"));
     return launch_combine_tok(L, T, k, y, s);

@@ -3,7 +3,7 @@ oracle (oracle/compress.py), through the C ABI, on the same residual and the
 same Gaussian test matrix.
 
 Bar, derived from the arithmetic (fp32 products, Cholesky factors and Jacobi
-rotations; float64 Gram sums and Rayleigh quotients; the same subspaces as the
+rotations; Gram sums and Rayleigh quotients to float64 accuracy; the same subspaces as the
 oracle's float64 algorithm, so only rounding separates the two):
   * the rank-r approximation U V^T within 1e-4 of max|U_ref V_ref^T|;
   * singular values within 1e-5 of the largest;

@@ -205,20 +205,32 @@ def factors(Wd, Wm, omega, r, iters):
         MWn[j], Wn[j] = (v / nw).astype(F32), (w / nw).astype(F32)
     top = np.lexsort((np.arange(l), -sig))[:r]
     rs = np.sqrt(sig[top]).astype(F32)
-    U, V = gemm(Q, (MWn[top] / rs[:, None]).T), gemm(Z, (Wn[top] * rs[:, None]).T)
+    keep = (sig[top] > 1e-6 * sig[top[0]])[:, None]
+    with np.errstate(all="ignore"):
+        Wu, Wv = np.where(keep, MWn[top] / rs[:, None], F32(0)), np.where(keep, Wn[top] * rs[:, None], F32(0))
+    U, V = gemm(Q, Wu.T), gemm(Z, Wv.T)
     flip = U[np.argmax(np.abs(U), axis=0), np.arange(r)] < 0
     U[:, flip], V[:, flip] = -U[:, flip], -V[:, flip]
     return U, V, sig[top].astype(F32)
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("rows,cols,l,r,iters", [
-    (24, 40, 1, 1, 1), (24, 40, 2, 2, 0), (40, 24, 9, 7, 1), (64, 56, 24, 20, 2), (88, 72, 37, 30, 1),
-    (64, 104, 50, 50, 0), (168, 152, 146, 140, 0),
+@pytest.mark.parametrize("rows,cols,l,r,iters,kind", [
+    (24, 40, 1, 1, 1, "random"), (24, 40, 2, 2, 0, "random"), (40, 24, 9, 7, 1, "random"),
+    (64, 56, 24, 20, 2, "random"), (88, 72, 37, 30, 1, "random"), (64, 104, 50, 50, 0, "random"),
+    (168, 152, 146, 140, 0, "random"),
+    # singular values in near-equal clusters, and graded over five decades
+    (64, 72, 40, 32, 1, "clusters"), (72, 64, 33, 33, 0, "clusters"), (64, 72, 40, 32, 1, "graded"),
 ])
-def test_factors_bit_for_bit(rows, cols, l, r, iters):
+def test_factors_bit_for_bit(rows, cols, l, r, iters, kind):
     rng = np.random.default_rng(rows + l)
     Wd, Wm, om = (rng.standard_normal(s).astype(F32) for s in ((rows, cols), (rows, cols), (cols, l)))
+    if kind != "random":
+        n = min(rows, cols)
+        sv = 10.0 ** (-5 * np.arange(n) / n) if kind == "graded" else \
+            0.5 ** (np.arange(n) // 8) * (1 + 1e-5 * rng.random(n))
+        Uq, Vq = (np.linalg.qr(rng.standard_normal((m, n)))[0] for m in (rows, cols))
+        Wm = Wd + ((Uq * sv) @ Vq.T).astype(F32)
     ref = factors(Wd, Wm, om, r, iters)
     got = lx.compress_factor(*(torch.from_numpy(a).cuda() for a in (Wd, Wm, om)), r, iters)
     for name, a, b in zip("UVs", ref, got):

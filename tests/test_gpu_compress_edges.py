@@ -1,7 +1,8 @@
 """The compression kernels at the edges of their tilings: sketch widths l around
-the 16-column Cholesky blocks, the Jacobi's values per lane (64, 96, 128, 160,
-192 columns) and its change from four to eight CTAs (160 / 161), and bases
-short enough that the Gram takes one row range.  Same bars as the parity tests.
+the 16-column Cholesky blocks, the Jacobi's values per lane (32, 48, 80, 144 and
+192 columns) and the dealing of a column's entries to its lanes (up to 144 columns
+and above), fewer pairs than CTAs, and runs of pairs of unequal length.  Same bars
+as the parity tests.
 """
 import numpy as np
 import pytest

@@ -5,8 +5,8 @@ Bar: firing and co-activation counts bit-exact (integers); NPMI within 1e-12
 absolute (both sides evaluate the same float64 expression; only the last bits
 of the natural logarithm may differ).  Ids are drawn by a seeded generator with
 the method's structure (Zipf-skewed, cluster-correlated top-k sets) plus
-invalid and repeated ids; both the shared-memory (E <= 256) and the
-global-atomic (E > 256) kernels are covered.
+invalid and repeated ids; both the popcount form (E <= 256) and the additions a
+pair (E > 256, few ids a token) are covered.
 """
 import numpy as np
 import pytest
