@@ -173,20 +173,22 @@ __device__ __forceinline__ void gg_chunk_mma(uint32_t ws, uint32_t as, float (&s
     for (int c = 0; c < 4; ++c) sum[j][c] += acc[j][c];
 }
 
-// The sums of this thread's fragments that came out NaN, term by term in ascending
-// K: a zero part of a split activation times an infinite weight is a NaN that the
-// plain product is not.  Out of line, so that the kernel's registers do not see it
-// (in line: 199 -> 210 us a forward at rank 32, 96 tokens).
-__device__ __noinline__ void gg_redo_nan(float (&sum)[G_BM / 8][4], const float* const* arow, int rows,
-                                         int cols, bool tiled, const __nv_bfloat16* W, int col0, int K) {
+// The sums of this thread's fragments that came out NaN (bit 4 j + c of `nan`), term
+// by term in ascending K: a zero part of a split activation times an infinite weight
+// is a NaN that the plain product is not.  Out of line and by value, so that the
+// kernel's registers do not see it (rank 32, 96 tokens: 198 us a forward with it and
+// without; 202 with the sums passed by reference, 210 in line).
+__device__ __noinline__ void gg_redo_nan(unsigned nan, const float* const* arow, int rows, int cols,
+                                         bool tiled, const __nv_bfloat16* W, int col0, int K, float* out,
+                                         long ldo) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int e = 0; e < 4 * (G_BM / 8); ++e) {
-    const int j = e >> 2, c = e & 3;
+  for (; nan; nan &= nan - 1) {
+    const int e = __ffs(nan) - 1, j = e >> 2, c = e & 3;
     const int m = 8 * j + 2 * (lane & 3) + (c & 1), col = 16 * warp + (lane >> 2) + (c >= 2 ? 8 : 0);
-    if (m >= rows || col >= cols || sum[j][c] == sum[j][c]) continue;
+    if (m >= rows || col >= cols) continue;
     float v = 0.f;
     for (int k = 0; k < K && v == v; ++k) v = fmaf(arow[m][k], to_f32(*gg_weight(W, tiled, col0 + col, k, K)), v);
-    sum[j][c] = v;
+    out[(size_t)m * ldo + col] = v;
   }
 }
 
@@ -340,13 +342,6 @@ k_grouped_gemm(const __grid_constant__ GemmLaunch P) {
     float* out = o.out + (size_t)row0 * o.ldo + (size_t)grp * Ng + col0;
     if constexpr (C::MMA) {
       const int g = lane >> 2, q = lane & 3;
-      if constexpr (sizeof(TA) == 4) {
-        float nan = 0.f;  // a NaN among the sums of rows that count
-#pragma unroll
-        for (int j = 0; j < G_BM / 8; ++j)
-          if (8 * j < rows) nan += (sum[j][0] + sum[j][1]) + (sum[j][2] + sum[j][3]);
-        if (nan != nan) gg_redo_nan(sum, arow, rows, cols, o.tiled, W, col0, K);
-      }
 #pragma unroll
       for (int j = 0; j < G_BM / 8; ++j)
 #pragma unroll
@@ -354,6 +349,14 @@ k_grouped_gemm(const __grid_constant__ GemmLaunch P) {
           const int m = 8 * j + 2 * q + (c & 1), col = 16 * warp + g + (c >= 2 ? 8 : 0);
           if (m < rows && col < cols) out[(size_t)m * o.ldo + col] = sum[j][c];
         }
+      if constexpr (sizeof(TA) == 4) {
+        unsigned nan = 0;
+#pragma unroll
+        for (int j = 0; j < G_BM / 8; ++j)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) nan |= (sum[j][c] != sum[j][c] ? 1u : 0u) << (4 * j + c);
+        if (nan) gg_redo_nan(nan, arow, rows, cols, o.tiled, W, col0, K, out, o.ldo);
+      }
     } else {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
