@@ -733,11 +733,11 @@ def run_offline(args, rank, world, local_rank):
                 e.record(st)
                 main.wait_event(e)
         ms = _event_ms(step_conc, args.steps, args.warmup, world) / n_conc
-        # launches of one projection: the R products (split, transposes, MMA,
-        # ordered sum), 2q single and 2 double CholeskyQR passes (Gram, Cholesky,
-        # basis product each), then trmm, Jacobi, Ritz, finish, two factor
-        # products and the sign rule
-        launches_per_projection = ((1 + q) * 3 + (1 + q) * 5 + 3 * (2 * q + 4) + 7)
+        # launches of one projection: the R products (split, MMA, ordered sum; the
+        # two transposes once), 2q single and 2 double CholeskyQR passes (Gram,
+        # Cholesky, inverse, basis product each), then trmm, Jacobi, Ritz, finish,
+        # two factor products and the sign rule
+        launches_per_projection = ((2 + 2 * q) * 3 + 2 + 4 * (2 * q + 4) + 7)
         big = sum((2 + 2 * q) * 2.0 * a * b * l for a, b in shapes)        # the R-sized products
         # CholeskyQR passes: q + 2 on each side (rows and cols), each a lower
         # Gram (n l^2) and a basis product (2 n l^2); then the two factor products
